@@ -146,7 +146,7 @@ def run_case(lbm, torch, name, nx, ny, nz, tau, force, storage, rates, bc, steps
     ok = bool(np.isfinite(st["kinetic_energy"]))
     # algorithmic bytes of one sweep launch: every visited cell reads and
     # writes 19 populations; the flag byte is read where the sweep needs it
-    # (the pipe's IBB sweep walks fluid-run segments and reads no flags)
+    # (the pipe's IBB sweep walks fluid columns and reads no flags)
     sb = {lbm.F64: 8, lbm.F32: 4}.get(storage, 2)
     N = nx * ny * nz
     if bc == lbm.BC_IBB:
@@ -444,7 +444,7 @@ def cpu_baseline(target_seconds=12.0):
             "sample": f"FP64 oracle, IBB pipe slab 148x148x16 ({fluid} fluid cells), {steps} steps, {sec:.1f} s"}
 
 
-SWEEP_SOURCES = {"stream_collide_pipe_pipe148_f32": ("sweep_pipe.cu", "lbm_device.cuh", "segments.h"),
+SWEEP_SOURCES = {"sweep_columns_pipe148_f32": ("sweep_columns.cu", "lbm_device.cuh", "columns.cuh"),
                  "stream_collide_bulk_pipe148_ibm_f32": ("sweep.cu", "lbm_device.cuh")}
 
 
@@ -670,11 +670,11 @@ def main():
                        "fluid_cells": main_res["fluid_cells"], "parallelism": f"replicas x{world}",
                        "l2": "no flush: populations 2x1.46 GB >> 129 MB L2"},
             "roofline": {"bound": "hbm",
-                         "kernel": ("stream_collide_pipe<" if args.wall == "ibb" else "stream_collide_bulk<") +
+                         "kernel": ("sweep_columns<" if args.wall == "ibb" else "stream_collide_bulk<") +
                                    args.storage + ",srt," + args.wall[:3] + ">",
                          "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                          "frac": round(achieved / hbm_peak, 4), "peak_source": peak_kind,
-                         "traffic": traffic_for("stream_collide_pipe_pipe148_f32")
+                         "traffic": traffic_for("sweep_columns_pipe148_f32")
                          if (args.wall == "ibb" and args.storage == "f32" and NZ == PIPE["nz"]) else None,
                          "algorithmic_bytes_per_launch": bulk_bytes,
                          "avg_launch_ms": round(bulk_ms, 5),

@@ -1,0 +1,50 @@
+// The column layout of the pipe: populations with z fastest.
+//
+// The pipe of Sec. 2.1 is the same in every z plane, so a whole column
+// (x, y) is either fluid or solid and all cells of a fluid column have the
+// same wall links with the same wall fractions. A context with a pipe keeps
+// its populations, from its first step with a wall on, as
+//   g[i * Np + z + zp * (x + nx * y)],   zp >= nz the column pitch, Np = nx ny zp,
+// so that a warp sweeps 32 consecutive z of one column: full, aligned
+// sectors on every access, no solid cell touched, and the wall a
+// warp-uniform branch with uniform weights. Everything outside the sweeps
+// (fields, flags, link and site lists, checkpoint files) keeps x fastest;
+// the kernels here convert.
+#pragma once
+
+#include "lbm_internal.cuh"
+
+namespace lbmgb {
+
+constexpr int COL_TILE = 32;  // x by z tile of the conversions, at one y
+
+// blocks per (z tile, x tile, y; y strided beyond the grid limit)
+inline dim3 column_tiles(const Ctx &c) {
+    return dim3((unsigned)((c.nz + COL_TILE - 1) / COL_TILE), (unsigned)((c.nx + COL_TILE - 1) / COL_TILE),
+                (unsigned)(c.ny < 65535 ? c.ny : 65535));
+}
+
+// body(x, z, value) for the cells of a block's tile in z-fast order, then in
+// x-fast order: PUT(x, z) -> V runs with lanes along z, GET(x, z, V) with
+// lanes along x (TOX), or the other way round; the values cross through
+// shared memory (one pad word per row: no bank conflicts for 4-byte V)
+template <typename V, bool TOX, typename Put, typename Get>
+__device__ __forceinline__ void column_exchange(V (*sh)[COL_TILE + 1], int nx, int nz, Put put, Get get) {
+    const int z0 = blockIdx.x * COL_TILE, x0 = blockIdx.y * COL_TILE;
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5, rows = blockDim.x >> 5;
+    for (int r = row; r < COL_TILE; r += rows) {
+        const int x = x0 + (TOX ? r : lane), z = z0 + (TOX ? lane : r);
+        if (x < nx && z < nz) {
+            if (TOX) sh[lane][r] = put(x, z);  // sh[z][x]
+            else sh[r][lane] = put(x, z);
+        }
+    }
+    __syncthreads();
+    for (int r = row; r < COL_TILE; r += rows) {
+        const int x = x0 + (TOX ? lane : r), z = z0 + (TOX ? r : lane);
+        if (x < nx && z < nz) get(x, z, TOX ? sh[r][lane] : sh[lane][r]);
+    }
+    __syncthreads();  // the tile is free for the next exchange
+}
+
+}  // namespace lbmgb

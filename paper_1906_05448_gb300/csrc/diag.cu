@@ -73,6 +73,7 @@ __global__ void macro_kernel(const void *A, const uint8_t *flags, const int *aux
 
 cudaError_t launch_macro(Ctx &c, int /*mask_mode*/, float *u32) {
     if (c.q == 27) return launch_q27_macro(c);
+    if (c.zlay) return launch_column_macro(c);
     count_launch(c, G_STATS);
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     const int ibb = c.armed_bc == LBM_BC_IBB;

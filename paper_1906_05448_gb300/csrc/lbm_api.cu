@@ -1,7 +1,6 @@
 // C ABI of the library (declared in include/lbm.h): workspace layout, set-up
 // of the geometry, the per-step kernel sequence and host-side checks.
 #include "lbm_internal.cuh"
-#include "segments.h"
 
 #include <cmath>
 #include <ctime>
@@ -11,16 +10,6 @@
 #include <algorithm>
 #include <utility>
 #include <vector>
-
-#ifndef LBM_WALL_VALUES
-#define LBM_WALL_VALUES 1  // the sweep keeps the wall cells' values for the next ghost pass
-#endif
-#ifndef LBM_STATIC_LINKS
-#define LBM_STATIC_LINKS 1  // 1: static-wall links regrouped by direction for the ghost pass
-#endif
-#ifndef LBM_SEG_SECTOR
-#define LBM_SEG_SECTOR 1  // 1: sweep segments complete the 32-byte sectors at the ends of fluid runs
-#endif
 
 namespace lbmgb {
 size_t stats_partials_doubles();
@@ -44,9 +33,10 @@ struct Plan {
     size_t fA, fB, flags, owner, aux;
     size_t site_cell, site_first, site_mask, sup_ru, sup_F, sup_Fp;
     size_t link_cell, link_pid, link_dir, link_scheme, link_q, link_dP, link_dT;
-    size_t blk_sites, blk_links, counts, status, seg, slink, slink_rank, slink4, seg_bnd, bvals, wrec, gidx, gvals, wcoef, wlane, pair_items, pair_wall, wslot, refill;
+    size_t blk_sites, blk_links, counts, status, col_list, col_wall, col_coef, refill;
     long long max_refill;
-    long long max_seg;
+    int zp;
+    long long Np;
     size_t xy_start, xy_j, xy_w, it_k, it_w;
     int max_ring;
     long long max_xy;
@@ -83,8 +73,18 @@ bool make_plan(const lbm_grid *g, Plan &P) {
     const size_t np = (size_t)(P.max_np > 0 ? P.max_np : 1);
     Layout L;
     const size_t nq = g->lattice == 27 ? 27 : 19;
-    P.fA = L.take(nq * n * sb);
-    P.fB = L.take(nq * n * sb);
+    // the populations, and beside them room for the padding of the pipe's
+    // columns (columns.cuh): a pitch of whole 16-cell groups where it fits,
+    // so that every column starts on a sector in every storage type
+    const size_t slack = 10 * ms;
+    P.fA = L.take((nq * n + slack) * sb);
+    P.fB = L.take((nq * n + slack) * sb);
+    P.zp = (g->nz + 15) / 16 * 16;
+    P.Np = (long long)g->nx * g->ny * P.zp;
+    if (nq * (size_t)P.Np > nq * n + slack || P.Np >= (1LL << 31) - 4096) {
+        P.zp = g->nz;
+        P.Np = N;
+    }
     P.flags = L.take(n + 8);
     P.owner = L.take(4 * n);
     P.aux = L.take(4 * n);
@@ -108,21 +108,10 @@ bool make_plan(const lbm_grid *g, Plan &P) {
     P.max_ring = 4 * (g->nx + g->ny);
     P.it_k = L.take(4 * 16 * (size_t)P.max_ring);
     P.it_w = L.take(8 * 16 * (size_t)P.max_ring);
-    P.max_seg = (long long)g->ny * g->nz * ((g->nx + 31) / 32 + 1);
-    P.seg = L.take(16 * (size_t)P.max_seg);
-    P.slink = L.take(8 * ml);
-    P.slink_rank = L.take(4 * ml);
-    P.slink4 = L.take(16 * ml);
-    P.seg_bnd = L.take(8 * (size_t)P.max_seg);
-    P.bvals = L.take(19 * sb * ms);
-    P.wrec = L.take(8 * ms);
-    P.gidx = L.take(4 * ml);
-    P.gvals = L.take(sb * ml);
-    P.wcoef = L.take(8 * ml);
-    P.wlane = L.take(2 * ml);
-    P.pair_items = L.take(16 * (size_t)P.max_seg);
-    P.pair_wall = L.take(16 * (size_t)P.max_seg);
-    P.wslot = L.take(2 * ml);
+    const size_t nxy = (size_t)g->nx * g->ny;
+    P.col_list = L.take(8 * nxy);
+    P.col_wall = L.take(16 * nxy);
+    P.col_coef = L.take(16 * 19 * nxy);
     P.blk_sites = L.take(8 * (size_t)P.nblk);
     P.blk_links = L.take(8 * (size_t)P.nblk);
     P.counts = L.take(64);
@@ -233,6 +222,7 @@ __global__ void f64_to_plane(void *dst, const double *src, long long N, int i) {
 }
 
 cudaError_t plane_copy(Ctx &c, int i, bool to_f64) {
+    if (c.zlay) return column_plane_copy(c, i, wgt(i), to_f64);
     const unsigned nb = (unsigned)((c.N + 255) / 256);
 #define PC(S)                                                                                 \
     if (to_f64) plane_to_f64<S><<<nb, 256, 0, c.stream>>>(c.fA, c.rho_f, c.N, i);            \
@@ -505,8 +495,87 @@ lbm_status build_pipe_interp(Ctx &c) {
     return LBM_OK;
 }
 
+// Fluid columns of the pipe and the wall links of each (the same in every z
+// plane: those of plane 0 of the link list), with the weights of the
+// populations that come back along them: (2q, 1 - 2q) with f*_l(x_f - c_l)
+// for q < 1/2, (1/(2q), (2q - 1)/(2q)) with f*_ibar(x_f) for q >= 1/2, and
+// for the single-node scheme its factor (1 - 2q)/2.
+lbm_status build_columns(Ctx &c) {
+    const size_t nxy = (size_t)c.nx * c.ny, nl = (size_t)(c.nlinks / c.nz);
+    std::vector<uint8_t> fl(nxy);
+    CK(cudaMemcpy(fl.data(), c.flags, nxy, cudaMemcpyDeviceToHost));
+    std::vector<int> lcell(nl);
+    std::vector<int8_t> ldir(nl), lsch(nl);
+    std::vector<double> lq(nl);
+    if (nl > 0) {
+        CK(cudaMemcpy(lcell.data(), c.link_cell, 4 * nl, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(ldir.data(), c.link_dir, nl, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(lsch.data(), c.link_scheme, nl, cudaMemcpyDeviceToHost));
+        CK(cudaMemcpy(lq.data(), c.link_q, 8 * nl, cudaMemcpyDeviceToHost));
+    }
+    std::vector<int2> cols;
+    std::vector<uint4> wall;
+    std::vector<double> coef;
+    c.static_single = 0;
+    c.pipe_nowrap = 1;
+    size_t k = 0;
+    for (size_t cell = 0; cell < nxy; cell++) {
+        if (fl[cell] & FL_SOLID) continue;
+        const int x = (int)(cell % c.nx), y = (int)(cell / c.nx);
+        if (x == 0 || x == c.nx - 1 || y == 0 || y == c.ny - 1) c.pipe_nowrap = 0;
+        int slot = -1;
+        for (; k < nl && lcell[k] == (int)cell; k++) {
+            if (slot < 0) {
+                slot = (int)wall.size();
+                wall.push_back(make_uint4(0u, 0u, 0u, 0u));
+                coef.resize(coef.size() + 2 * 19, 0.0);
+            }
+            const int l = ldir[k];
+            // 32- and 16-bit storage: weights of the FP32 value of q
+            const double q = c.storage == LBM_F64 ? lq[k] : (double)(float)lq[k];
+            double *w = &coef[2 * (19 * (size_t)slot + l)];
+            wall[slot].x |= 1u << l;
+            if (lsch[k] == 2) {
+                wall[slot].z |= 1u << l;
+                c.static_single++;
+                w[1] = 0.5 * (1.0 - 2.0 * q);
+            } else if (q < 0.5) {
+                w[0] = 2.0 * q;
+                w[1] = 1.0 - 2.0 * q;
+            } else {
+                wall[slot].y |= 1u << l;
+                w[0] = 1.0 / (2.0 * q);
+                w[1] = (2.0 * q - 1.0) / (2.0 * q);
+            }
+        }
+        cols.push_back(make_int2((int)cell, slot));
+    }
+    if (k != nl) return fail(c, LBM_EINVAL, "link list is not in cell order");
+    c.ncols = (long long)cols.size();
+    if (!cols.empty()) CK(cudaMemcpy(c.col_list, cols.data(), sizeof(int2) * cols.size(), cudaMemcpyHostToDevice));
+    if (!wall.empty()) CK(cudaMemcpy(c.col_wall, wall.data(), sizeof(uint4) * wall.size(), cudaMemcpyHostToDevice));
+    CK(upload_weights(c, c.col_coef, coef));
+    return LBM_OK;
+}
+
+// put the state into the column layout (first step with a wall on a pipe)
+lbm_status enter_columns(Ctx &c) {
+    const size_t bytes = (size_t)c.q * (size_t)c.Np * storage_bytes(c.storage);
+    count_launch(c, G_BND);
+    CK(cudaMemsetAsync(c.fB, 0, bytes, c.stream));
+    CK(convert_columns(c, c.fA, c.fB, false, c.q == 19));
+    CK(cudaMemsetAsync(c.fA, 0, bytes, c.stream));
+    std::swap(c.fA, c.fB);
+    c.zlay = 1;
+    return LBM_OK;
+}
+
 lbm_status arm(Ctx &c, int bc) {
     c.armed_bc = bc;
+    if (bc == LBM_BC_IBB && c.has_pipe && c.q == 19) {
+        lbm_status s = enter_columns(c);
+        if (s != LBM_OK) return s;
+    }
     if (bc == LBM_BC_IBM_U || bc == LBM_BC_IBM_B) {
         c.rd = bc == LBM_BC_IBM_B ? 0.4 : 0.0;
         if (c.has_pipe || c.np > 0) {
@@ -604,28 +673,11 @@ lbm_status lbm_create(const lbm_grid *grid, double tau, const double force[3], v
     c.pipe_max_ring = P.max_ring;
     c.pipe_sp = 0;
     c.pipe_max_xy = P.max_xy;
-    c.seg = (uint4 *)(b + P.seg);
-    c.slink = (uint2 *)(b + P.slink);
-    c.static_links = 0;
-    c.slink_rank = (int *)(b + P.slink_rank);
-    c.slink4 = (uint4 *)(b + P.slink4);
-    c.seg_bnd = (uint2 *)(b + P.seg_bnd);
-    c.bvals = b + P.bvals;
-    c.wrec = (uint2 *)(b + P.wrec);
-    c.gidx = (int *)(b + P.gidx);
-    c.gvals = b + P.gvals;
-    c.wcoef = (uint2 *)(b + P.wcoef);
-    c.wlane = (unsigned short *)(b + P.wlane);
-    c.pair_items = (uint4 *)(b + P.pair_items);
-    c.pair_wall = (uint4 *)(b + P.pair_wall);
-    c.wslot = (unsigned short *)(b + P.wslot);
-    c.pair_ready = 0;
-    c.wcoef_ready = 0;
-    c.max_bvals = P.max_sites;
-    c.bvals_ready = 0;
-    c.bvals_valid = 0;
-    c.max_seg = P.max_seg;
-    c.nseg = 0;
+    c.zp = P.zp;
+    c.Np = P.Np;
+    c.col_list = (int2 *)(b + P.col_list);
+    c.col_wall = (uint4 *)(b + P.col_wall);
+    c.col_coef = b + P.col_coef;
     c.nblk = P.nblk;
     c.blk_sites = (long long *)(b + P.blk_sites);
     c.blk_links = (long long *)(b + P.blk_links);
@@ -718,7 +770,6 @@ lbm_status lbm_init_velocity(lbm_ctx *h, const double *u_host, double rho0) {
     CTX_CHECK(h);
     if (!u_host || !(rho0 > 0)) return fail(c, LBM_EINVAL, "bad velocity field or rho0");
     if (c.broken || c.armed_bc >= 0) return fail(c, LBM_ESTATE, "init_velocity only before the first step");
-    c.bvals_valid = 0;
     CK(cudaMemcpyAsync(c.u_f, u_host, sizeof(double) * 3 * c.N, cudaMemcpyHostToDevice, c.stream));
     if (c.q == 27) CK(launch_q27_init(c, c.u_f, rho0));
     else CK(launch_init_equilibrium(c, c.u_f, rho0));
@@ -730,7 +781,6 @@ lbm_status lbm_set_populations(lbm_ctx *h, const double *f_host) {
     CTX_CHECK(h);
     if (!f_host) return fail(c, LBM_EINVAL, "null populations");
     if (c.broken) return fail(c, LBM_ESTATE, "context unusable after an error");
-    c.bvals_valid = 0;
     for (int i = 0; i < c.q; i++) {
         CK(cudaMemcpyAsync(c.rho_f, f_host + (size_t)i * c.N, sizeof(double) * c.N, cudaMemcpyHostToDevice, c.stream));
         if (c.q == 27) CK(q27_plane_copy(c, i, false));
@@ -769,202 +819,7 @@ lbm_status lbm_set_pipe(lbm_ctx *h, double radius) {
     if (s != LBM_OK) return s;
     c.nsites_hint = c.nsites;
     c.nlinks_hint = c.nlinks;
-    // IBB sweep work list (segments of fluid runs, see segments.h)
-    std::vector<uint8_t> fl((size_t)c.N);
-    CK(cudaMemcpy(fl.data(), c.flags, (size_t)c.N, cudaMemcpyDeviceToHost));
-    // cells per 32-byte sector; 16-bit storage is not widened (its 16-cell
-    // sectors add more zero lanes than the full-sector stores save)
-    const long long sec = (LBM_SEG_SECTOR && storage_bytes(c.storage) >= 4) ? 32 / (long long)storage_bytes(c.storage) : 1;
-    std::vector<unsigned long long> segs;
-    const bool seg_ok = build_sweep_segments(fl.data(), c.nx, c.ny, c.nz, FL_SOLID, sec, segs);
-    std::vector<SweepItem> items;
-    if (seg_ok) pack_sweep_items(segs, items);
-    if (seg_ok && (long long)items.size() <= c.max_seg) {
-        static_assert(sizeof(SweepItem) == sizeof(uint4), "warp item layout");
-        CK(cudaMemcpy(c.seg, items.data(), sizeof(SweepItem) * items.size(), cudaMemcpyHostToDevice));
-        c.nseg = (long long)items.size();
-    }
-    // single-node links of the wall (their correction runs as its own pass)
-    c.static_single = 0;
-    if (c.nlinks > 0 && c.nlinks <= c.max_links) {
-        std::vector<int8_t> sch((size_t)c.nlinks);
-        CK(cudaMemcpy(sch.data(), c.link_scheme, (size_t)c.nlinks, cudaMemcpyDeviceToHost));
-        for (int8_t v : sch) c.static_single += v == 2;
-    }
-    // the lean sweep needs every fluid cell off the x and y faces (no x/y wrap of a pull)
-    c.pipe_nowrap = 1;
-    for (long long cell = 0; cell < c.N && c.pipe_nowrap; cell++) {
-        if (fl[(size_t)cell] & FL_SOLID) continue;
-        const long long x = cell % c.nx, y = (cell / c.nx) % c.ny;
-        if (x == 0 || x == c.nx - 1 || y == 0 || y == c.ny - 1) c.pipe_nowrap = 0;
-    }
-    // the wall is static: regroup its links by direction (cell order kept
-    // inside a group) so that neighbouring threads of the ghost pass touch
-    // neighbouring cells of one population plane
-    if (LBM_STATIC_LINKS && c.storage != LBM_F64 && c.nlinks > 0 && c.nlinks <= c.max_links && c.N < (1LL << 30)) {
-        const size_t nl = (size_t)c.nlinks;
-        std::vector<int> lcell(nl);
-        std::vector<int8_t> ldir(nl), lsch(nl);
-        std::vector<double> lq(nl);
-        CK(cudaMemcpy(lcell.data(), c.link_cell, 4 * nl, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(ldir.data(), c.link_dir, nl, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(lsch.data(), c.link_scheme, nl, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(lq.data(), c.link_q, 8 * nl, cudaMemcpyDeviceToHost));
-        int cnt[19] = {0};
-        bool ok = true;
-        for (size_t k = 0; k < nl; k++) {
-            if (ldir[k] < 0 || ldir[k] > 18 || lsch[k] < 0 || lsch[k] > 3) ok = false;
-            else cnt[ldir[k]]++;
-        }
-        if (ok) {
-            c.slink_off[0] = 0;
-            for (int l = 0; l < 19; l++) c.slink_off[l + 1] = c.slink_off[l] + cnt[l];
-            int pos[19];
-            for (int l = 0; l < 19; l++) pos[l] = c.slink_off[l];
-            // wall cells (cells with links; the list is in cell order) and their ranks
-            std::vector<int> bcells;
-            bool sorted = true;
-            for (size_t k = 0; k < nl; k++) {
-                if (k > 0 && lcell[k] < lcell[k - 1]) sorted = false;
-                if (k == 0 || lcell[k] != lcell[k - 1]) bcells.push_back(lcell[k]);
-            }
-            auto rank_of = [&](long long cell) -> long long {
-                auto it = std::lower_bound(bcells.begin(), bcells.end(), (int)cell);
-                return (it != bcells.end() && *it == (int)cell) ? (long long)(it - bcells.begin()) : -1;
-            };
-            std::vector<uint2> pk(nl);
-            std::vector<int> rk(nl);
-            for (size_t k = 0; k < nl; k++) {
-                const float qf = (float)lq[k];
-                unsigned qb;
-                std::memcpy(&qb, &qf, 4);
-                const int at = pos[ldir[k]]++;
-                pk[at] = make_uint2((unsigned)lcell[k] | ((unsigned)lsch[k] << 30), qb);
-                rk[at] = (int)rank_of(lcell[k]);
-            }
-            CK(cudaMemcpy(c.slink, pk.data(), 8 * nl, cudaMemcpyHostToDevice));
-            c.static_links = 1;
-            // per sweep item: rank of its first wall cell and the lanes that hold wall cells
-            bool bok = LBM_WALL_VALUES && sorted && c.nseg > 0 && (long long)bcells.size() <= c.max_bvals;
-            std::vector<uint2> sb(bok ? items.size() : 0);
-            std::vector<int> lane_of(bok ? bcells.size() : 0, -1);  // sweep lane of each wall cell
-            for (size_t it = 0; bok && it < items.size(); it++) {
-                const SweepItem &w = items[it];
-                const unsigned la = (w.word_a >> 16) & 0xff;
-                long long base = -1;
-                unsigned mask = 0;
-                for (unsigned lane = 0; lane < 32 && bok; lane++) {
-                    const bool pa = lane < la;
-                    const unsigned wd = pa ? w.word_a : w.word_b, row = pa ? w.row_a : w.row_b;
-                    const int lp = pa ? (int)lane : (int)(lane - la);
-                    const int len = (int)((wd >> 16) & 0xff), lead = (int)((wd >> 24) & 15), trail = (int)(wd >> 28);
-                    if (lp >= len || lp < lead || lp >= len - trail) continue;  // idle or zero lane
-                    const long long cell = (long long)row * c.nx + (long long)(wd & 0xffff) - lead + lp;
-                    const long long r = rank_of(cell);
-                    if (r < 0) continue;
-                    if (base < 0) base = r;
-                    if (r != base + __builtin_popcount(mask)) bok = false;  // ranks must follow the lanes
-                    mask |= 1u << lane;
-                    lane_of[(size_t)r] = (int)lane;
-                }
-                sb[it] = make_uint2((unsigned)(base < 0 ? 0 : base), mask);
-            }
-            // compact ghosts: per wall cell the directions ibar = opp(l) of its
-            // links and the first of its values; per link the index of its value
-            std::vector<uint2> wr(bok ? bcells.size() : 0);
-            std::vector<int> gx(bok ? nl : 0);
-            if (bok) {
-                std::vector<unsigned> dm(bcells.size(), 0u);
-                for (size_t k = 0; k < nl; k++) dm[(size_t)rank_of(lcell[k])] |= 1u << (ldir[k] == 0 ? 0 : ((ldir[k] & 1) ? ldir[k] + 1 : ldir[k] - 1));
-                unsigned acc = 0;
-                for (size_t r = 0; r < bcells.size(); r++) {
-                    wr[r] = make_uint2(acc, dm[r]);
-                    acc += (unsigned)__builtin_popcount(dm[r]);
-                }
-                int pos2[19];
-                for (int l = 0; l < 19; l++) pos2[l] = c.slink_off[l];
-                for (size_t k = 0; k < nl; k++) {
-                    const int l = ldir[k], i = l == 0 ? 0 : ((l & 1) ? l + 1 : l - 1);
-                    const size_t r = (size_t)rank_of(lcell[k]);
-                    gx[pos2[l]++] = (int)(wr[r].x + (unsigned)__builtin_popcount(dm[r] & ((1u << i) - 1u)));
-                }
-                if (acc != (unsigned)nl) bok = false;  // one value per link
-            }
-            if (bok) {
-                CK(cudaMemcpy(c.wrec, wr.data(), 8 * wr.size(), cudaMemcpyHostToDevice));
-                CK(cudaMemcpy(c.gidx, gx.data(), 4 * nl, cudaMemcpyHostToDevice));
-                CK(cudaMemcpy(c.slink_rank, rk.data(), 4 * nl, cudaMemcpyHostToDevice));
-                CK(cudaMemcpy(c.seg_bnd, sb.data(), 8 * sb.size(), cudaMemcpyHostToDevice));
-                c.bvals_ready = 1;
-                c.bvals_valid = 0;
-                // ghost-pass records once the wall cells' values are kept:
-                // upstream cell, the two interpolation weights, wall-cell rank
-                // (the linear scheme: 2q, 1 - 2q on f_l(x_f), f_l(x_f - c_l)
-                // for q < 1/2; 1/(2q), (2q - 1)/(2q) on f_l(x_f), f_ibar(x_f)
-                // for q >= 1/2; the single-node scheme keeps 0.5 (1 - 2q))
-                std::vector<uint4> r4(nl);
-                // the inline wall form's weights and lanes, in the order of the compact values
-                std::vector<uint2> wc(nl);
-                std::vector<unsigned short> wl(nl, 0);
-                bool rok = true;
-                for (size_t at = 0; at < nl && rok; at++) {
-                    const unsigned cell = pk[at].x & 0x3fffffffu, sch = pk[at].x >> 30;
-                    float qf;
-                    std::memcpy(&qf, &pk[at].y, 4);
-                    int l = 0;
-                    while (l < 19 && (long long)at >= c.slink_off[l + 1]) l++;
-                    const long long x = cell % c.nx, y = (cell / c.nx) % c.ny, z = cell / ((long long)c.nx * c.ny);
-                    const long long x1 = (x - cx(l) + c.nx) % c.nx, y1 = (y - cy(l) + c.ny) % c.ny,
-                                    z1 = (z - cz(l) + c.nz) % c.nz;
-                    const unsigned c1 = (unsigned)(x1 + c.nx * (y1 + (long long)c.ny * z1));
-                    const double q = (double)qf;
-                    float k1, k2;
-                    unsigned own = 0, single = 0;
-                    if (sch == 1 && q < 0.5) {
-                        k1 = (float)(2.0 * q);
-                        k2 = (float)(1.0 - 2.0 * q);
-                    } else if (sch == 1) {
-                        k1 = (float)(1.0 / (2.0 * q));
-                        k2 = (float)((2.0 * q - 1.0) / (2.0 * q));
-                        own = 1;
-                    } else if (sch == 2) {
-                        k1 = 1.0f;
-                        k2 = (float)(0.5 * (1.0 - 2.0 * q));
-                        single = 1;
-                    } else {
-                        rok = false;  // the quadratic scheme keeps the general pass
-                        break;
-                    }
-                    unsigned b1, b2;
-                    std::memcpy(&b1, &k1, 4);
-                    std::memcpy(&b2, &k2, 4);
-                    r4[at] = make_uint4(c1 | (own << 30) | (single << 31), b1, b2, (unsigned)rk[at]);
-                    wc[(size_t)gx[at]] = make_uint2(b1, b2 | (own << 31));
-                }
-                for (size_t r = 0; r < bcells.size() && rok; r++) {
-                    if (lane_of[r] < 0) {
-                        rok = false;  // a wall cell no sweep lane holds
-                        break;
-                    }
-                    for (int i = 0; i < 19; i++)
-                        if ((wr[r].y >> i) & 1u)
-                            wl[wr[r].x + (unsigned)__builtin_popcount(wr[r].y & ((1u << i) - 1u))] =
-                                (unsigned short)(lane_of[r] | (i << 5));
-                }
-                rok = rok && c.pipe_nowrap;  // the pass recovers x_f from x_f - c_l across z ends only
-                if (rok) {
-                    CK(cudaMemcpy(c.slink4, r4.data(), 16 * nl, cudaMemcpyHostToDevice));
-                    CK(cudaMemcpy(c.wcoef, wc.data(), 8 * nl, cudaMemcpyHostToDevice));
-                    CK(cudaMemcpy(c.wlane, wl.data(), 2 * nl, cudaMemcpyHostToDevice));
-                }
-                c.slink4_ready = rok ? 1 : 0;
-                c.wcoef_ready = rok ? 1 : 0;
-                // 16-bit storage: the pair sweep's work list and wall tables
-                if (rok && (c.storage == LBM_F16S || c.storage == LBM_BF16S)) build_pair16(c, fl.data(), bcells, wr);
-            }
-        }
-    }
-    return LBM_OK;
+    return build_columns(c);
 }
 
 lbm_status lbm_add_spheres(lbm_ctx *h, int n, const double *xyz, const double *radius, double density_ratio,
@@ -1058,12 +913,11 @@ lbm_status lbm_step(lbm_ctx *h, int nsteps, int bc) {
             close(G_BULK, b0);
         } else if (bc == LBM_BC_IBB) {
             const long long l0 = c.group_launches[G_BND];
-            CK(launch_ibb_links(c));
+            if (c.np > 0) CK(launch_ibb_links(c));
             close(G_BND, l0);
             b0 = c.group_launches[G_BULK];
-            CK(launch_stream_collide(c, bc));
-            // what the sweep left for the next step's wall
-            c.bvals_valid = pipe_inline_walls(c) ? 2 : (c.bvals_ready ? 1 : 0);
+            if (c.zlay) CK(launch_column_sweep(c));
+            else CK(launch_stream_collide(c, bc));
             close(G_BULK, b0);
             const long long p0 = c.group_launches[G_PART];
             if (c.np > 0) CK(launch_gimem(c));
@@ -1432,7 +1286,12 @@ lbm_status lbm_checkpoint(lbm_ctx *h, const char *path) {
     F.f = fopen(path, "wb");
     if (!F.f) return io_fail(c, "open", path);
     if (fwrite(&H, sizeof(H), 1, F.f) != 1) return io_fail(c, "write", path);
-    CKS(dev_to_file(c, F.f, c.fA, (size_t)c.q * (size_t)c.N * storage_bytes(c.storage), path));
+    const void *pops = c.fA;
+    if (c.zlay) {  // the file keeps x fastest; the other buffer is free between steps
+        CK(convert_columns(c, c.fA, c.fB, true, false));
+        pops = c.fB;
+    }
+    CKS(dev_to_file(c, F.f, pops, (size_t)c.q * (size_t)c.N * storage_bytes(c.storage), path));
     if (c.np > 0) {
         const size_t b3 = sizeof(double) * 3 * (size_t)c.np;
         for (const double *p : {c.X, c.U, c.W, c.Fh, c.Th, c.Fprev, c.Tprev, c.Fc, c.Iu, c.Ir})
@@ -1504,8 +1363,11 @@ lbm_status lbm_restore(lbm_ctx *h, const char *path) {
     if (H.armed_bc >= 0) CKS(arm(c, H.armed_bc));
     // then the saved state over what the set-up computed
     if (fseek(F.f, (long)sizeof(H), SEEK_SET) != 0) return io_fail(c, "seek", path);
-    CKS(file_to_dev(c, F.f, c.fA, pop_bytes, path));
-    c.bvals_valid = 0;  // the next ghost pass reads the wall cells from the populations
+    CKS(file_to_dev(c, F.f, c.zlay ? c.fB : c.fA, pop_bytes, path));
+    if (c.zlay) {
+        CK(convert_columns(c, c.fB, c.fA, false, c.q == 19));
+        CK(cudaMemsetAsync(c.fB, 0, (size_t)c.q * (size_t)c.Np * storage_bytes(c.storage), c.stream));
+    }
     if (H.np > 0) {
         if (fseek(F.f, (long)(sizeof(double) * (10 * 3 + 1) * (size_t)H.np + sizeof(int) * (size_t)H.np), SEEK_CUR) != 0)
             return io_fail(c, "seek", path);

@@ -47,45 +47,15 @@ struct Ctx {
     int8_t *link_dir, *link_scheme;
     double *link_q;
     void *link_dP, *link_dT;  // per-link momentum exchange and torque (arithmetic type of the storage)
-    // row segments of the fluid extent (IBB walls with a solid margin)
-    uint4 *seg;  // warp items of the pipe sweep (segments.h)
-    long long nseg, max_seg;
-    // static wall (pipe) links regrouped by direction for the ghost pass:
-    // x = cell | scheme << 30, y = bits of q rounded to FP32
-    uint2 *slink;
-    int slink_off[20];  // first link of each direction, and the total
-    int static_links;   // 1: the ghost pass uses slink (FP32-arithmetic storages)
-    long long static_single;  // single-node (scheme 2) links of the static wall
-    // wall cells' post-collision populations, written by the sweep for the
-    // next ghost pass: 19 values (storage type) per wall cell in cell order
-    int *slink_rank;    // per static link: rank of its wall cell
-    uint4 *slink4;      // per static link: upstream cell | flags, two weights, wall-cell rank
-    int slink4_ready;   // 1: the records hold every static link
-    uint2 *seg_bnd;     // per sweep item: rank of its first wall cell, lane mask of wall cells
-    void *bvals;
-    long long max_bvals;
-    // compact ghosts: the ghost pass stores the bounced values here (one per
-    // link, storage type) instead of in the solid nodes' slots; per wall
-    // cell (rank) a record {first value, mask of the directions it replaces}
-    uint2 *wrec;
-    int *gidx;          // per static link: index of its value
-    void *gvals;
-    int bvals_ready;    // the tables above are built
-    int pipe_nowrap;    // no fluid cell on an x or y face: pulls wrap only in z (lean pipe sweep)
-    // what the last sweep left for the next step's wall: 0 nothing (read
-    // the populations), 1 bvals holds the wall cells' values of the current
-    // state, 2 gvals holds the partial values p of the inline wall form
-    int bvals_valid;
-    uint2 *wcoef;       // inline wall form: per compact value k1, k2 (bit 31: q >= 1/2)
-    unsigned short *wlane;  // inline wall form: per compact value its wall cell's sweep lane | direction << 5
-    // the pair sweep of 16-bit storage (sweep_pair16.cu): items of up to 32
-    // cell pairs, per item {first slot, links, 64-bit wall-cell mask}, per
-    // compact value the cell of its item | direction << 6
-    uint4 *pair_items, *pair_wall;
-    unsigned short *wslot;
-    long long npair_items;
-    int pair_ready;
-    int wcoef_ready;
+    // column layout of the pipe (columns.cuh), in use once zlay is set
+    int zlay, zp;      // zp: elements from a column to the next (>= nz)
+    long long Np;      // elements of a population plane in that layout
+    int2 *col_list;    // fluid columns: x + nx y, index of the column's wall record or -1
+    long long ncols;
+    uint4 *col_wall;   // per wall column: direction masks of its links, of those with q >= 1/2, of single-node ones
+    void *col_coef;    // per wall column 19 pairs of weights (arithmetic type of the storage)
+    long long static_single;  // single-node (scheme 2) links of a plane of the wall
+    int pipe_nowrap;   // no fluid cell on an x or y face: pulls wrap only in z
     // compaction scratch
     int nblk;
     long long *blk_sites, *blk_links;
@@ -174,11 +144,12 @@ cudaError_t launch_init_equilibrium(Ctx &c, const double *u_dev, double rho0);
 cudaError_t launch_set_populations(Ctx &c, const double *f_dev);
 cudaError_t launch_get_populations(Ctx &c, double *f_dev);
 cudaError_t launch_stream_collide(Ctx &c, int bc);
-bool launch_pipe_sweep(Ctx &c, cudaError_t &err);  // sweep_pipe.cu: false when it does not apply
-bool pipe_inline_walls(const Ctx &c);             // the lean sweep runs the inline wall form
-bool launch_pair16_sweep(Ctx &c, cudaError_t &err);  // sweep_pair16.cu: false when it does not apply
-bool build_pair16(Ctx &c, const uint8_t *fl, const std::vector<int> &bcells, const std::vector<uint2> &wr);
-cudaError_t launch_pipe_wall_prime(Ctx &c);       // partial values p from the populations
+cudaError_t launch_column_sweep(Ctx &c);  // sweep_columns.cu: the pipe's IBB step
+// columns.cu: the state between the two layouts, one plane to or from
+// c.rho_f, the macroscopic fields
+cudaError_t convert_columns(Ctx &c, const void *src, void *dst, bool to_x, bool zero_solid);
+cudaError_t column_plane_copy(Ctx &c, int i, double w, bool to_f64);
+cudaError_t launch_column_macro(Ctx &c);
 cudaError_t launch_ibb_links(Ctx &c);
 cudaEvent_t prof_event(Ctx &c);  // profiling event on the stream (null when off)
 void prof_span(Ctx &c, int g, cudaEvent_t a, cudaEvent_t b);  // time from a to b into group g

@@ -81,9 +81,7 @@ struct LinkArgs {
 };
 
 
-// PART: some links belong to moving walls (particles); the pipe wall alone
-// needs neither the wall velocity nor the momentum exchange
-template <int S, bool PART>
+template <int S>
 __global__ void __launch_bounds__(256) ibb_links(LinkArgs a) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
@@ -96,7 +94,7 @@ __global__ void __launch_bounds__(256) ibb_links(LinkArgs a) {
         const int c = a.link_cell[k];
         const int l = a.link_dir[k];
         const int sch = a.link_scheme[k];
-        const int pid = PART ? a.link_pid[k] : -1;
+        const int pid = a.link_pid[k];
         const double q = a.link_q[k];
         const unsigned zq = a.dxy.div((unsigned)c), rem = (unsigned)c - zq * (unsigned)(nx * ny);
         const unsigned yq = a.dx.div(rem);
@@ -112,10 +110,7 @@ __global__ void __launch_bounds__(256) ibb_links(LinkArgs a) {
         const R fi0 = Store<S>::ld(A + (size_t)i * N + c);  // f*_ibar(x_f)
         // scheme 2 stores the halfway value here; single_node_fix adds the
         // single-node correction (and its momentum) afterwards
-        if constexpr (!PART) {
-            const R v = ibb_value<S>(A, N, l, i, sch, R(q), c1, c2, R(0), fl0, fi0);
-            Store<S>::st(A + (size_t)i * N + cb, v);  // pulled by x_f as f_ibar(x_f, t+1)
-        } else if constexpr (sizeof(R) == 8) {
+        if constexpr (sizeof(R) == 8) {
             // FP64 storage: wall velocity and momentum exchange in FP64
             double uw[3] = {0.0, 0.0, 0.0};
             if (pid >= 0) {
@@ -192,7 +187,7 @@ __global__ void __launch_bounds__(256) ibb_links(LinkArgs a) {
 // particle links the momentum the correction carries, (c_l + u_w) dv, and
 // its torque. Kept out of ibb_links so that the rare scheme costs the
 // common link pass no registers.
-template <int S, bool PART>
+template <int S>
 __global__ void __launch_bounds__(256) single_node_fix(LinkArgs a) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
@@ -217,47 +212,45 @@ __global__ void __launch_bounds__(256) single_node_fix(LinkArgs a) {
                      single_node_pair<S>(A + c, N, l, body_force<R>(a, 0), body_force<R>(a, 1), body_force<R>(a, 2), a.rt);
         T *slot = A + (size_t)i * N + cb;
         Store<S>::st(slot, Store<S>::ld(slot) + dv);
-        if constexpr (PART) {
-            const int pid = a.link_pid[k];
-            if (pid < 0) continue;
-            // the wall velocity and lever arm of ibb_links, in the same arithmetic
-            R uw[3], m[3];
-            if constexpr (sizeof(R) == 8) {
-                const double r0 = mimg(x + q * lx - a.X[3 * pid + 0], nx);
-                const double r1 = mimg(y + q * ly - a.X[3 * pid + 1], ny);
-                const double r2 = mimg(z + q * lz - a.X[3 * pid + 2], nz);
-                const double *Wp = a.W + 3 * pid, *Up = a.U + 3 * pid;
-                uw[0] = Up[0] + (Wp[1] * r2 - Wp[2] * r1);
-                uw[1] = Up[1] + (Wp[2] * r0 - Wp[0] * r2);
-                uw[2] = Up[2] + (Wp[0] * r1 - Wp[1] * r0);
-                m[0] = mimg(x + 0.5 * lx - a.X[3 * pid + 0], nx);
-                m[1] = mimg(y + 0.5 * ly - a.X[3 * pid + 1], ny);
-                m[2] = mimg(z + 0.5 * lz - a.X[3 * pid + 2], nz);
-            } else {
-                const float d0 = float(mimg(double(x) - a.X[3 * pid + 0], nx));
-                const float d1 = float(mimg(double(y) - a.X[3 * pid + 1], ny));
-                const float d2 = float(mimg(double(z) - a.X[3 * pid + 2], nz));
-                const float qf = float(q);
-                const float r0 = d0 + qf * lx, r1 = d1 + qf * ly, r2 = d2 + qf * lz;
-                const double *Wp = a.W + 3 * pid, *Up = a.U + 3 * pid;
-                const float W0 = float(Wp[0]), W1 = float(Wp[1]), W2 = float(Wp[2]);
-                uw[0] = float(Up[0]) + (W1 * r2 - W2 * r1);
-                uw[1] = float(Up[1]) + (W2 * r0 - W0 * r2);
-                uw[2] = float(Up[2]) + (W0 * r1 - W1 * r0);
-                m[0] = d0 + 0.5f * lx;
-                m[1] = d1 + 0.5f * ly;
-                m[2] = d2 + 0.5f * lz;
-            }
-            // dP = (c_l - u_w) f_out - (c_ibar - u_w) f_in: f_in grew by dv
-            const R e0 = (R(lx) + uw[0]) * dv, e1 = (R(ly) + uw[1]) * dv, e2 = (R(lz) + uw[2]) * dv;
-            R *dP = (R *)a.link_dP + 3 * k, *dT = (R *)a.link_dT + 3 * k;
-            dP[0] += e0;
-            dP[1] += e1;
-            dP[2] += e2;
-            dT[0] += m[1] * e2 - m[2] * e1;
-            dT[1] += m[2] * e0 - m[0] * e2;
-            dT[2] += m[0] * e1 - m[1] * e0;
+        const int pid = a.link_pid[k];
+        if (pid < 0) continue;
+        // the wall velocity and lever arm of ibb_links, in the same arithmetic
+        R uw[3], m[3];
+        if constexpr (sizeof(R) == 8) {
+            const double r0 = mimg(x + q * lx - a.X[3 * pid + 0], nx);
+            const double r1 = mimg(y + q * ly - a.X[3 * pid + 1], ny);
+            const double r2 = mimg(z + q * lz - a.X[3 * pid + 2], nz);
+            const double *Wp = a.W + 3 * pid, *Up = a.U + 3 * pid;
+            uw[0] = Up[0] + (Wp[1] * r2 - Wp[2] * r1);
+            uw[1] = Up[1] + (Wp[2] * r0 - Wp[0] * r2);
+            uw[2] = Up[2] + (Wp[0] * r1 - Wp[1] * r0);
+            m[0] = mimg(x + 0.5 * lx - a.X[3 * pid + 0], nx);
+            m[1] = mimg(y + 0.5 * ly - a.X[3 * pid + 1], ny);
+            m[2] = mimg(z + 0.5 * lz - a.X[3 * pid + 2], nz);
+        } else {
+            const float d0 = float(mimg(double(x) - a.X[3 * pid + 0], nx));
+            const float d1 = float(mimg(double(y) - a.X[3 * pid + 1], ny));
+            const float d2 = float(mimg(double(z) - a.X[3 * pid + 2], nz));
+            const float qf = float(q);
+            const float r0 = d0 + qf * lx, r1 = d1 + qf * ly, r2 = d2 + qf * lz;
+            const double *Wp = a.W + 3 * pid, *Up = a.U + 3 * pid;
+            const float W0 = float(Wp[0]), W1 = float(Wp[1]), W2 = float(Wp[2]);
+            uw[0] = float(Up[0]) + (W1 * r2 - W2 * r1);
+            uw[1] = float(Up[1]) + (W2 * r0 - W0 * r2);
+            uw[2] = float(Up[2]) + (W0 * r1 - W1 * r0);
+            m[0] = d0 + 0.5f * lx;
+            m[1] = d1 + 0.5f * ly;
+            m[2] = d2 + 0.5f * lz;
         }
+        // dP = (c_l - u_w) f_out - (c_ibar - u_w) f_in: f_in grew by dv
+        const R e0 = (R(lx) + uw[0]) * dv, e1 = (R(ly) + uw[1]) * dv, e2 = (R(lz) + uw[2]) * dv;
+        R *dP = (R *)a.link_dP + 3 * k, *dT = (R *)a.link_dT + 3 * k;
+        dP[0] += e0;
+        dP[1] += e1;
+        dP[2] += e2;
+        dT[0] += m[1] * e2 - m[2] * e1;
+        dT[1] += m[2] * e0 - m[0] * e2;
+        dT[2] += m[0] * e1 - m[1] * e0;
     }
 }
 
@@ -317,164 +310,9 @@ static unsigned site_grid(const Ctx &c, int tb) {
     return (unsigned)nb;
 }
 
-// Ghost pass of a static wall (no particle links), FP32 arithmetic: links
-// regrouped by direction, blockIdx.y = direction l, so l, c_l and ibar are
-// uniform over the block and neighbouring threads touch neighbouring cells.
-struct StaticLinkArgs {
-    void *A;
-    const uint4 *slink4;  // link records of the kept-values pass (see ibb_links_kept)
-    const uint2 *slink;  // x = cell | scheme << 30, y = FP32 bits of q
-    const int *rank;     // wall-cell rank of each link
-    const void *bvals;   // wall cells' values (19 per cell), or null: read A
-    const int *gidx;     // compact ghost value of each link
-    void *gvals;         // compact ghost values (null: store in the solid nodes' slots)
-    int off[20];
-    int nx, ny, nz;
-    long long N;
-    FastDiv dx, dxy;
-    double F[3];  // body force on fluid cells (single-node fallback)
-    float Fs[3];
-    Rates rt;
-};
-
-// The ghost pass of the static wall from per-link records (16 bytes: the
-// upstream cell x_f - c_l with the flags "second value is f_ibar(x_f)" and
-// "single-node", the two FP32 weights, the wall cell's rank), grouped by
-// direction as the links are:
-//   v = k1 f*_l(x_f) + k2 f*_l(x_f - c_l)   (linear, q < 1/2)
-//   v = k1 f*_l(x_f) + k2 f*_ibar(x_f)      (linear, q >= 1/2)
-//   v = f*_l(x_f) + k2 (d_l + d_ibar)       (single-node, Sec. 3.1)
-// The wall cell's own populations come from the values the last sweep kept
-// (19 per wall cell), or, before the first sweep, from A at x_f (only z
-// wraps between x_f - c_l and x_f: the walls of this pass touch no x or y
-// face). No division or index decoding per link.
-template <int S, bool SN>
-__global__ void __launch_bounds__(256) ibb_links_kept(StaticLinkArgs a) {
-    typedef typename Store<S>::T T;
-    typedef typename Store<S>::R R;
-    const int l = blockIdx.y;
-    const int k0 = a.off[l], k1 = a.off[l + 1];
-    const size_t N = (size_t)a.N;
-    const T *A = (const T *)a.A + (size_t)l * N;  // plane l
-    const int i = opp(l);
-    const bool kept = a.bvals != nullptr;
-    const long long offl = (long long)cx(l) + (long long)a.nx * (cy(l) + (long long)a.ny * cz(l));
-    for (int k = k0 + blockIdx.x * blockDim.x + threadIdx.x; k < k1; k += gridDim.x * blockDim.x) {
-        const uint4 m = __ldg(a.slink4 + k);
-        const int gi = __ldg(a.gidx + k);
-        const unsigned c1 = m.x & 0x3fffffffu;
-        const bool own = (m.x >> 30) & 1u, single = m.x >> 31;
-        const T *wv;
-        size_t stride;
-        if (kept) {
-            wv = (const T *)a.bvals + (size_t)19 * m.w;
-            stride = 1;
-        } else {
-            long long c = (long long)c1 + offl;
-            c = c < 0 ? c + (long long)N : (c >= (long long)N ? c - (long long)N : c);
-            wv = (const T *)a.A + c;
-            stride = N;
-        }
-        const R fl0 = Store<S>::ld(wv + (size_t)l * stride);
-        const R second = own ? Store<S>::ld(wv + (size_t)i * stride) : (single ? R(0) : Store<S>::ld(A + c1));
-        R v = fmaf(R(__uint_as_float(m.y)), fl0, R(__uint_as_float(m.z)) * second);
-        if (SN && single)
-            v = fmaf(R(__uint_as_float(m.z)),
-                     single_node_pair<S>(wv, stride, l, body_force<R>(a, 0), body_force<R>(a, 1), body_force<R>(a, 2),
-                                         a.rt),
-                     fl0);
-        Store<S>::st((T *)a.gvals + gi, v);
-    }
-}
-
-template <int S, bool SN>
-__global__ void __launch_bounds__(256) ibb_links_static(StaticLinkArgs a) {
-    typedef typename Store<S>::T T;
-    typedef typename Store<S>::R R;
-    const int l = blockIdx.y;
-    const int k0 = a.off[l], k1 = a.off[l + 1];
-    T *A = (T *)a.A;
-    const size_t N = (size_t)a.N;
-    const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const int lx = cx(l), ly = cy(l), lz = cz(l), i = opp(l);
-    for (int k = k0 + blockIdx.x * blockDim.x + threadIdx.x; k < k1; k += gridDim.x * blockDim.x) {
-        const uint2 m = __ldg(a.slink + k);
-        const int c = (int)(m.x & 0x3fffffffu), sch = (int)(m.x >> 30);
-        const R qq = R(__uint_as_float(m.y));
-        const unsigned zq = a.dxy.div((unsigned)c), rem = (unsigned)c - zq * (unsigned)(nx * ny);
-        const unsigned yq = a.dx.div(rem);
-        const int z = (int)zq, y = (int)yq, x = (int)(rem - yq * (unsigned)nx);
-        const int cb = wrap(x + lx, nx) + nx * (wrap(y + ly, ny) + ny * wrap(z + lz, nz));
-        const int x1 = wrap(x - lx, nx), y1 = wrap(y - ly, ny), z1 = wrap(z - lz, nz);
-        const int c1 = x1 + nx * (y1 + ny * z1);
-        const int c2 = wrap(x1 - lx, nx) + nx * (wrap(y1 - ly, ny) + ny * wrap(z1 - lz, nz));
-        R fl0, fi0;
-        if (a.bvals) {  // the same values, kept contiguous by the last sweep
-            const T *wv = (const T *)a.bvals + (size_t)19 * __ldg(a.rank + k);
-            fl0 = Store<S>::ld(wv + l);
-            fi0 = Store<S>::ld(wv + i);
-        } else {
-            fl0 = Store<S>::ld(A + (size_t)l * N + c);
-            fi0 = Store<S>::ld(A + (size_t)i * N + c);
-        }
-        R v = ibb_value<S>(A, N, l, i, sch, qq, c1, c2, R(0), fl0, fi0);
-        if (SN && sch == 2) {  // single-node fallback from the wall cell's own values
-            const T *p = a.bvals ? (const T *)a.bvals + (size_t)19 * __ldg(a.rank + k) : A + c;
-            v += R(0.5) * (R(1) - R(2) * qq) *
-                 single_node_pair<S>(p, a.bvals ? 1 : N, l, body_force<R>(a, 0), body_force<R>(a, 1),
-                                     body_force<R>(a, 2), a.rt);
-        }
-        if (a.gvals)
-            Store<S>::st((T *)a.gvals + __ldg(a.gidx + k), v);  // read by the sweep in place of the pull
-        else
-            Store<S>::st(A + (size_t)i * N + cb, v);
-    }
-}
-
 template <int S>
 static cudaError_t launch_links_s(Ctx &c) {
     if (c.max_links == 0) return cudaSuccess;
-    if (c.static_links && c.np == 0 && S != LBM_F64) {
-        // the inline wall form: the last sweep left the partial values, or
-        // they are formed once from the populations
-        if (pipe_inline_walls(c)) return c.bvals_valid == 2 ? cudaSuccess : launch_pipe_wall_prime(c);
-        StaticLinkArgs a;
-        a.A = c.fA;
-        a.slink4 = c.slink4;
-        a.slink = c.slink;
-        a.rank = c.slink_rank;
-        a.bvals = c.bvals_valid == 1 ? c.bvals : nullptr;
-        a.gidx = c.gidx;
-        a.gvals = c.bvals_ready ? c.gvals : nullptr;
-        for (int l = 0; l < 20; l++) a.off[l] = c.slink_off[l];
-        a.nx = c.nx;
-        a.ny = c.ny;
-        a.nz = c.nz;
-        a.N = c.N;
-        a.dx = FastDiv((unsigned)c.nx);
-        a.dxy = FastDiv((unsigned)(c.nx * c.ny));
-        for (int d = 0; d < 3; d++) {
-            a.F[d] = c.F[d];
-            a.Fs[d] = (float)c.F[d];
-        }
-        a.rt = c.rt;
-        int most = 0;
-        for (int l = 0; l < 19; l++) most = std::max(most, c.slink_off[l + 1] - c.slink_off[l]);
-        unsigned nbx = (unsigned)((most + 255) / 256);
-        if (nbx < 1) nbx = 1;
-
-        count_launch(c, G_BND);
-        // the variant with the single-node scheme only for walls that have such links
-        if (c.slink4_ready && a.gvals) {  // every step, so a restart repeats the same arithmetic
-            if (c.static_single > 0) ibb_links_kept<S, true><<<dim3(nbx, 19), 256, 0, c.stream>>>(a);
-            else ibb_links_kept<S, false><<<dim3(nbx, 19), 256, 0, c.stream>>>(a);
-        } else if (c.static_single > 0) {
-            ibb_links_static<S, true><<<dim3(nbx, 19), 256, 0, c.stream>>>(a);
-        } else {
-            ibb_links_static<S, false><<<dim3(nbx, 19), 256, 0, c.stream>>>(a);
-        }
-        return cudaGetLastError();
-    }
     LinkArgs a{c.fA, c.link_cell, c.link_pid, c.link_dir, c.link_scheme, c.link_q, c.link_dP, c.link_dT,
                c.X, c.U, c.W, c.d_counts, c.max_links, c.nx, c.ny, c.nz, c.N,
                FastDiv((unsigned)c.nx), FastDiv((unsigned)(c.nx * c.ny)), {c.F[0], c.F[1], c.F[2]},
@@ -485,18 +323,13 @@ static cudaError_t launch_links_s(Ctx &c) {
     if (nb < 1) nb = 1;
     if (nb > 152LL * 64) nb = 152LL * 64;
     count_launch(c, G_BND);
-    if (c.np > 0) ibb_links<S, true><<<(unsigned)nb, 256, 0, c.stream>>>(a);
-    else ibb_links<S, false><<<(unsigned)nb, 256, 0, c.stream>>>(a);
+    ibb_links<S><<<(unsigned)nb, 256, 0, c.stream>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // moving walls may have single-node links at any step; a static wall only if its list has some
-    if (c.np > 0 || c.static_single > 0) {
-        count_launch(c, G_BND);
-        const unsigned nbs = 152u * 2u;  // a few single-node links: a small grid striding over the list
-        if (c.np > 0) single_node_fix<S, true><<<nbs, 256, 0, c.stream>>>(a);
-        else single_node_fix<S, false><<<nbs, 256, 0, c.stream>>>(a);
-        e = cudaGetLastError();
-    }
+    // there may be single-node links at any step: a small grid striding over their list
+    count_launch(c, G_BND);
+    single_node_fix<S><<<152u * 2u, 256, 0, c.stream>>>(a);
+    e = cudaGetLastError();
     return e;
 }
 

@@ -1,0 +1,86 @@
+"""The pipe sweep on the column layout (z fastest) against the oracle: plane
+counts around the 32-cell chunk and the column pitch, odd sections, walls
+that touch the box faces, single-node links, every storage type and both
+collisions; populations in and out of the layout."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"f64": 1e-12, "f32": 1e-5, "f16s": 2e-3, "bf16s": 3e-2}
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1906_05448_gb300 import build, lbm as L
+    build.build()
+    L.load()
+    return L
+
+
+def rel(a, b):
+    return float(np.max(np.abs(a - b)) / max(np.max(np.abs(b)), 1e-300))
+
+
+def pair(lbm, nx, ny, nz, R, storage, rates, seed=3):
+    u = workloads.pipe_velocity(nx, ny, nz, R, 0.03, perturbation=0.1, seed=seed)
+    g = lbm.Lattice(nx, ny, nz, 0.57, force=(1e-6, 0, 4e-6), storage=storage, rates=rates)
+    o = oracle.Sim(nx, ny, nz, 0.57, force=(1e-6, 0, 4e-6), rates=rates)
+    for s in (g, o):
+        s.init_velocity(u)
+        s.set_pipe(R)
+    return g, o
+
+
+@pytest.mark.parametrize("nx,ny,nz,R", [
+    (24, 24, 4, 10.3),     # fewer planes than a pitch group
+    (27, 26, 31, 11.7),    # one chunk, one lane idle
+    (27, 26, 32, 11.7),    # one whole chunk
+    (27, 29, 33, 12.1),    # a second chunk of one cell
+    (31, 30, 65, 13.6),
+    (16, 16, 20, 8.0),     # the wall touches the box faces: pulls wrap in x and y
+    (16, 16, 9, 6.4),      # single-node links
+])
+@pytest.mark.parametrize("storage", ["f64", "f32", "f16s", "bf16s"])
+def test_steps_match_the_oracle(lbm, nx, ny, nz, R, storage):
+    for rates in (oracle.RATES_SRT, oracle.RATES_DHUMIERES):
+        g, o = pair(lbm, nx, ny, nz, R, storage, rates)
+        g.step(20, lbm.BC_IBB)
+        o.step(20, oracle.BC_IBB)
+        fluid = o.solid()[0] == 0
+        rg, ug = g.macro()
+        ro, uo = o.macro()
+        assert rel(ug[:, fluid], uo[:, fluid]) < TOL[storage]
+        assert rel(rg[fluid], ro[fluid]) < TOL[storage]
+        assert not np.any(ug[:, ~fluid]) and not np.any(rg[~fluid])
+        if storage == "f64":
+            assert rel(g.populations()[:, fluid], o.populations()[:, fluid]) < TOL[storage]
+        g.close()
+        o.close()
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_populations_set_between_steps(lbm, storage):
+    """Populations taken out of the layout and put into another context that
+    is already stepping continue the same run."""
+    g, _ = pair(lbm, 27, 26, 33, 11.7, storage, oracle.RATES_SRT)
+    h, _ = pair(lbm, 27, 26, 33, 11.7, storage, oracle.RATES_SRT, seed=8)
+    g.step(3, lbm.BC_IBB)
+    h.step(1, lbm.BC_IBB)
+    f = g.populations()
+    h.set_populations(f)
+    assert rel(h.populations(), f) < 1e-7
+    g.step(4, lbm.BC_IBB)
+    h.step(4, lbm.BC_IBB)
+    fluid = (g.flags() & 1) == 0
+    # FP32: f = g + w read out in FP64 loses nothing, put back it rounds to the same g
+    assert np.array_equal(g.populations()[:, fluid], h.populations()[:, fluid]) if storage == "f32" else \
+        rel(h.populations()[:, fluid], g.populations()[:, fluid]) < 1e-14
+    g.close()
+    h.close()
