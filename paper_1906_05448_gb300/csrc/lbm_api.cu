@@ -572,7 +572,7 @@ lbm_status enter_columns(Ctx &c) {
 
 lbm_status arm(Ctx &c, int bc) {
     c.armed_bc = bc;
-    if (bc == LBM_BC_IBB && c.has_pipe && c.q == 19) {
+    if (c.has_pipe && (bc == LBM_BC_IBB || c.q == 27)) {
         lbm_status s = enter_columns(c);
         if (s != LBM_OK) return s;
     }
@@ -803,12 +803,17 @@ lbm_status lbm_set_pipe(lbm_ctx *h, double radius) {
         q27_pipe_colmask(c, mask);
         CK(cudaMemcpy(c.q27_colmask, mask.data(), sizeof(unsigned) * mask.size(), cudaMemcpyHostToDevice));
         CK(launch_q27_coef(c));
-        // no fluid column on an x or y face: the sweep addresses pulls by plane pointers
+        std::vector<int2> cols;
         c.pipe_nowrap = 1;
         for (int y = 0; y < c.ny; y++)
-            for (int x = 0; x < c.nx; x++)
-                if (!(mask[(size_t)x + (size_t)c.nx * y] & 1u) && (x == 0 || x == c.nx - 1 || y == 0 || y == c.ny - 1))
-                    c.pipe_nowrap = 0;
+            for (int x = 0; x < c.nx; x++) {
+                const unsigned m = mask[(size_t)x + (size_t)c.nx * y];
+                if (m & 1u) continue;
+                cols.push_back(make_int2(x + c.nx * y, m != 0u));
+                if (x == 0 || x == c.nx - 1 || y == 0 || y == c.ny - 1) c.pipe_nowrap = 0;
+            }
+        c.ncols = (long long)cols.size();
+        if (!cols.empty()) CK(cudaMemcpy(c.col_list, cols.data(), sizeof(int2) * cols.size(), cudaMemcpyHostToDevice));
         return sync_all(c);
     }
     c.has_pipe = 1;

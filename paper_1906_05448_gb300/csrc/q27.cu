@@ -7,13 +7,9 @@
 // faces, the 12 edges, the 8 corners; within a group the triples
 // (c_x, c_y, c_z) over {-1, 0, 1}^3 in lexicographic order (c_x slowest).
 // Weights 8/27, 2/27, 1/54, 1/216 by |c|^2 = 0 .. 3.
-#include "lbm_internal.cuh"
+#include "columns.cuh"
 
 #include <vector>
-
-#ifndef LBM_Q27_MINB
-#define LBM_Q27_MINB 0  // resident blocks of 256 per SM the pipe kernel's registers are sized for (0: per storage)
-#endif
 
 namespace lbmgb {
 
@@ -84,6 +80,43 @@ __global__ void q27_macro_kernel(const void *A, double *rho_o, double *u_o, long
     u_o[c] = double((j0 - R(0.5) * R(F0)) * ir);
     u_o[N + c] = double((j1 - R(0.5) * R(F1)) * ir);
     u_o[2 * N + c] = double((j2 - R(0.5) * R(F2)) * ir);
+}
+
+// the same on the column layout (columns.cuh): read along z, written along x
+template <int S>
+__global__ void __launch_bounds__(256) q27_column_macro_kernel(const void *A, double *rho_o, double *u_o, int nx, int ny,
+                                                               int nz, int zp, long long N, long long Np, double F0,
+                                                               double F1, double F2) {
+    typedef typename Store<S>::T T;
+    typedef typename Store<S>::R R;
+    struct V {
+        R rho, ux, uy, uz;
+    };
+    __shared__ V sh[COL_TILE][COL_TILE + 1];
+    for (int y = blockIdx.z; y < ny; y += gridDim.z)
+        column_exchange<V, true>(
+            sh, nx, nz,
+            [&](int x, int z) {
+                const T *P = (const T *)A + (size_t)(x + nx * y) * zp + z;
+                R r = R(0), j0 = R(0), j1 = R(0), j2 = R(0);
+#pragma unroll
+                for (int i = 0; i < Q27; i++) {
+                    const R g = Store<S>::ld(P + i * Np);
+                    r += g;
+                    j0 += g * R(q27x(i));
+                    j1 += g * R(q27y(i));
+                    j2 += g * R(q27z(i));
+                }
+                const R rho = R(1) + r, ir = R(1) / rho;
+                return V{rho, (j0 - R(0.5) * R(F0)) * ir, (j1 - R(0.5) * R(F1)) * ir, (j2 - R(0.5) * R(F2)) * ir};
+            },
+            [&](int x, int z, const V &v) {
+                const long long c = x + (long long)nx * (y + (long long)ny * z);
+                rho_o[c] = double(v.rho);
+                u_o[c] = double(v.ux);
+                u_o[N + c] = double(v.uy);
+                u_o[2 * N + c] = double(v.uz);
+            });
 }
 
 struct Q27Args {
@@ -182,12 +215,15 @@ struct Q27PipeArgs {
     Q27Args b;
     const unsigned *colmask, *hmask;
     const void *coef;  // per column x 27 directions: two weights in the arithmetic type
-    // when no fluid cell touches an x or y face: the pull of direction i
-    // for cell c is Ap[i][c] (plus N or minus N across the z ends), its
-    // store Bp[i][c]: one address operation per access
-    int nowrap;
-    const void *Ap[Q27];  // A + i N - (c_x + nx c_y + nx ny c_z)
-    void *Bp[Q27];        // B + i N
+    const int2 *cols;  // fluid columns: x + nx y, nonzero if the column has wall links
+    unsigned ncols, nchunk;
+    FastDiv fd_chunk;
+    int zp;
+    long long Np;
+    // the pull of direction i for element e of a plane is Ap[i][e] (plus nz
+    // or minus nz across the z ends), its store Bp[i][e]
+    const void *Ap[Q27];  // A + i Np - (c_z + zp (c_x + nx c_y))
+    void *Bp[Q27];        // B + i Np
 };
 
 template <typename R>
@@ -233,49 +269,52 @@ __global__ void q27_coef_kernel(const unsigned *colmask, unsigned *hmask, void *
     hmask[col] = h;
 }
 
-// FP32: registers for 4 resident blocks of 256 per SM (64, no spills):
-// 0.387 ms per step on the benchmark pipe against 0.477 ms at 80 registers
-// (3 blocks), where only 13 of the 24 possible warps were active (the solid
-// cells' threads end at once, their blocks stay resident)
-constexpr int q27_min_blocks(int S) { return LBM_Q27_MINB > 0 ? LBM_Q27_MINB : (S == LBM_F32 ? 4 : 1); }
+// On the column layout (columns.cuh): one warp per 32 consecutive z of a
+// fluid column, the column's mask and weights uniform over the warp. What
+// bounds it: HBM. 0.259 ms per step on the benchmark pipe (148 x 148 x 438,
+// R = 73, FP32): 6.12 TB/s of its 216 B per fluid cell; the sweep over
+// x-fast cells, whose warps mixed fluid, wall and solid cells, took 0.386.
+// Registers for 4 resident blocks of 256 per SM (64, no spills); 3, 5 and 6
+// blocks took 0.283, 0.267 (32 bytes spilled) and 0.315 ms.
+constexpr int q27_min_blocks(int S) { return S == LBM_F32 ? 4 : 2; }
 
-template <int S, bool FORCE>
-__global__ void __launch_bounds__(256, q27_min_blocks(S)) q27_pipe_kernel(Q27PipeArgs pa) {
+// WRAP: fluid columns touch an x or y face of the box
+template <int S, bool FORCE, bool WRAP>
+__global__ void __launch_bounds__(256, q27_min_blocks(S)) q27_columns_kernel(Q27PipeArgs pa) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
     const Q27Args &a = pa.b;
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= a.N) return;
+    const unsigned item = blockIdx.x * 8 + threadIdx.x / 32;
+    const unsigned ci = pa.fd_chunk.div(item);
+    if (ci >= pa.ncols) return;
+    const int2 col = __ldg(pa.cols + ci);
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const unsigned zq = a.fxy.div((unsigned)c), rem = (unsigned)c - zq * (unsigned)(nx * ny);
-    const unsigned yq = a.fx.div(rem);
-    const int z = (int)zq, y = (int)yq, x = (int)(rem - yq * (unsigned)nx);
-    const unsigned m = __ldg(pa.colmask + rem);
-    if (m & 1u) return;  // solid: keeps its values, never read
-    const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
-    const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
-    const int zm = z == 0 ? nz - 1 : z - 1, zp = z == nz - 1 ? 0 : z + 1;
+    const int z = (int)(item - ci * pa.nchunk) * 32 + (int)(threadIdx.x & 31);
+    if (z >= nz) return;
+    const int c = col.x * pa.zp + z;
+    const int zlo = z == 0 ? nz : 0, zhi = z == nz - 1 ? nz : 0;
     const T *__restrict__ A = (const T *)a.A;
-    T *__restrict__ B = (T *)a.B;
-    const size_t N = (size_t)a.N;
+    const size_t N = (size_t)pa.Np;
     R g[Q27];
-    if (pa.nowrap) {
-        const int zpl = z == 0 ? (int)N : 0, zmi = z == nz - 1 ? (int)N : 0;
-#pragma unroll
-        for (int i = 0; i < Q27; i++) {
-            const int o = (int)c + (q27z(i) > 0 ? zpl : 0) - (q27z(i) < 0 ? zmi : 0);
-            g[i] = Store<S>::ld((const T *)pa.Ap[i] + o);
-        }
-    } else {
+    if constexpr (WRAP) {
+        const int y = (int)a.fx.div((unsigned)col.x), x = col.x - y * nx;
+        const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+        const int ym = y == 0 ? ny - 1 : y - 1, yp = y == ny - 1 ? 0 : y + 1;
 #pragma unroll
         for (int i = 0; i < Q27; i++) {
             const int xs = q27x(i) > 0 ? xm : (q27x(i) < 0 ? xp : x);
             const int ys = q27y(i) > 0 ? ym : (q27y(i) < 0 ? yp : y);
-            const int zs = q27z(i) > 0 ? zm : (q27z(i) < 0 ? zp : z);
-            g[i] = Store<S>::ld(A + (i * N + (size_t)(xs + nx * (ys + ny * zs))));
+            const int zs = z - q27z(i) + (q27z(i) > 0 ? zlo : 0) - (q27z(i) < 0 ? zhi : 0);
+            g[i] = Store<S>::ld(A + i * N + (xs + nx * ys) * pa.zp + zs);
         }
+    } else {
+#pragma unroll
+        for (int i = 0; i < Q27; i++)
+            g[i] = Store<S>::ld((const T *)pa.Ap[i] + (c + (q27z(i) > 0 ? zlo : 0) - (q27z(i) < 0 ? zhi : 0)));
     }
-    if (m) {  // wall cell: the populations coming back from the wall
+    const unsigned rem = (unsigned)col.x;
+    if (col.y) {  // wall column (uniform over the warp): the populations coming back from the wall
+        const unsigned m = __ldg(pa.colmask + rem);
         const unsigned h = __ldg(pa.hmask + rem);
         const Q27Coef<R> *kc = (const Q27Coef<R> *)pa.coef + (size_t)rem * Q27;
 #pragma unroll
@@ -315,7 +354,7 @@ __global__ void __launch_bounds__(256, q27_min_blocks(S)) q27_pipe_kernel(Q27Pip
             const R cF = R(q27x(i)) * Fx + R(q27y(i)) * Fy + R(q27z(i)) * Fz;
             v += (c1 * R(q27w(i))) * (R(3) * cF - uF3 + R(9) * cu * cF);
         }
-        Store<S>::st(pa.nowrap ? (T *)pa.Bp[i] + c : B + (i * N + (size_t)c), v);
+        Store<S>::st((T *)pa.Bp[i] + c, v);
     }
     watchdog(rho, ux, uy, uz, a.status);
 }
@@ -351,21 +390,29 @@ cudaError_t launch_q27_step(Ctx &c) {
         pa.colmask = c.q27_colmask;
         pa.hmask = c.q27_hmask;
         pa.coef = c.q27_coef;
-        pa.nowrap = c.pipe_nowrap && c.N < (1LL << 30);
-        const size_t sb = storage_bytes(c.storage);
+        pa.cols = c.col_list;
+        pa.ncols = (unsigned)c.ncols;
+        pa.nchunk = (unsigned)((c.nz + 31) / 32);
+        pa.fd_chunk = FastDiv(pa.nchunk);
+        pa.zp = c.zp;
+        pa.Np = c.Np;
+        const long long sb = (long long)storage_bytes(c.storage);
         for (int i = 0; i < Q27; i++) {
-            const long long off = q27x(i) + (long long)c.nx * q27y(i) + (long long)c.nx * c.ny * q27z(i);
-            pa.Ap[i] = (const void *)((const char *)c.fA + sb * (size_t)((long long)i * c.N - off));
-            pa.Bp[i] = (void *)((char *)c.fB + sb * (size_t)((long long)i * c.N));
+            const long long off = q27z(i) + (long long)c.zp * (q27x(i) + (long long)c.nx * q27y(i));
+            pa.Ap[i] = (const void *)((const char *)c.fA + sb * (i * c.Np - off));
+            pa.Bp[i] = (void *)((char *)c.fB + sb * (i * c.Np));
         }
-        const unsigned nb = (unsigned)((c.N + 255) / 256);
+        const unsigned nb = (unsigned)(((long long)pa.ncols * pa.nchunk + 7) / 8);
+        if (nb == 0) return cudaSuccess;
+#define QC(S, W)                                                                       \
+    if (force) q27_columns_kernel<S, true, W><<<nb, 256, 0, c.stream>>>(pa);           \
+    else q27_columns_kernel<S, false, W><<<nb, 256, 0, c.stream>>>(pa)
         if (c.storage == LBM_F64) {
-            if (force) q27_pipe_kernel<LBM_F64, true><<<nb, 256, 0, c.stream>>>(pa);
-            else q27_pipe_kernel<LBM_F64, false><<<nb, 256, 0, c.stream>>>(pa);
+            if (c.pipe_nowrap) { QC(LBM_F64, false); } else { QC(LBM_F64, true); }
         } else {
-            if (force) q27_pipe_kernel<LBM_F32, true><<<nb, 256, 0, c.stream>>>(pa);
-            else q27_pipe_kernel<LBM_F32, false><<<nb, 256, 0, c.stream>>>(pa);
+            if (c.pipe_nowrap) { QC(LBM_F32, false); } else { QC(LBM_F32, true); }
         }
+#undef QC
         return cudaGetLastError();
     }
     return c.storage == LBM_F64 ? q27_step_s<LBM_F64>(c, a, force) : q27_step_s<LBM_F32>(c, a, force);
@@ -413,6 +460,7 @@ cudaError_t launch_q27_init(Ctx &c, const double *u_dev, double rho0) {
 
 // one population plane to or from the FP64 scratch c.rho_f (unshifted f)
 cudaError_t q27_plane_copy(Ctx &c, int i, bool to_f64) {
+    if (c.zlay) return column_plane_copy(c, i, q27w(i), to_f64);
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     if (c.storage == LBM_F64) q27_plane_kernel<LBM_F64><<<nb, 256, 0, c.stream>>>(c.fA, c.rho_f, c.N, i, to_f64);
     else q27_plane_kernel<LBM_F32><<<nb, 256, 0, c.stream>>>(c.fA, c.rho_f, c.N, i, to_f64);
@@ -421,6 +469,15 @@ cudaError_t q27_plane_copy(Ctx &c, int i, bool to_f64) {
 
 cudaError_t launch_q27_macro(Ctx &c) {
     count_launch(c, G_STATS);
+    if (c.zlay) {
+#define MK(S)                                                                                                      \
+    q27_column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, c.rho_f, c.u_f, c.nx, c.ny, c.nz, c.zp, c.N, \
+                                                                    c.Np, c.F[0], c.F[1], c.F[2])
+        if (c.storage == LBM_F64) MK(LBM_F64);
+        else MK(LBM_F32);
+#undef MK
+        return cudaGetLastError();
+    }
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     if (c.storage == LBM_F64)
         q27_macro_kernel<LBM_F64><<<nb, 256, 0, c.stream>>>(c.fA, c.rho_f, c.u_f, c.N, c.F[0], c.F[1], c.F[2]);

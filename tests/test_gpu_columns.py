@@ -84,3 +84,26 @@ def test_populations_set_between_steps(lbm, storage):
         rel(h.populations()[:, fluid], g.populations()[:, fluid]) < 1e-14
     g.close()
     h.close()
+
+
+@pytest.mark.parametrize("nz", [4, 32, 33])
+@pytest.mark.parametrize("nx,ny,R", [(27, 24, 10.3), (16, 16, 8.0)])  # the second wraps in x and y
+def test_d3q27_plane_counts(lbm, nx, ny, R, nz):
+    from oracle import d3q27 as q27
+    tau, F = 0.62, (1e-6, 0.0, 3e-6)
+    u = workloads.pipe_velocity(nx, ny, nz, R, 0.02, perturbation=0.1, seed=5)
+    g = lbm.Lattice(nx, ny, nz, tau, force=F, storage="f64", lattice=27)
+    g.init_velocity(u)
+    g.set_pipe(R)
+    solid = q27.pipe_solid(nx, ny, nz, R)
+    links = q27.pipe_links(solid, R)
+    o = q27.feq(np.ones((nz, ny, nx)), u)
+    fl = ~solid.reshape(-1)
+    g.step(3, lbm.BC_IBB)
+    for _ in range(3):
+        o = q27.step_pipe(o, solid, links, tau, F)
+    assert rel(g.populations()[:, fl], o.reshape(27, -1)[:, fl]) < 1e-12
+    rg, ug = g.macro()
+    ro, uo = q27.macro(o, F)
+    assert rel(ug[:, fl], uo.reshape(3, -1)[:, fl]) < 1e-12 and rel(rg[fl], ro.reshape(-1)[fl]) < 1e-12
+    g.close()
