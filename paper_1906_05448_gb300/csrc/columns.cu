@@ -81,11 +81,14 @@ cudaError_t column_plane_copy(Ctx &c, int i, double w, bool to_f64) {
 }
 
 // rho and u of the post-collision state (macro_kernel's arithmetic), read
-// along z and written along x as FP64
+// along z and written along x as FP64. IBM (info not null): the total force
+// of the last collision is the body force on fluid columns plus the IBM
+// force planes sF of the support columns.
 template <int S>
-__global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const uint8_t *flags, double *rho_o,
-                                                           double *u_o, int nx, int ny, int nz, int zp, long long N,
-                                                           long long Np, double F0, double F1, double F2) {
+__global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const uint8_t *flags, const int *info,
+                                                           const void *sFv, long long SF, double *rho_o, double *u_o,
+                                                           int nx, int ny, int nz, int zp, long long N, long long Np,
+                                                           double F0, double F1, double F2) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
     struct V {
@@ -97,7 +100,8 @@ __global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const 
         sh, nx, nz,
         [&](int x, int z) {
             const int col = x + nx * y;
-            if (flags[col] & FL_SOLID) return V{R(0), R(0), R(0), R(0)};  // solid column: plane 0 tells
+            const bool solid = flags[col] & FL_SOLID;  // plane 0 tells
+            if (solid && !info) return V{R(0), R(0), R(0), R(0)};
             const T *P = (const T *)A + (size_t)col * zp + z;
             R r = R(0), j0 = R(0), j1 = R(0), j2 = R(0);
 #pragma unroll
@@ -108,8 +112,16 @@ __global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const 
                 j1 += g * R(cy(i));
                 j2 += g * R(cz(i));
             }
+            R Fx = solid ? R(0) : R(F0), Fy = solid ? R(0) : R(F1), Fz = solid ? R(0) : R(F2);
+            const int k = info ? (info[col] >> 1) - 1 : -1;
+            if (k >= 0) {
+                const R *sF = (const R *)sFv + (size_t)k * nz + z;
+                Fx += sF[0];
+                Fy += sF[SF];
+                Fz += sF[2 * SF];
+            }
             const R rho = R(1) + r, ir = R(1) / rho;
-            return V{rho, (j0 - R(0.5) * R(F0)) * ir, (j1 - R(0.5) * R(F1)) * ir, (j2 - R(0.5) * R(F2)) * ir};
+            return V{rho, (j0 - R(0.5) * Fx) * ir, (j1 - R(0.5) * Fy) * ir, (j2 - R(0.5) * Fz) * ir};
         },
         [&](int x, int z, const V &v) {
             const long long c = x + (long long)nx * (y + (long long)ny * z);
@@ -122,8 +134,10 @@ __global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const 
 
 cudaError_t launch_column_macro(Ctx &c) {
     count_launch(c, G_STATS);
+    const int *info = c.armed_bc == LBM_BC_IBB ? nullptr : c.col_ibm;
+    const long long SF = (long long)c.pipe_sp * c.nz;
     switch (c.storage) {
-#define MK(S) column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, c.flags, c.rho_f, c.u_f, c.nx, c.ny, \
+#define MK(S) column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, c.flags, info, c.sup_F, SF, c.rho_f, c.u_f, c.nx, c.ny, \
                                                                            c.nz, c.zp, c.N, c.Np, c.F[0], c.F[1], c.F[2])
     case LBM_F64: MK(LBM_F64); break;
     case LBM_F32: MK(LBM_F32); break;

@@ -33,7 +33,7 @@ struct Plan {
     size_t fA, fB, flags, owner, aux;
     size_t site_cell, site_first, site_mask, sup_ru, sup_F, sup_Fp;
     size_t link_cell, link_pid, link_dir, link_scheme, link_q, link_dP, link_dT;
-    size_t blk_sites, blk_links, counts, status, col_list, col_wall, col_coef, refill;
+    size_t blk_sites, blk_links, counts, status, col_list, col_wall, col_coef, col_ibm, refill;
     long long max_refill;
     int zp;
     long long Np;
@@ -112,6 +112,7 @@ bool make_plan(const lbm_grid *g, Plan &P) {
     P.col_list = L.take(8 * nxy);
     P.col_wall = L.take(16 * nxy);
     P.col_coef = L.take(16 * 19 * nxy);
+    P.col_ibm = L.take(4 * nxy);
     P.blk_sites = L.take(8 * (size_t)P.nblk);
     P.blk_links = L.take(8 * (size_t)P.nblk);
     P.counts = L.take(64);
@@ -457,19 +458,23 @@ lbm_status build_markers(Ctx &c) {
 }
 
 // The pipe's support set is the same in every z plane and the sites are
-// listed in cell order, so site (x, y, z) = z * S_p + k(x, y). For each ring
-// marker, its 4 x 4 column box gives up to 16 (k, x-y weight) entries; the
-// interpolation then needs no per-node lookup. Left unbuilt (pipe_sp = 0)
-// when the site list is not of that form.
+// listed in cell order, so site (x, y, z) = z * S_p + k(x, y): a set of
+// support columns k. For each ring marker, its 4 x 4 column box gives up to
+// 16 (k, x-y weight) entries; per column the step needs k and whether it is
+// solid.
 lbm_status build_pipe_interp(Ctx &c) {
-    c.pipe_sp = 0;
     const long long ns = c.nsites;
-    if (ns <= 0 || ns % c.nz != 0 || c.pipe_nc <= 0 || c.pipe_nc > c.pipe_max_ring || ns > c.max_sites) return LBM_OK;
+    if (ns <= 0 || ns % c.nz != 0 || c.pipe_nc <= 0 || c.pipe_nc > c.pipe_max_ring || ns > c.max_sites)
+        return fail(c, LBM_EINVAL, "pipe support set of %lld cells does not fit its columns", ns);
     const long long sp = ns / c.nz, nxy = (long long)c.nx * c.ny;
-    std::vector<int> cell((size_t)ns);
-    CK(cudaMemcpy(cell.data(), c.site_cell, sizeof(int) * ns, cudaMemcpyDeviceToHost));
-    for (long long i = 0; i < ns; i++)
-        if ((long long)cell[i] - (i / sp) * nxy != (long long)cell[i % sp]) return LBM_OK;  // not plane-invariant
+    std::vector<int> cell((size_t)sp), info((size_t)nxy);
+    std::vector<uint8_t> fl((size_t)nxy);
+    CK(cudaMemcpy(cell.data(), c.site_cell, sizeof(int) * sp, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(fl.data(), c.flags, (size_t)nxy, cudaMemcpyDeviceToHost));
+    if (cell[(size_t)sp - 1] >= nxy) return fail(c, LBM_EINVAL, "pipe support set differs between planes");
+    for (long long k = 0; k < nxy; k++) info[k] = fl[k] & FL_SOLID ? 1 : 0;
+    for (long long k = 0; k < sp; k++) info[cell[k]] |= (int)(k + 1) << 1;
+    CK(cudaMemcpy(c.col_ibm, info.data(), sizeof(int) * nxy, cudaMemcpyHostToDevice));
     std::vector<int> local((size_t)nxy, -1);
     for (long long k = 0; k < sp; k++) local[cell[k]] = (int)k;
     const double RL = c.pipe_R + c.rd;
@@ -558,12 +563,13 @@ lbm_status build_columns(Ctx &c) {
     return LBM_OK;
 }
 
-// put the state into the column layout (first step with a wall on a pipe)
-lbm_status enter_columns(Ctx &c) {
+// put the state into the column layout (first step with a wall on a pipe);
+// zero_solid: nothing is kept of the solid columns
+lbm_status enter_columns(Ctx &c, bool zero_solid) {
     const size_t bytes = (size_t)c.q * (size_t)c.Np * storage_bytes(c.storage);
     count_launch(c, G_BND);
     CK(cudaMemsetAsync(c.fB, 0, bytes, c.stream));
-    CK(convert_columns(c, c.fA, c.fB, false, c.q == 19));
+    CK(convert_columns(c, c.fA, c.fB, false, zero_solid));
     CK(cudaMemsetAsync(c.fA, 0, bytes, c.stream));
     std::swap(c.fA, c.fB);
     c.zlay = 1;
@@ -573,7 +579,7 @@ lbm_status enter_columns(Ctx &c) {
 lbm_status arm(Ctx &c, int bc) {
     c.armed_bc = bc;
     if (c.has_pipe && (bc == LBM_BC_IBB || c.q == 27)) {
-        lbm_status s = enter_columns(c);
+        lbm_status s = enter_columns(c, c.q == 19);
         if (s != LBM_OK) return s;
     }
     if (bc == LBM_BC_IBM_U || bc == LBM_BC_IBM_B) {
@@ -596,6 +602,7 @@ lbm_status arm(Ctx &c, int bc) {
         c.nsites_hint = c.nsites;
         if (c.has_pipe && c.np == 0) {
             s = build_pipe_interp(c);
+            if (s == LBM_OK) s = enter_columns(c, false);
             if (s != LBM_OK) return s;
         }
     }
@@ -678,6 +685,7 @@ lbm_status lbm_create(const lbm_grid *grid, double tau, const double force[3], v
     c.col_list = (int2 *)(b + P.col_list);
     c.col_wall = (uint4 *)(b + P.col_wall);
     c.col_coef = b + P.col_coef;
+    c.col_ibm = (int *)(b + P.col_ibm);
     c.nblk = P.nblk;
     c.blk_sites = (long long *)(b + P.blk_sites);
     c.blk_links = (long long *)(b + P.blk_links);
@@ -944,13 +952,16 @@ lbm_status lbm_step(lbm_ctx *h, int nsteps, int bc) {
             }
             close(G_GEOM, g0);
             b0 = c.group_launches[G_BULK];
-            CK(launch_stream_collide(c, bc));
+            if (c.zlay) CK(launch_ibm_columns_sweep(c));
+            else CK(launch_stream_collide(c, bc));
             close(G_BULK, b0);
             const long long i0 = c.group_launches[G_IBM];
-            CK(launch_ibm_passes(c));
+            if (c.zlay) CK(launch_ibm_columns_passes(c));
+            else CK(launch_ibm_passes(c));
             close(G_IBM, i0);
             const long long k0 = c.group_launches[G_IBMCOL];
-            CK(launch_ibm_collide(c));
+            if (c.zlay) CK(launch_ibm_columns_collide(c));
+            else CK(launch_ibm_collide(c));
             close(G_IBMCOL, k0);
             const long long p0 = c.group_launches[G_PART];
             if (c.np > 0) CK(launch_ibm_particle_sums(c, false));
@@ -1078,14 +1089,18 @@ lbm_status lbm_get_field(lbm_ctx *h, int which, void *dst, size_t bytes) {
     case LBM_FIELD_IBM_FORCE: {
         if (bytes < 3 * N * sizeof(double)) return fail(c, LBM_EINVAL, "destination too small");
         CK(cudaMemsetAsync(c.u_f, 0, 3 * N * sizeof(double), c.stream));
-        if (c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B)
-        {
+        if (c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B) {
+            const void *sF = c.sup_F;
+            if (c.zlay) {  // in the order of the site list, in the buffer that the next step overwrites
+                CK(copy_site_force(c, c.fB, true));
+                sF = c.fB;
+            }
             if (c.storage == LBM_F64)
-                dense_ibm_force<double><<<1024, 256, 0, c.stream>>>(c.u_f, (const double *)c.sup_F, c.site_cell,
-                                                                     c.d_counts, c.max_sites, c.N);
+                dense_ibm_force<double><<<1024, 256, 0, c.stream>>>(c.u_f, (const double *)sF, c.site_cell, c.d_counts,
+                                                                     c.max_sites, c.N);
             else
-                dense_ibm_force<float><<<1024, 256, 0, c.stream>>>(c.u_f, (const float *)c.sup_F, c.site_cell,
-                                                                    c.d_counts, c.max_sites, c.N);
+                dense_ibm_force<float><<<1024, 256, 0, c.stream>>>(c.u_f, (const float *)sF, c.site_cell, c.d_counts,
+                                                                    c.max_sites, c.N);
         }
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(dst, c.u_f, 3 * N * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
@@ -1166,6 +1181,7 @@ lbm_status lbm_get_markers(lbm_ctx *h, long long capacity, double *X, double *F,
     if (capacity < c.nm) return fail(c, LBM_EINVAL, "capacity %lld < %lld markers", capacity, c.nm);
     if (c.nm == 0) return s;
     if (X) CK(cudaMemcpyAsync(X, c.mX, 24 * c.nm, cudaMemcpyDeviceToHost, c.stream));
+    if (F) CK(refresh_markers(c));
     if (F) CK(cudaMemcpyAsync(F, c.mFacc, 24 * c.nm, cudaMemcpyDeviceToHost, c.stream));
     if (dV) CK(cudaMemcpyAsync(dV, c.mdV, 8 * c.nm, cudaMemcpyDeviceToHost, c.stream));
     if (pid) CK(cudaMemcpyAsync(pid, c.mpid, 4 * c.nm, cudaMemcpyDeviceToHost, c.stream));
@@ -1306,8 +1322,14 @@ lbm_status lbm_checkpoint(lbm_ctx *h, const char *path) {
     }
     if (H.nsites > 0) {
         CKS(dev_to_file(c, F.f, c.site_cell, sizeof(int) * (size_t)H.nsites, path));
-        CKS(dev_to_file(c, F.f, c.sup_F, 3 * arith_bytes(c) * (size_t)H.nsites, path));
+        const void *sF = c.sup_F;
+        if (c.zlay) {
+            CK(copy_site_force(c, c.fB, true));
+            sF = c.fB;
+        }
+        CKS(dev_to_file(c, F.f, sF, 3 * arith_bytes(c) * (size_t)H.nsites, path));
     }
+    if (H.nm > 0) CK(refresh_markers(c));
     if (H.nm > 0) CKS(dev_to_file(c, F.f, c.mFacc, sizeof(double) * 3 * (size_t)H.nm, path));
     if (c.cl_ready) CKS(dev_to_file(c, F.f, c.cl_w, sizeof(float) * LBM_MLP_NPARAM, path));
     if (fflush(F.f) != 0) return io_fail(c, "write", path);
@@ -1370,7 +1392,7 @@ lbm_status lbm_restore(lbm_ctx *h, const char *path) {
     if (fseek(F.f, (long)sizeof(H), SEEK_SET) != 0) return io_fail(c, "seek", path);
     CKS(file_to_dev(c, F.f, c.zlay ? c.fB : c.fA, pop_bytes, path));
     if (c.zlay) {
-        CK(convert_columns(c, c.fB, c.fA, false, c.q == 19));
+        CK(convert_columns(c, c.fB, c.fA, false, c.q == 19 && c.armed_bc == LBM_BC_IBB));
         CK(cudaMemsetAsync(c.fB, 0, (size_t)c.q * (size_t)c.Np * storage_bytes(c.storage), c.stream));
     }
     if (H.np > 0) {
@@ -1397,7 +1419,8 @@ lbm_status lbm_restore(lbm_ctx *h, const char *path) {
         CKS(sync_all(c));
         if (H.nsites != c.nsites) return fail(c, LBM_EINVAL, "checkpoint support set is not a support set of this grid");
         c.nsites_hint = c.nsites;
-        CKS(file_to_dev(c, F.f, c.sup_F, 3 * arith_bytes(c) * (size_t)H.nsites, path));
+        CKS(file_to_dev(c, F.f, c.zlay ? c.fB : c.sup_F, 3 * arith_bytes(c) * (size_t)H.nsites, path));
+        if (c.zlay) CK(copy_site_force(c, c.fB, false));
     }
     if (H.nm > 0) {
         if (H.nm != c.nm) return fail(c, LBM_EINVAL, "checkpoint markers differ from the rebuilt ones");

@@ -54,6 +54,8 @@ struct Ctx {
     long long ncols;
     uint4 *col_wall;   // per wall column: direction masks of its links, of those with q >= 1/2, of single-node ones
     void *col_coef;    // per wall column 19 pairs of weights (arithmetic type of the storage)
+    int *col_ibm;      // IBM: per column (support index + 1) << 1 | solid
+    int markers_stale; // IBM on columns: the marker forces of the last step are not in mFacc yet
     long long static_single;  // single-node (scheme 2) links of a plane of the wall
     int pipe_nowrap;   // no fluid cell on an x or y face: pulls wrap only in z
     // compaction scratch
@@ -90,7 +92,7 @@ struct Ctx {
     void *pipe_xy_w;  // x-y weights in the storage's arithmetic type
     long long pipe_max_xy;
     // pipe interpolation: per ring marker, 16 (support site in a plane, x-y
-    // weight) entries; pipe_sp = support sites per z plane (0: not built)
+    // weight) entries; pipe_sp = support sites per z plane
     int *pipe_it_k;
     void *pipe_it_w;  // arithmetic type of the storage
     int pipe_sp, pipe_max_ring;
@@ -150,6 +152,12 @@ cudaError_t launch_column_sweep(Ctx &c);  // sweep_columns.cu: the pipe's IBB st
 cudaError_t convert_columns(Ctx &c, const void *src, void *dst, bool to_x, bool zero_solid);
 cudaError_t column_plane_copy(Ctx &c, int i, double w, bool to_f64);
 cudaError_t launch_column_macro(Ctx &c);
+// ibm_columns.cu: the pipe's IBM step, and its forces in the order of the ABI
+cudaError_t launch_ibm_columns_sweep(Ctx &c);
+cudaError_t launch_ibm_columns_passes(Ctx &c);
+cudaError_t launch_ibm_columns_collide(Ctx &c);
+cudaError_t refresh_markers(Ctx &c);
+cudaError_t copy_site_force(Ctx &c, void *list, bool out);
 cudaError_t launch_ibb_links(Ctx &c);
 cudaEvent_t prof_event(Ctx &c);  // profiling event on the stream (null when off)
 void prof_span(Ctx &c, int g, cudaEvent_t a, cudaEvent_t b);  // time from a to b into group g

@@ -573,85 +573,6 @@ __global__ void __launch_bounds__(256) ibm_interp_warp_kernel(IbmArgs a) {
     }
 }
 
-// Pipe wall tiles. The ring of markers is the same in every z plane and sits
-// at integer z, so the z factor of the 4-point kernel takes the constants
-// phi(0) = 1/2, phi(+-1) = 1/4 (phi(+-2) = 0), and the x-y factor of every
-// (marker, site) pair is the same in all planes. A block takes 32 ring
-// markers (or 32 sites of a plane) over PIPE_ZT consecutive planes: it forms
-// the x-y sums once per plane, for its planes and one halo plane on each
-// side, in shared memory, and combines three neighbouring planes per output.
-// Each plane's x-y sum is gathered once instead of three times.
-#ifndef LBM_PIPE_ZT
-#define LBM_PIPE_ZT 6  // measured: 6, 14, 30 planes -> 0.165, 0.166, 0.176 ms for 3 passes
-#endif
-constexpr int PIPE_ZT = LBM_PIPE_ZT;
-constexpr int PIPE_ZH = PIPE_ZT + 2;  // with the halo planes
-
-__device__ __forceinline__ int zwrap(int z, int nz) {
-    z %= nz;
-    return z < 0 ? z + nz : z;
-}
-
-struct PipeInterpArgs {
-    const int *it_k;
-    const void *it_w;  // R
-    const void *sup_ru;
-    double *mFacc;
-    void *mFaccR, *mFr;
-    int nc, nz, sp, pass, last;
-    double dV;  // ring marker volume
-};
-
-// U*_l = sum over planes dz = -1, 0, 1 of phi_z(dz) times the sum over the
-// 16 column entries of ring marker j of w_xy u*(site) in plane z + dz (the
-// 4-point delta interpolation, Sec. 3.1); then the direct-forcing force
-// F_l = 2 rho_l (U_d - U*_l) with U_d = 0 on the fixed wall (Sec. 2.1)
-template <typename R>
-__global__ void __launch_bounds__(256) ibm_interp_pipe_kernel(PipeInterpArgs a) {
-    __shared__ R P[PIPE_ZH][32][4];
-    const int jj = threadIdx.x & 31, j = blockIdx.x * 32 + jj;
-    const int z0 = blockIdx.y * PIPE_ZT;
-    const R *ru = (const R *)a.sup_ru;
-    const R *tw = (const R *)a.it_w + 16 * (size_t)j;
-    const int *tk = a.it_k + 16 * (size_t)j;
-    for (int pz = threadIdx.x >> 5; pz < PIPE_ZH; pz += blockDim.x >> 5) {
-        R q[4] = {R(0), R(0), R(0), R(0)};
-        if (j < a.nc) {
-            // all 16 gathers in flight at once (an entry without a site has
-            // weight 0 and index 0: its load is in bounds and not summed)
-            const R *rp = ru + 4 * (size_t)zwrap(z0 - 1 + pz, a.nz) * a.sp;
-            R v[16][4];
-#pragma unroll
-            for (int e = 0; e < 16; e++) ld_site4(rp + 4 * (size_t)tk[e], v[e]);
-#pragma unroll
-            for (int e = 0; e < 16; e++) {
-                const R w = tw[e];
-                if (w != R(0))
-                    for (int d = 0; d < 4; d++) q[d] += w * v[e][d];
-            }
-        }
-        for (int d = 0; d < 4; d++) P[pz][jj][d] = q[d];
-    }
-    __syncthreads();
-    if (j >= a.nc) return;
-    R *mFr = (R *)a.mFr, *acc = (R *)a.mFaccR;
-    const R dVl = R(a.dV);
-    for (int pz = threadIdx.x >> 5; pz < PIPE_ZT; pz += blockDim.x >> 5) {
-        const int z = z0 + pz;
-        if (z >= a.nz) break;
-        const long long l = (long long)z * a.nc + j;
-        R q[4];
-        for (int d = 0; d < 4; d++) q[d] = R(0.25) * P[pz][jj][d] + R(0.5) * P[pz + 1][jj][d] + R(0.25) * P[pz + 2][jj][d];
-        for (int d = 0; d < 3; d++) {
-            const R Fl = R(2) * q[0] * (R(0) - q[1 + d]);
-            mFr[3 * l + d] = Fl * dVl;  // spread weight F_l dV_l
-            const R s = a.pass == 0 ? Fl : acc[3 * l + d] + Fl;
-            acc[3 * l + d] = s;
-            if (a.last) a.mFacc[3 * l + d] = double(s);
-        }
-    }
-}
-
 // generic spreading with global atomics (large particles only)
 template <typename R>
 __global__ void ibm_spread_kernel(IbmArgs a) {
@@ -685,112 +606,6 @@ __global__ void ibm_update_kernel(IbmArgs a) {
             ru[4 * s + 1 + d] += f * ir;
             sF[3 * s + d] = a.pass == 0 ? f : sF[3 * s + d] + f;
             Fp[3 * s + d] = R(0);
-        }
-    }
-}
-
-// Pipe wall: the ring of markers is the same in every z plane and sits at
-// integer z, so the z weights of the 4-point kernel are the constants
-// phi(0) = 1/2, phi(+-1) = 1/4 (phi(+-2) = 0). Each support cell gathers
-// from a fixed list of ring markers of its (x, y) column in the planes
-// z-1, z, z+1 -- no atomics, fixed order -- and applies the u* update.
-struct PipeSpreadArgs {
-    const int *site_cell;
-    const int *xy_start, *xy_j;
-    const void *xy_w;  // R
-    const void *mFr;
-    void *sup_ru, *sup_F;
-    const long long *counts;
-    long long max_sites;
-    int nx, ny, nz, nc;
-    int pass;
-};
-
-template <typename R>
-__global__ void __launch_bounds__(256) ibm_spread_pipe_kernel(PipeSpreadArgs a) {
-    const long long ns = a.counts[0] < a.max_sites ? a.counts[0] : a.max_sites;
-    const R *mFr = (const R *)a.mFr;
-    R *ru = (R *)a.sup_ru, *sF = (R *)a.sup_F;
-    const int nxy = a.nx * a.ny;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += (long long)gridDim.x * blockDim.x) {
-        const int c = a.site_cell[s];
-        const int z = c / nxy, xy = c - z * nxy;
-        const int j0 = a.xy_start[xy], j1 = a.xy_start[xy + 1];
-        R F0 = 0, F1 = 0, F2 = 0;
-        for (int dz = -1; dz <= 1; dz++) {
-            int zm = z - dz;
-            zm = zm < 0 ? zm + a.nz : (zm >= a.nz ? zm - a.nz : zm);
-            const R wz = R(dz == 0 ? 0.5 : 0.25);
-            const R *Fp = mFr + 3 * (long long)zm * a.nc;
-            for (int k = j0; k < j1; k++) {
-                const R w = ((const R *)a.xy_w)[k] * wz;
-                const int j = a.xy_j[k];
-                F0 += Fp[3 * j] * w;
-                F1 += Fp[3 * j + 1] * w;
-                F2 += Fp[3 * j + 2] * w;
-            }
-        }
-        const R ir = R(0.5) / ru[4 * s];
-        ru[4 * s + 1] += F0 * ir;
-        ru[4 * s + 2] += F1 * ir;
-        ru[4 * s + 3] += F2 * ir;
-        sF[3 * s] = a.pass == 0 ? F0 : sF[3 * s] + F0;
-        sF[3 * s + 1] = a.pass == 0 ? F1 : sF[3 * s + 1] + F1;
-        sF[3 * s + 2] = a.pass == 0 ? F2 : sF[3 * s + 2] + F2;
-    }
-}
-
-// The same spreading on the z tiles (sites s = z sp + k, plane-invariant):
-// the x-y sum Q(z', k) = sum over the ring markers of column k of
-// w_xy F_l dV_l in plane z' is formed once per plane, then
-// F(z, k) = Q(z+1, k)/4 + Q(z, k)/2 + Q(z-1, k)/4, followed by the u* update.
-struct PipeSpreadTileArgs {
-    const int *site_cell;  // the first sp sites (plane 0) give the (x, y) columns
-    const int *xy_start, *xy_j;
-    const void *xy_w;  // R
-    const void *mFr;
-    void *sup_ru, *sup_F;
-    int nz, nc, sp, pass;
-};
-
-template <typename R>
-__global__ void __launch_bounds__(256) ibm_spread_pipe_tiled_kernel(PipeSpreadTileArgs a) {
-    __shared__ R Q[PIPE_ZH][32][3];
-    const int kk = threadIdx.x & 31, k = blockIdx.x * 32 + kk;
-    const int z0 = blockIdx.y * PIPE_ZT;
-    const R *mFr = (const R *)a.mFr, *xw = (const R *)a.xy_w;
-    int e0 = 0, e1 = 0;
-    if (k < a.sp) {
-        const int xy = a.site_cell[k];
-        e0 = a.xy_start[xy];
-        e1 = a.xy_start[xy + 1];
-    }
-    for (int pz = threadIdx.x >> 5; pz < PIPE_ZH; pz += blockDim.x >> 5) {
-        const R *Fp = mFr + 3 * (size_t)zwrap(z0 - 1 + pz, a.nz) * a.nc;
-        R q0 = R(0), q1 = R(0), q2 = R(0);
-        for (int e = e0; e < e1; e++) {
-            const R w = xw[e];
-            const int j = a.xy_j[e];
-            q0 += Fp[3 * j] * w;
-            q1 += Fp[3 * j + 1] * w;
-            q2 += Fp[3 * j + 2] * w;
-        }
-        Q[pz][kk][0] = q0;
-        Q[pz][kk][1] = q1;
-        Q[pz][kk][2] = q2;
-    }
-    __syncthreads();
-    if (k >= a.sp) return;
-    R *ru = (R *)a.sup_ru, *sF = (R *)a.sup_F;
-    for (int pz = threadIdx.x >> 5; pz < PIPE_ZT; pz += blockDim.x >> 5) {
-        const int z = z0 + pz;
-        if (z >= a.nz) break;
-        const size_t s = (size_t)z * a.sp + k;
-        const R ir = R(0.5) / ru[4 * s];
-        for (int d = 0; d < 3; d++) {
-            const R F = R(0.25) * Q[pz + 2][kk][d] + R(0.5) * Q[pz + 1][kk][d] + R(0.25) * Q[pz][kk][d];
-            ru[4 * s + 1 + d] += F * ir;
-            sF[3 * s + d] = a.pass == 0 ? F : sF[3 * s + d] + F;
         }
     }
 }
@@ -874,7 +689,6 @@ static cudaError_t ibm_passes_t(Ctx &c) {
     long long ub = (ns + 255) / 256;
     if (ub < 1) ub = 1;
     if (ub > 152 * 32) ub = 152 * 32;
-    const bool pipe_gather = c.has_pipe && c.nm > 0 && c.pipe_nc > 0;
     // sphere boxes in shared memory when they fit
     const double RLmax = c.max_radius - c.rd;
     const int W = 2 * (int)ceil(RLmax) + 6;
@@ -891,31 +705,9 @@ static cudaError_t ibm_passes_t(Ctx &c) {
     for (int pass = 0; pass < 3; pass++) {
         a.pass = pass;
         a.last = pass == 2;
-        const bool pipe_tiles = c.nm > 0 && pipe_gather && c.pipe_sp > 0 && c.nm == (long long)c.nz * c.pipe_nc &&
-                                c.nz <= 65535LL * PIPE_ZT;
-        const dim3 zt_grid((unsigned)((c.nz + PIPE_ZT - 1) / PIPE_ZT));
-        if (pipe_tiles) {
-            PipeInterpArgs pi{c.pipe_it_k, c.pipe_it_w, c.sup_ru, c.mFacc, c.mFaccR, c.mFr,
-                              c.pipe_nc, c.nz, c.pipe_sp, pass, pass == 2, c.pipe_dV};
-            count_launch(c, G_IBM);
-            ibm_interp_pipe_kernel<R><<<dim3((unsigned)((c.pipe_nc + 31) / 32), zt_grid.x), 256, 0, c.stream>>>(pi);
-        } else if (c.nm > 0) {
+        if (c.nm > 0) {
             count_launch(c, G_IBM);
             ibm_interp_warp_kernel<R><<<(unsigned)((c.nm * 32 + 255) / 256), 256, 0, c.stream>>>(a);
-        }
-        if (pipe_tiles) {
-            PipeSpreadTileArgs ps{c.site_cell, c.pipe_xy_start, c.pipe_xy_j, c.pipe_xy_w, c.mFr, c.sup_ru,
-                                  c.sup_F, c.nz, c.pipe_nc, c.pipe_sp, pass};
-            count_launch(c, G_IBM);
-            ibm_spread_pipe_tiled_kernel<R><<<dim3((unsigned)((c.pipe_sp + 31) / 32), zt_grid.x), 256, 0, c.stream>>>(ps);
-            continue;
-        }
-        if (pipe_gather) {
-            PipeSpreadArgs ps{c.site_cell, c.pipe_xy_start, c.pipe_xy_j, c.pipe_xy_w, c.mFr, c.sup_ru,
-                              c.sup_F, c.d_counts, c.max_sites, c.nx, c.ny, c.nz, c.pipe_nc, pass};
-            count_launch(c, G_IBM);
-            ibm_spread_pipe_kernel<R><<<(unsigned)ub, 256, 0, c.stream>>>(ps);
-            continue;
         }
         if (c.nm > 0) {
             count_launch(c, G_IBM);

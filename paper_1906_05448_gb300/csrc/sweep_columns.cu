@@ -30,23 +30,18 @@ struct ColumnCoef {
 
 struct ColumnArgs {
     const void *A;
-    void *B;
     const int2 *cols;   // fluid columns: x + nx y, index of the column's wall record (-1: no wall link)
     const uint4 *wall;  // per wall column: direction masks of its links (x), of those with q >= 1/2 (y), single-node (z)
     const void *coef;   // per wall column 19 pairs of weights (arithmetic type of the storage)
     unsigned ncols, nchunk;
-    FastDiv fd_chunk, fd_nx;
-    int nx, ny, nz, zp;
+    FastDiv fd_chunk;
+    ColumnPtrs p;
     long long Np;
     unsigned *status;
     PairK pk;
     Rates rt;
     double F[3];
     float Fs[3];
-    // the pull of direction i for element e of a plane is Ap[i][e] (plus nz
-    // or minus nz across the z ends), its store Bp[i][e]
-    const void *Ap[19];  // A + i Np - (c_z + zp (c_x + nx c_y))
-    void *Bp[19];        // B + i Np
 };
 
 // Resident blocks of 256 per SM the registers are sized for. The sweep lives
@@ -92,25 +87,10 @@ __global__ void __launch_bounds__(256, column_min_blocks(S, SRT)) sweep_columns(
     if (ci >= a.ncols) return;
     const int2 col = __ldg(a.cols + ci);
     const int z = (int)(item - ci * a.nchunk) * 32 + (int)(threadIdx.x & 31);
-    if (z >= a.nz) return;
-    const int e = col.x * a.zp + z;
-    const int zlo = z == 0 ? a.nz : 0, zhi = z == a.nz - 1 ? a.nz : 0;
+    if (z >= a.p.nz) return;
+    const int e = col.x * a.p.zp + z;
     R g[19];
-    if constexpr (WRAP) {
-        const int y = (int)a.fd_nx.div((unsigned)col.x), x = col.x - y * a.nx;
-        const int xm = x == 0 ? a.nx - 1 : x - 1, xp = x == a.nx - 1 ? 0 : x + 1;
-        const int ym = y == 0 ? a.ny - 1 : y - 1, yp = y == a.ny - 1 ? 0 : y + 1;
-#pragma unroll
-        for (int i = 0; i < 19; i++) {
-            const int xs = cx(i) > 0 ? xm : (cx(i) < 0 ? xp : x), ys = cy(i) > 0 ? ym : (cy(i) < 0 ? yp : y);
-            const int zs = z - cz(i) + (cz(i) > 0 ? zlo : 0) - (cz(i) < 0 ? zhi : 0);
-            g[i] = ld((const T *)a.A + i * a.Np + (xs + a.nx * ys) * a.zp + zs);
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < 19; i++)
-            g[i] = ld((const T *)a.Ap[i] + (e + (cz(i) > 0 ? zlo : 0) - (cz(i) < 0 ? zhi : 0)));
-    }
+    column_pull<T, WRAP>(g, a.p, col.x, z, ld);
     if (col.y >= 0) {  // uniform over the warp
         // the populations that come back from the wall (linear interpolated
         // bounce-back, or the single-node scheme): f_ibar(x_f, t+1) =
@@ -147,8 +127,8 @@ __global__ void __launch_bounds__(256, column_min_blocks(S, SRT)) sweep_columns(
     }
 #pragma unroll
     for (int i = 0; i < 19; i++) {
-        if constexpr (scaled) Store<LBM_F16S>::st_scaled((T *)a.Bp[i] + e, g[i]);
-        else Store<S>::st((T *)a.Bp[i] + e, g[i]);
+        if constexpr (scaled) Store<LBM_F16S>::st_scaled((T *)a.p.Bp[i] + e, g[i]);
+        else Store<S>::st((T *)a.p.Bp[i] + e, g[i]);
     }
 }
 
@@ -156,31 +136,20 @@ template <int S, bool FORCE, bool SRT>
 static cudaError_t launch_columns_t(Ctx &c) {
     ColumnArgs a{};
     a.A = c.fA;
-    a.B = c.fB;
     a.cols = c.col_list;
     a.wall = c.col_wall;
     a.coef = c.col_coef;
     a.ncols = (unsigned)c.ncols;
     a.nchunk = (unsigned)((c.nz + 31) / 32);
     a.fd_chunk = FastDiv(a.nchunk);
-    a.fd_nx = FastDiv((unsigned)c.nx);
-    a.nx = c.nx;
-    a.ny = c.ny;
-    a.nz = c.nz;
-    a.zp = c.zp;
+    column_ptrs(c, a.p);
     a.Np = c.Np;
     a.status = c.d_status;
     a.pk = make_pair_k(c.rt.d_nu, c.F);
     a.rt = c.rt;
-    const size_t sb = storage_bytes(c.storage);
     for (int d = 0; d < 3; d++) {
         a.F[d] = c.F[d];
         a.Fs[d] = (float)c.F[d];
-    }
-    for (int i = 0; i < 19; i++) {
-        const long long off = cz(i) + (long long)c.zp * (cx(i) + (long long)c.nx * cy(i));
-        a.Ap[i] = (const void *)((const char *)c.fA + (long long)sb * (i * c.Np - off));
-        a.Bp[i] = (void *)((char *)c.fB + (long long)sb * (i * c.Np));
     }
     const unsigned nb = (unsigned)(((long long)a.ncols * a.nchunk + 7) / 8);
     count_launch(c, G_BULK);
