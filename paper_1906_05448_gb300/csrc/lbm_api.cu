@@ -8,8 +8,13 @@
 #include <cstdio>
 #include <cstring>
 #include <algorithm>
+#include <thread>
 #include <utility>
 #include <vector>
+
+#include <sched.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 namespace lbmgb {
 size_t stats_partials_doubles();
@@ -239,7 +244,10 @@ cudaError_t plane_copy(Ctx &c, int i, bool to_f64) {
 }
 
 // Check the status word copied by the last asynchronous check (bounded
-// host wait: polls the event, gives up after the context's wait limit).
+// host wait: polls the event, gives up after the context's wait limit). The
+// first millisecond polls without sleeping: a read-back usually waits for a
+// few microseconds of work, and sleeping a millisecond per poll cost a small
+// step-and-read loop a third of its time.
 lbm_status check_status(Ctx &c, bool wait) {
     if (!c.status_pending) return LBM_OK;
     const double timeout_s = c.wait_limit_s;
@@ -247,12 +255,21 @@ lbm_status check_status(Ctx &c, bool wait) {
     if (q == cudaErrorNotReady) {
         if (!wait) return LBM_OK;
         // bounded wait
-        const long long sleeps = (long long)(timeout_s * 1000.0);
-        for (long long k = 0; k < sleeps; k++) {
+        auto now = []() {
+            struct timespec t;
+            clock_gettime(CLOCK_MONOTONIC, &t);
+            return (double)t.tv_sec + 1e-9 * (double)t.tv_nsec;
+        };
+        const double t0 = now();
+        for (double t = t0; t - t0 < timeout_s; t = now()) {
             q = cudaEventQuery(c.ev_status);
             if (q != cudaErrorNotReady) break;
-            struct timespec ts = {0, 1000000};
-            nanosleep(&ts, nullptr);
+            if (t - t0 < 1e-3) {
+                sched_yield();
+            } else {
+                struct timespec ts = {0, 50000};
+                nanosleep(&ts, nullptr);
+            }
         }
         if (q == cudaErrorNotReady) return fail(c, LBM_ETIMEOUT, "stream did not finish within %g s", timeout_s);
     }
@@ -279,14 +296,58 @@ lbm_status enqueue_status(Ctx &c) {
     return LBM_OK;
 }
 
-lbm_status sync_all(Ctx &c) {
+// Populate the pages of a caller's destination that was never touched (a
+// fresh array): the copy engine's own faults cost 10.6 ms for 307 MB against
+// 1.6 ms for the copy into present pages. Contents are not changed. Runs
+// while the steps ahead of a read-back are still on the GPU; several
+// threads, for a call that finds it idle (10.1 ms with one, 3.2 with four,
+// 2.7 with eight).
+void populate(void *dst, size_t bytes) noexcept {
+#ifdef MADV_POPULATE_WRITE
+    if (bytes < ((size_t)4 << 20)) return;
+    const long ps = sysconf(_SC_PAGESIZE);
+    if (ps <= 0) return;
+    const uintptr_t page = (uintptr_t)ps, a = ((uintptr_t)dst + page - 1) / page * page,
+                    b = ((uintptr_t)dst + bytes) / page * page;
+    if (b <= a) return;
+    const unsigned hw = std::thread::hardware_concurrency();
+    const int T = hw >= 16 ? 8 : (hw >= 4 ? (int)hw / 2 : 1);
+    const uintptr_t per = ((b - a) / T / page + 1) * page;
+    std::thread th[8];
+    for (int k = 0; k < T; k++) {
+        const uintptr_t lo = a + k * per, hi = std::min(b, lo + per);
+        if (lo >= hi) break;
+        // errors are ignored: the copy then faults the pages itself
+        auto work = [lo, hi]() { (void)madvise((void *)lo, hi - lo, MADV_POPULATE_WRITE); };
+        if (k == T - 1 || hi == b) {
+            work();
+            break;
+        }
+        try {
+            th[k] = std::thread(work);
+        } catch (...) {
+            work();
+        }
+    }
+    for (auto &t : th)
+        if (t.joinable()) t.join();
+#else
+    (void)dst;
+    (void)bytes;
+#endif
+}
+
+// Wait for the enqueued work and its status word; dst: the caller's
+// destination of a read-back that follows
+lbm_status sync_all(Ctx &c, void *dst = nullptr, size_t bytes = 0) {
+    CK(cudaMemcpyAsync(c.h_status + 2, c.d_counts, 2 * sizeof(long long), cudaMemcpyDeviceToHost, c.stream));
     lbm_status s = enqueue_status(c);
     if (s != LBM_OK) return s;
+    if (dst) populate(dst, bytes);
     s = check_status(c, true);
     if (s != LBM_OK) return s;
     long long cnt[2];
-    CK(cudaMemcpyAsync(cnt, c.d_counts, sizeof(cnt), cudaMemcpyDeviceToHost, c.stream));
-    CK(cudaStreamSynchronize(c.stream));
+    memcpy(cnt, c.h_status + 2, sizeof(cnt));
     c.nsites = cnt[0];
     c.nlinks = cnt[1];
     return LBM_OK;
@@ -749,7 +810,7 @@ lbm_status lbm_create(const lbm_grid *grid, double tau, const double force[3], v
         return LBM_ECUDA;
     };
     cudaError_t e;
-    if ((e = cudaMallocHost((void **)&c.h_status, sizeof(unsigned))) != cudaSuccess) {
+    if ((e = cudaMallocHost((void **)&c.h_status, 64)) != cudaSuccess) {
         c.h_status = nullptr;
         return bad(e, "cudaMallocHost");
     }
@@ -1056,13 +1117,21 @@ lbm_status lbm_tke_budget(lbm_ctx *h, int flags, int nbins, double *out) {
 lbm_status lbm_get_field(lbm_ctx *h, int which, void *dst, size_t bytes) {
     CTX_CHECK(h);
     if (!dst) return fail(c, LBM_EINVAL, "null destination");
-    lbm_status s = sync_all(c);
-    if (s != LBM_OK && s != LBM_EUNSTABLE) return s;
     const size_t N = (size_t)c.N;
+    size_t need = 0;  // what the field fills of dst
+    switch (which) {
+    case LBM_FIELD_RHO: need = N * sizeof(double); break;
+    case LBM_FIELD_U:
+    case LBM_FIELD_IBM_FORCE: need = 3 * N * sizeof(double); break;
+    case LBM_FIELD_POPS: need = (size_t)c.q * N * sizeof(double); break;
+    case LBM_FIELD_FLAGS: need = N; break;
+    default: break;
+    }
+    lbm_status s = sync_all(c, dst, std::min(need, bytes));
+    if (s != LBM_OK && s != LBM_EUNSTABLE) return s;
     switch (which) {
     case LBM_FIELD_RHO:
     case LBM_FIELD_U: {
-        const size_t need = (which == LBM_FIELD_RHO ? 1 : 3) * N * sizeof(double);
         if (bytes < need) return fail(c, LBM_EINVAL, "destination too small");
         CK(launch_macro(c, 0));
         CK(cudaMemcpyAsync(dst, which == LBM_FIELD_RHO ? (void *)c.rho_f : (void *)c.u_f, need,

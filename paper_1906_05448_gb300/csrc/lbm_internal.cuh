@@ -101,7 +101,7 @@ struct Ctx {
     unsigned long long *near_key;  // nearest particle surface per cell (diag.cu)
     // status
     unsigned *d_status;
-    unsigned *h_status;
+    unsigned *h_status;  // pinned: [0] status word, [2..5] d_counts[0..1]
     cudaEvent_t ev_status;
     bool status_pending;
     double wait_limit_s;  // bound of the host waits on the stream (lbm_set_wait_limit)
