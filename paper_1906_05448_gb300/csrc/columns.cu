@@ -11,7 +11,7 @@ template <typename T, bool TOX>
 __global__ void __launch_bounds__(256) convert_kernel(const void *src, void *dst, int q, int nx, int ny, int nz, int zp,
                                                       long long N, long long Np, const uint8_t *solid) {
     __shared__ T sh[COL_TILE][COL_TILE + 1];
-    for (int y = blockIdx.z; y < ny; y += gridDim.z)
+    for (int y = blockIdx.y; y < ny; y += gridDim.y)
     for (int i = 0; i < q; i++) {
         const T *s = (const T *)src + i * (TOX ? Np : N);
         T *d = (T *)dst + i * (TOX ? N : Np);
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256) plane_kernel(void *plane, double *v, doub
     typedef typename Store<S>::R R;
     __shared__ double sh[COL_TILE][COL_TILE + 1];
     T *p = (T *)plane;
-    for (int y = blockIdx.z; y < ny; y += gridDim.z) {
+    for (int y = blockIdx.y; y < ny; y += gridDim.y) {
     auto at_x = [&](int x, int z) { return x + (long long)nx * (y + (long long)ny * z); };
     auto at_z = [&](int x, int z) { return z + (long long)zp * (x + (long long)nx * y); };
     column_exchange<double, TOX>(
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const 
         R rho, ux, uy, uz;
     };
     __shared__ V sh[COL_TILE][COL_TILE + 1];
-    for (int y = blockIdx.z; y < ny; y += gridDim.z)
+    for (int y = blockIdx.y; y < ny; y += gridDim.y)
     column_exchange<V, true>(
         sh, nx, nz,
         [&](int x, int z) {

@@ -67,10 +67,11 @@ __device__ __forceinline__ void column_pull(R g[19], const ColumnPtrs &p, int co
 
 constexpr int COL_TILE = 32;  // x by z tile of the conversions, at one y
 
-// blocks per (z tile, x tile, y; y strided beyond the grid limit)
+// blocks: z tiles x x tiles (linear in x, so that no grid limit is met), y
+// strided beyond the limit
 inline dim3 column_tiles(const Ctx &c) {
-    return dim3((unsigned)((c.nz + COL_TILE - 1) / COL_TILE), (unsigned)((c.nx + COL_TILE - 1) / COL_TILE),
-                (unsigned)(c.ny < 65535 ? c.ny : 65535));
+    const long long t = (long long)((c.nz + COL_TILE - 1) / COL_TILE) * ((c.nx + COL_TILE - 1) / COL_TILE);
+    return dim3((unsigned)t, (unsigned)(c.ny < 65535 ? c.ny : 65535));
 }
 
 // body(x, z, value) for the cells of a block's tile in z-fast order, then in
@@ -79,7 +80,8 @@ inline dim3 column_tiles(const Ctx &c) {
 // shared memory (one pad word per row: no bank conflicts for 4-byte V)
 template <typename V, bool TOX, typename Put, typename Get>
 __device__ __forceinline__ void column_exchange(V (*sh)[COL_TILE + 1], int nx, int nz, Put put, Get get) {
-    const int z0 = blockIdx.x * COL_TILE, x0 = blockIdx.y * COL_TILE;
+    const unsigned nzt = (unsigned)((nz + COL_TILE - 1) / COL_TILE);
+    const int z0 = (int)(blockIdx.x % nzt) * COL_TILE, x0 = (int)(blockIdx.x / nzt) * COL_TILE;
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5, rows = blockDim.x >> 5;
     for (int r = row; r < COL_TILE; r += rows) {
         const int x = x0 + (TOX ? r : lane), z = z0 + (TOX ? lane : r);
@@ -94,6 +96,37 @@ __device__ __forceinline__ void column_exchange(V (*sh)[COL_TILE + 1], int nx, i
         if (x < nx && z < nz) get(x, z, TOX ? sh[r][lane] : sh[lane][r]);
     }
     __syncthreads();  // the tile is free for the next exchange
+}
+
+// Statistics of the pipe's columns: cylindrical basis and radial bin
+// b = floor(r nbins / R) of a column, formed with explicitly rounded
+// operations so that a cell on a bin edge falls in the same bin everywhere.
+struct PipeColumn {
+    double r, ca, sa;  // e_r = (ca, sa, 0), e_theta = (-sa, ca, 0); on the axis (1, 0)
+    int bin;
+};
+// false outside the pipe or beyond the last bin
+__device__ __forceinline__ bool pipe_column(const uint8_t *flags, int x, int y, int nx, int ny, double pcx, double pcy,
+                                            double R, int nbins, PipeColumn &k) {
+    if (x >= nx || y >= ny || (flags[x + nx * y] & FL_SOLID)) return false;
+    const double dx = __dsub_rn((double)x, pcx), dy = __dsub_rn((double)y, pcy);
+    k.r = sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+    k.bin = (int)floor(__ddiv_rn(__dmul_rn(k.r, (double)nbins), R));
+    if (k.bin < 0 || k.bin >= nbins) return false;
+    k.ca = k.r > 0.0 ? dx / k.r : 1.0;
+    k.sa = k.r > 0.0 ? dy / k.r : 0.0;
+    return true;
+}
+// 32 x 8 columns per block, numbered linearly over the section; y: runs of z
+constexpr int COL_RUN = 32;  // planes per thread (more where the grid limit asks for it)
+inline int column_run(int nz) { return nz / 65535 >= COL_RUN ? nz / 65535 + 1 : COL_RUN; }
+inline dim3 column_blocks(int nx, int ny, int nz, int run) {
+    return dim3((unsigned)(((nx + 31) / 32) * (long long)((ny + 7) / 8)), (unsigned)((nz + run - 1) / run));
+}
+__device__ __forceinline__ void column_of_thread(int nx, int &x, int &y) {
+    const unsigned nxt = (unsigned)((nx + 31) / 32);
+    x = (int)(blockIdx.x % nxt) * 32 + (int)(threadIdx.x & 31);
+    y = (int)(blockIdx.x / nxt) * 8 + (int)(threadIdx.x >> 5);
 }
 
 }  // namespace lbmgb

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256, ibm_column_min_blocks(S)) ibm_columns_col
 // first and the last those of the halo planes, and the z factor combines
 // three neighbours through shared memory.
 struct IbmPassArgs {
-    int nz, pass;
+    int nz, pass, nc, sp;  // a launch: nc markers or sp columns for each run of planes in turn
     // markers: 16 (support column, x-y weight) entries each
     const int *it_k;
     const void *it_w;
@@ -159,8 +159,8 @@ __device__ __forceinline__ int pass_plane(int z0, int nz) {
 template <typename R>
 __global__ void __launch_bounds__(256) ibm_columns_interp(IbmPassArgs a) {
     __shared__ R P[4][256];
-    const int j = blockIdx.x, t = threadIdx.x;
-    const int z0 = blockIdx.y * (blockDim.x - 2), z = pass_plane(z0, a.nz);
+    const int j = (int)(blockIdx.x % (unsigned)a.nc), t = threadIdx.x;
+    const int z0 = (int)(blockIdx.x / (unsigned)a.nc) * (int)(blockDim.x - 2), z = pass_plane(z0, a.nz);
     const R *tw = (const R *)a.it_w + 16 * (size_t)j;
     const int *tk = a.it_k + 16 * (size_t)j;
     const R *ru = (const R *)a.ru + 4 * (size_t)z;
@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(256) ibm_columns_interp(IbmPassArgs a) {
 template <typename R>
 __global__ void __launch_bounds__(256) ibm_columns_spread(IbmPassArgs a) {
     __shared__ R Q[3][256];
-    const int k = blockIdx.x, t = threadIdx.x;
-    const int z0 = blockIdx.y * (blockDim.x - 2), z = pass_plane(z0, a.nz);
+    const int k = (int)(blockIdx.x % (unsigned)a.sp), t = threadIdx.x;
+    const int z0 = (int)(blockIdx.x / (unsigned)a.sp) * (int)(blockDim.x - 2), z = pass_plane(z0, a.nz);
     const int xy = __ldg(a.sites + k);
     const int e0 = __ldg(a.xy_start + xy), e1 = __ldg(a.xy_start + xy + 1);
     const R *xw = (const R *)a.xy_w, *mF = (const R *)a.mF + z;
@@ -264,7 +264,7 @@ static cudaError_t collide_t(Ctx &c) {
 
 template <typename R>
 static cudaError_t passes_t(Ctx &c) {
-    IbmPassArgs a{c.nz, 0, c.pipe_it_k, c.pipe_it_w, c.mFr, c.mFaccR, (long long)c.pipe_nc * c.nz, c.pipe_dV,
+    IbmPassArgs a{c.nz, 0, c.pipe_nc, c.pipe_sp, c.pipe_it_k, c.pipe_it_w, c.mFr, c.mFaccR, (long long)c.pipe_nc * c.nz, c.pipe_dV,
                   c.site_cell, c.pipe_xy_start, c.pipe_xy_j, c.pipe_xy_w, c.sup_ru, c.sup_F, (long long)c.pipe_sp * c.nz};
     // equal runs of at most 254 planes, whole warps with the two halo threads
     const int tiles = (c.nz + 253) / 254, run = (c.nz + tiles - 1) / tiles;
@@ -273,8 +273,8 @@ static cudaError_t passes_t(Ctx &c) {
     for (int pass = 0; pass < 3; pass++) {
         a.pass = pass;
         count_launch(c, G_IBM, 2);
-        ibm_columns_interp<R><<<dim3((unsigned)c.pipe_nc, ty), tb, 0, c.stream>>>(a);
-        ibm_columns_spread<R><<<dim3((unsigned)c.pipe_sp, ty), tb, 0, c.stream>>>(a);
+        ibm_columns_interp<R><<<(unsigned)c.pipe_nc * ty, tb, 0, c.stream>>>(a);
+        ibm_columns_spread<R><<<(unsigned)c.pipe_sp * ty, tb, 0, c.stream>>>(a);
     }
     c.markers_stale = 1;
     return cudaGetLastError();

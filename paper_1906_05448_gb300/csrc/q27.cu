@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(256) q27_column_macro_kernel(const void *A, do
         R rho, ux, uy, uz;
     };
     __shared__ V sh[COL_TILE][COL_TILE + 1];
-    for (int y = blockIdx.z; y < ny; y += gridDim.z)
+    for (int y = blockIdx.y; y < ny; y += gridDim.y)
         column_exchange<V, true>(
             sh, nx, nz,
             [&](int x, int z) {

@@ -107,3 +107,29 @@ def test_d3q27_plane_counts(lbm, nx, ny, R, nz):
     ro, uo = q27.macro(o, F)
     assert rel(ug[:, fl], uo.reshape(3, -1)[:, fl]) < 1e-12 and rel(rg[fl], ro.reshape(-1)[fl]) < 1e-12
     g.close()
+
+
+@pytest.mark.parametrize("nx,ny,nz,R,nbins", [
+    (27, 26, 33, 11.7, 1), (27, 26, 33, 11.7, 7), (27, 26, 33, 11.7, 60), (25, 25, 4, 11.2, 1),
+    (25, 25, 4, 11.2, 7), (40, 33, 64, 15.9, 60),  # small sections refuse more bins (LBM_ENOMEM)
+])
+def test_pipe_statistics_of_a_snapshot(lbm, nx, ny, nz, R, nbins):
+    """Profiles and budget of the library's own fields against their numpy
+    statements: odd sections (a column on the axis: in the profiles, not in
+    the budget), runs of planes with a remainder, one bin to more bins than
+    columns along the radius. Bars of the full-field tests of each."""
+    from oracle import profiles, tke_budget as tb
+    g, _ = pair(lbm, nx, ny, nz, R, "f64", oracle.RATES_SRT)
+    g.step(5, lbm.BC_IBB)
+    rho, u = g.macro()
+    solid = g.flags() & 1
+    args = (u, rho, solid, nx, ny, nz, 0.5 * (nx - 1), 0.5 * (ny - 1), R, 0.07 / 3, nbins)
+    for got, ref, tol in ((g.pipe_profiles(nbins), profiles.pipe_profiles(*args), 1e-10),
+                          (g.tke_budget(nbins), tb.tke_budget(*args), 1e-7)):
+        assert np.array_equal(got[:, 0], ref[:, 0])
+        for k in range(1, ref.shape[1]):
+            scale = max(np.max(np.abs(ref[:, k])), 1e-300)
+            if k in (1, 2) and ref.shape[1] == 12:  # u_r, u_theta: means that nearly vanish, on the velocity's scale
+                scale = np.max(np.abs(u))
+            assert np.max(np.abs(got[:, k] - ref[:, k])) <= tol * scale, k
+    g.close()
