@@ -476,6 +476,31 @@ __device__ __noinline__ typename Store<S>::R single_node_pair(const typename Sto
     return R(2) * ev;
 }
 
+// ------------------------------------------------- unevaluated FP32 sums ----
+// A number as hi + lo of two floats (about 48 bits): sums and squares of FP32
+// data nearly as exact as in FP64, on the pipe that is 64 times as wide.
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {  // two-sum of the leading parts (Knuth)
+    const float s = a.x + b.x, t = s - a.x;
+    return make_float2(s, ((a.x - (s - t)) + (b.x - t)) + (a.y + b.y));
+}
+__device__ __forceinline__ float2 pair_diff(float a, float b) {  // a - b, exact
+    const float s = a - b, t = s - a;
+    return make_float2(s, (a - (s - t)) - (b + t));
+}
+__device__ __forceinline__ float2 pair_mul(float a, float b) {  // a b, exact
+    const float p = __fmul_rn(a, b);
+    return make_float2(p, fmaf(a, b, -p));
+}
+__device__ __forceinline__ float2 pair_square(float2 a) {
+    const float p = __fmul_rn(a.x, a.x);
+    return make_float2(p, fmaf(a.x + a.x, a.y, fmaf(a.x, a.x, -p)));
+}
+__device__ __forceinline__ float2 pair_of(double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+}
+__device__ __forceinline__ double pair_value(float2 a) { return (double)a.x + (double)a.y; }
+
 // ------------------------------------------------------------- helpers ----
 // body force component in the arithmetic type R
 template <typename R, typename Args>

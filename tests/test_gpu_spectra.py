@@ -89,3 +89,20 @@ def test_non_cube_is_rejected(lbm):
     with pytest.raises(lbm.LbmError):
         g.spectrum(8)
     g.close()
+
+
+@pytest.mark.parametrize("n", [8, 16, 32, 128, 256])
+def test_every_transform_length_on_noise(lbm, n):
+    """White noise fills every shell: the last pass of the transform is of
+    radix 8, 2 or 4 in turn, the smallest cubes take fewer lines per block;
+    the bars of the other spectra tests."""
+    u = workloads.noise_velocity((n, n, n), 0.02, seed=n)
+    g = lbm.Lattice(n, n, n, 0.6, storage=lbm.F32)
+    g.init_velocity(u)
+    nb = 7 if n == 8 else n  # 8^3: the scratch limit
+    Eg, Dg = g.spectrum(nb)
+    Eo, Do = spectra.spectra(u, n, 0.1 / 3, nb)
+    okE, eE = close(Eg, Eo)
+    okD, eD = close(Dg, Do)
+    assert okE and okD, (eE, eD)
+    g.close()
