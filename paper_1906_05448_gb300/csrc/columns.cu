@@ -86,7 +86,7 @@ cudaError_t column_plane_copy(Ctx &c, int i, double w, bool to_f64) {
 // force planes sF of the support columns.
 template <int S>
 __global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const uint8_t *flags, const int *info,
-                                                           const void *sFv, long long SF, double *rho_o, double *u_o,
+                                                           const void *sFv, long long SF, float4 *rec, double *rho_o, double *u_o,
                                                            int nx, int ny, int nz, int zp, long long N, long long Np,
                                                            double F0, double F1, double F2) {
     typedef typename Store<S>::T T;
@@ -125,6 +125,10 @@ __global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const 
         },
         [&](int x, int z, const V &v) {
             const long long c = x + (long long)nx * (y + (long long)ny * z);
+            if (rec) {
+                rec[c] = make_float4(float(v.ux), float(v.uy), float(v.uz), float(v.rho));
+                return;
+            }
             rho_o[c] = double(v.rho);
             u_o[c] = double(v.ux);
             u_o[N + c] = double(v.uy);
@@ -132,12 +136,12 @@ __global__ void __launch_bounds__(256) column_macro_kernel(const void *A, const 
         });
 }
 
-cudaError_t launch_column_macro(Ctx &c) {
+cudaError_t launch_column_macro(Ctx &c, float4 *rec) {
     count_launch(c, G_STATS);
     const int *info = c.armed_bc == LBM_BC_IBB ? nullptr : c.col_ibm;
     const long long SF = (long long)c.pipe_sp * c.nz;
     switch (c.storage) {
-#define MK(S) column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, c.flags, info, c.sup_F, SF, c.rho_f, c.u_f, c.nx, c.ny, \
+#define MK(S) column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, c.flags, info, c.sup_F, SF, rec, c.rho_f, c.u_f, c.nx, c.ny, \
                                                                            c.nz, c.zp, c.N, c.Np, c.F[0], c.F[1], c.F[2])
     case LBM_F64: MK(LBM_F64); break;
     case LBM_F32: MK(LBM_F32); break;

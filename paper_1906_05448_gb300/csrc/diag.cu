@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 namespace lbmgb {
@@ -23,19 +24,22 @@ __device__ __forceinline__ int dwrap(int a, int n) {
 
 // rho and u of the post-collision state: sum f c = rho u + F/2 after a Guo
 // collision with total force F (body force on fluid cells + IBM force).
-// u32, if not null, receives an FP32 copy of u, one 16-byte record (ux, uy,
-// uz, 0) per cell (the closure's gather input).
+// u32, if not null, receives FP32 records (ux, uy, uz, rho), 16 bytes per
+// cell (the closure's gather input, the statistics of 32- and 16-bit
+// storage), alone with rec_only.
 template <int S>
 __global__ void macro_kernel(const void *A, const uint8_t *flags, const int *aux, const void *sup_Fv, double *rho_o,
                              double *u_o, float *u32, long long N, double F0, double F1, double F2, int ibb, int ibm,
-                             long long max_sites) {
+                             long long max_sites, int rec_only) {
     typedef typename Store<S>::T T;
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     const uint8_t fl = flags[c];
     if (ibb && (fl & FL_SOLID)) {
-        rho_o[c] = 0.0;
-        u_o[c] = u_o[N + c] = u_o[2 * N + c] = 0.0;
+        if (!rec_only) {
+            rho_o[c] = 0.0;
+            u_o[c] = u_o[N + c] = u_o[2 * N + c] = 0.0;
+        }
         if (u32) reinterpret_cast<float4 *>(u32)[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
     }
@@ -62,26 +66,25 @@ __global__ void macro_kernel(const void *A, const uint8_t *flags, const int *aux
     }
     const R rho = R(1) + r;
     const R ir = R(1) / rho;
-    rho_o[c] = double(rho);
     const R ux = (j0 - R(0.5) * Fx) * ir, uy = (j1 - R(0.5) * Fy) * ir, uz = (j2 - R(0.5) * Fz) * ir;
+    if (u32) reinterpret_cast<float4 *>(u32)[c] = make_float4(float(ux), float(uy), float(uz), float(rho));
+    if (rec_only) return;
+    rho_o[c] = double(rho);
     u_o[c] = double(ux);
     u_o[N + c] = double(uy);
     u_o[2 * N + c] = double(uz);
-    if (u32) {
-        reinterpret_cast<float4 *>(u32)[c] = make_float4(float(ux), float(uy), float(uz), 0.f);
-    }
 }
 
-cudaError_t launch_macro(Ctx &c, int /*mask_mode*/, float *u32) {
-    if (c.q == 27) return launch_q27_macro(c);
-    if (c.zlay) return launch_column_macro(c);
+cudaError_t launch_macro(Ctx &c, int /*mask_mode*/, float *u32, bool rec_only) {
+    if (c.q == 27) return launch_q27_macro(c, rec_only ? (float4 *)u32 : nullptr);
+    if (c.zlay) return launch_column_macro(c, rec_only ? (float4 *)u32 : nullptr);
     count_launch(c, G_STATS);
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     const int ibb = c.armed_bc == LBM_BC_IBB;
     const int ibm = c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B;
     switch (c.storage) {
 #define MK(S) macro_kernel<S><<<nb, 256, 0, c.stream>>>(c.fA, c.flags, c.aux, c.sup_F, c.rho_f, c.u_f, u32, c.N, c.F[0], \
-                                                           c.F[1], c.F[2], ibb, ibm, c.max_sites)
+                                                           c.F[1], c.F[2], ibb, ibm, c.max_sites, rec_only)
     case LBM_F64: MK(LBM_F64); break;
     case LBM_F32: MK(LBM_F32); break;
     case LBM_F16S: MK(LBM_F16S); break;
@@ -92,106 +95,135 @@ cudaError_t launch_macro(Ctx &c, int /*mask_mode*/, float *u32) {
 }
 
 constexpr int SB = 256;     // threads per statistics block
-constexpr int SNB = 1024;   // statistics blocks (fixed: the reduction order does not depend on the grid)
-constexpr int NP = 16;      // partial sums per block
+constexpr int SNB = 1024;   // statistics blocks at most (the partial sums of each are kept)
+constexpr int NP = 16;      // sums per block
+constexpr int NBIN = LBM_NBINS;
+// sums of a block: over the cells that carry fluid in the statistics (mass,
+// momentum), over fluid and over solid cells (u.u and dissipation), fluid
+// cells, u_z of fluid cells; mass and momentum of masked solid cells
+enum { ST_MASS, ST_MX, ST_MY, ST_MZ, ST_KF, ST_EF, ST_KS, ST_ES, ST_NF, ST_UZ, ST_SMASS, ST_SX, ST_SY, ST_SZ };
 
-template <int NV>
-__device__ void sblock_sum(double v[NV], double *sh) {
-    for (int k = 0; k < NV; k++) sh[k * SB + threadIdx.x] = v[k];
+// fixed-order block sum of NV values per thread, results in v of thread 0
+template <int NV, int TB>
+__device__ void sblock_sum(double v[NV], double *sh /* NV * TB / 32 */) {
+#pragma unroll
+    for (int k = 0; k < NV; k++)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if ((threadIdx.x & 31) == 0)
+        for (int k = 0; k < NV; k++) sh[k * (TB / 32) + (threadIdx.x >> 5)] = v[k];
     __syncthreads();
-    for (int s = SB / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-            for (int k = 0; k < NV; k++) sh[k * SB + threadIdx.x] += sh[k * SB + threadIdx.x + s];
-        __syncthreads();
-    }
-    for (int k = 0; k < NV; k++) v[k] = sh[k * SB];
-}
-
-// partials: mass, momentum (3) over fluid-carrying cells
-__global__ void __launch_bounds__(SB) mass_kernel(const double *rho, const double *u, const uint8_t *flags, long long N,
-                                                  int ibb, double *part) {
-    __shared__ double sh[4 * SB];
-    double v[4] = {0, 0, 0, 0};
-    for (long long c = (long long)blockIdx.x * SB + threadIdx.x; c < N; c += (long long)SNB * SB) {
-        if (ibb && (flags[c] & FL_SOLID)) continue;
-        v[0] += rho[c];
-        v[1] += rho[c] * u[c];
-        v[2] += rho[c] * u[N + c];
-        v[3] += rho[c] * u[2 * N + c];
-    }
-    sblock_sum<4>(v, sh);
     if (threadIdx.x == 0)
-        for (int k = 0; k < 4; k++) part[blockIdx.x * NP + k] = v[k];
-}
-
-// replace the velocity of solid cells by the rigid-body velocity
-__global__ void mask_kernel(double *u, const uint8_t *flags, const int *owner, const double *X, const double *U,
-                            const double *W, int nx, int ny, int nz, long long N) {
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    if (!(flags[c] & FL_SOLID)) return;
-    const int p = owner[c];
-    double uw[3] = {0, 0, 0};
-    if (p != NO_OWNER) {
-        const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-        const double r0 = dmimg(x - X[3 * p], nx), r1 = dmimg(y - X[3 * p + 1], ny), r2 = dmimg(z - X[3 * p + 2], nz);
-        uw[0] = U[3 * p] + (W[3 * p + 1] * r2 - W[3 * p + 2] * r1);
-        uw[1] = U[3 * p + 1] + (W[3 * p + 2] * r0 - W[3 * p] * r2);
-        uw[2] = U[3 * p + 2] + (W[3 * p] * r1 - W[3 * p + 1] * r0);
-    }
-    u[c] = uw[0];
-    u[N + c] = uw[1];
-    u[2 * N + c] = uw[2];
-}
-
-__device__ __forceinline__ double cell_eps(const double *u, int x, int y, int z, int nx, int ny, int nz, long long N,
-                                           double nu) {
-    const long long xp = dwrap(x + 1, nx) + (long long)nx * (y + (long long)ny * z);
-    const long long xm = dwrap(x - 1, nx) + (long long)nx * (y + (long long)ny * z);
-    const long long yp = x + (long long)nx * (dwrap(y + 1, ny) + (long long)ny * z);
-    const long long ym = x + (long long)nx * (dwrap(y - 1, ny) + (long long)ny * z);
-    const long long zp = x + (long long)nx * (y + (long long)ny * dwrap(z + 1, nz));
-    const long long zm = x + (long long)nx * (y + (long long)ny * dwrap(z - 1, nz));
-    double g[3][3];
-    for (int a = 0; a < 3; a++) {
-        const double *ua = u + a * N;
-        g[a][0] = 0.5 * (ua[xp] - ua[xm]);
-        g[a][1] = 0.5 * (ua[yp] - ua[ym]);
-        g[a][2] = 0.5 * (ua[zp] - ua[zm]);
-    }
-    double ss = 0.0;
-    for (int a = 0; a < 3; a++)
-        for (int b = 0; b < 3; b++) {
-            const double s = 0.5 * (g[a][b] + g[b][a]);
-            ss += s * s;
+        for (int k = 0; k < NV; k++) {
+            v[k] = 0.0;
+            for (int w = 0; w < TB / 32; w++) v[k] += sh[k * (TB / 32) + w];
         }
-    return 2.0 * nu * ss;
 }
 
-// partials: ke, eps over all cells; ke, eps, count over fluid cells; pipe bulk
-__global__ void __launch_bounds__(SB) energy_kernel(const double *u, const uint8_t *flags, int nx, int ny, int nz,
-                                                    long long N, double nu, int pipe, double *part, const float *eps_o) {
-    __shared__ double sh[7 * SB];
-    double v[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (long long c = (long long)blockIdx.x * SB + threadIdx.x; c < N; c += (long long)SNB * SB) {
-        const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-        const double e = (eps_o && eps_o[c] >= 0.f) ? (double)eps_o[c] : cell_eps(u, x, y, z, nx, ny, nz, N, nu);
-        const double k = 0.5 * (u[c] * u[c] + u[N + c] * u[N + c] + u[2 * N + c] * u[2 * N + c]);
-        v[0] += k;
-        v[1] += e;
-        if (!(flags[c] & FL_SOLID)) {
-            v[2] += k;
-            v[3] += e;
-            v[4] += 1.0;
-            if (pipe) {
-                v[5] += u[2 * N + c];
-                v[6] += 1.0;
+// Replace the velocity of solid cells by the rigid-body velocity (zero
+// without an owner: outside the pipe). A block takes runs of 4096 cells, 16
+// flags per thread, lists the solid ones and spreads them over its threads.
+// part (statistics only): the mass and momentum that the solid cells held.
+// REC: the field is FP32 records; cells without an owner become zero there,
+// cells of a particle get their velocity as hi + lo of two floats (the
+// rigid-body velocity is FP64): hi in the record, whose density then says
+// so, lo in a record of its own at u.
+constexpr int MASK_RUN = SB * 16;
+constexpr float MASKED = -3.402823466e38f;  // no density
+template <bool REC>
+__global__ void __launch_bounds__(SB) mask_kernel(float4 *rec, double *u, const double *rho, const uint8_t *flags,
+                                                  const int *owner, const double *X, const double *U, const double *W,
+                                                  int nx, int ny, int nz, FastDiv fdx, FastDiv fdxy, long long N,
+                                                  double *part) {
+    __shared__ unsigned short list[MASK_RUN];
+    __shared__ int wsum[SB / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v[4] = {0, 0, 0, 0};
+    for (long long c0 = (long long)blockIdx.x * MASK_RUN; c0 < N; c0 += (long long)gridDim.x * MASK_RUN) {
+        const long long b = c0 + 16 * threadIdx.x;
+        unsigned w[4] = {0u, 0u, 0u, 0u};
+        if (b + 16 <= N) {
+            const uint4 q = *(const uint4 *)(flags + b);
+            w[0] = q.x;
+            w[1] = q.y;
+            w[2] = q.z;
+            w[3] = q.w;
+        } else {
+            for (int k = 0; k < 16 && b + k < N; k++) w[k >> 2] |= (unsigned)flags[b + k] << (8 * (k & 3));
+        }
+        int n = 0;
+        for (int k = 0; k < 4; k++) {
+            w[k] &= 0x01010101u * FL_SOLID;
+            n += __popc(w[k]);
+        }
+        // positions in cell order: scan over the warp, then over the warps
+        int inc = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int q = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += q;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        int at = inc - n, count = 0;
+        for (int k = 0; k < SB / 32; k++) {
+            at += k < warp ? wsum[k] : 0;
+            count += wsum[k];
+        }
+        if (n > 0)
+            for (int k = 0; k < 16; k++)
+                if ((w[k >> 2] >> (8 * (k & 3))) & 1u) list[at++] = (unsigned short)(16 * threadIdx.x + k);
+        __syncthreads();
+        for (int i = threadIdx.x; i < count; i += SB) {
+            const long long c = c0 + list[i];
+            if (part) {
+                if (REC) {
+                    const float4 f = rec[c];
+                    const double r = (double)f.w;
+                    v[0] += r;
+                    v[1] += r * (double)f.x;
+                    v[2] += r * (double)f.y;
+                    v[3] += r * (double)f.z;
+                } else {
+                    const double r = rho[c];
+                    v[0] += r;
+                    v[1] += r * u[c];
+                    v[2] += r * u[N + c];
+                    v[3] += r * u[2 * N + c];
+                }
+            }
+            const int p = owner[c];
+            if (REC && p == NO_OWNER) {
+                rec[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+                continue;
+            }
+            double uw[3] = {0, 0, 0};
+            if (p != NO_OWNER) {
+                const unsigned zq = fdxy.div((unsigned)c), rem = (unsigned)c - zq * (unsigned)(nx * ny);
+                const unsigned yq = fdx.div(rem);
+                const int x = (int)(rem - yq * (unsigned)nx), y = (int)yq, z = (int)zq;
+                const double r0 = dmimg(x - X[3 * p], nx), r1 = dmimg(y - X[3 * p + 1], ny), r2 = dmimg(z - X[3 * p + 2], nz);
+                uw[0] = U[3 * p] + (W[3 * p + 1] * r2 - W[3 * p + 2] * r1);
+                uw[1] = U[3 * p + 1] + (W[3 * p + 2] * r0 - W[3 * p] * r2);
+                uw[2] = U[3 * p + 2] + (W[3 * p] * r1 - W[3 * p + 1] * r0);
+            }
+            if (REC) {
+                const float2 v0 = pair_of(uw[0]), v1 = pair_of(uw[1]), v2 = pair_of(uw[2]);
+                rec[c] = make_float4(v0.x, v1.x, v2.x, MASKED);
+                ((float4 *)u)[c] = make_float4(v0.y, v1.y, v2.y, 0.f);
+            } else {
+                u[c] = uw[0];
+                u[N + c] = uw[1];
+                u[2 * N + c] = uw[2];
             }
         }
+        __syncthreads();
     }
-    sblock_sum<7>(v, sh);
+    if (!part) return;
+    __shared__ double sh[4 * (SB / 32)];
+    sblock_sum<4, SB>(v, sh);
     if (threadIdx.x == 0)
-        for (int k = 0; k < 7; k++) part[blockIdx.x * NP + 4 + k] = v[k];
+        for (int k = 0; k < 4; k++) part[blockIdx.x * NP + ST_SMASS + k] = v[k];
 }
 
 // Nearest particle surface of the fluid cells with 0 < s <= reach, s = r -
@@ -267,40 +299,279 @@ __device__ __forceinline__ long long warp_slot(bool take, long long *count) {
     return (long long)base + __popc(m & ((1u << lane) - 1u));
 }
 
-constexpr int NBIN = LBM_NBINS;
+// The sums of lbm_stats in one pass over the cells.
+//
+// What bounds it: FP64 storage, the FP64 pipe (two multiply-adds per clock
+// and SM; about 31 operations per cell). 32- and 16-bit storage have FP32
+// fields, so there the differences are exact as pairs of floats and sums and
+// squares are carried as such pairs (about 48 bits, see pair_add): some 250
+// FP32 operations in place of 45 FP64 issues of 16 clocks each (cells with a
+// masked particle cell among their neighbours add its low part), and every
+// 64 planes the pairs go into FP64 sums.
+// A thread takes a column (x, y) over a run of z: every velocity is loaded
+// once along z, s_ij s_ij comes from undivided differences, no division. The
+// radial bins are private to the thread (shared memory, [bin][thread]: no
+// atomics, no bank conflicts); FP64 atomics on 40 shared bins per block,
+// contended by the lanes of a warp, were most of the former bins pass. The
+// bin index is decided in FP32 from the distance in the cell's key (20 bits
+// of mantissa) away from the bin edges and by the exact FP64 quotient within
+// 2e-4 of one. A plane's loads are issued one plane ahead: only 8 warps per SM
+// fit beside the bins.
+// 256^3, 2000 spheres, FP32, with bins: 0.7 ms in place of 1.57 (energies) +
+// 2.9 (bins); 1.74 ms in FP64, 1.12 without the loads ahead.
+constexpr int ST_TB = 128;   // threads: 32 x 4 columns
+constexpr int ST_RUN = 64;   // planes per tile
 
-__global__ void __launch_bounds__(SB) bins_kernel(const double *u, const uint8_t *flags, const unsigned long long *near_key,
-                                                  const double *X, const double *R, int nx, int ny, int nz,
-                                                  long long N, double nu, double *bpart, const float *eps_o) {
-    __shared__ double sk[NBIN], se[NBIN], sc[NBIN];
-    for (int b = threadIdx.x; b < NBIN; b += SB) sk[b] = se[b] = sc[b] = 0.0;
-    __syncthreads();
-    // accumulate per block in shared memory with FP64 atomics, then write
-    // (per-bin sums of a few values each; order effects stay at round-off)
-    for (long long c = (long long)blockIdx.x * SB + threadIdx.x; c < N; c += (long long)SNB * SB) {
-        if (flags[c] & FL_SOLID) continue;
-        const unsigned long long key = near_key[c];
-        if (key == NEAR_EMPTY) continue;
-        const int p = near_pid_of(key);
-        const int x = (int)(c % nx), y = (int)((c / nx) % ny), z = (int)(c / ((long long)nx * ny));
-        const double dx = dmimg(__dsub_rn((double)x, X[3 * p]), nx);
-        const double dy = dmimg(__dsub_rn((double)y, X[3 * p + 1]), ny);
-        const double dz = dmimg(__dsub_rn((double)z, X[3 * p + 2]), nz);
+struct StatsArgs {
+    const double *u, *rho;  // FP64 fields; with records: u holds the low parts of masked particle cells' velocities
+    const float4 *rec;      // FP32 records, or null
+    const uint8_t *flags;
+    const unsigned long long *near_key;
+    const double *X, *R;
+    float bins_per_unit;  // 1 / (0.05 R) where all particles have one radius, else 0
+    const float *eps_o;  // dissipation from the closure where >= 0, or null
+    int nx, ny, nz;
+    long long N;
+    double nu;
+    int pipe, ibb, raw;  // raw: solid cells hold the virtual fluid (no mask) and count in mass and momentum
+    double *part, *bpart;
+};
+
+// radial bin of a fluid cell from its nearest particle's key, or -1
+__device__ __forceinline__ int radial_bin(const StatsArgs &a, unsigned long long key, int x, int y, int z) {
+    if (key == NEAR_EMPTY) return -1;
+    const int p = near_pid_of(key);
+    // the key's distance s with the upper 20 bits of its mantissa
+    const unsigned hi = (unsigned)(key >> 32);
+    const float s = __uint_as_float((((hi >> 20) - 896u) << 23) | ((hi & 0xfffffu) << 3));
+    const float tb = s * (a.bins_per_unit > 0.f ? a.bins_per_unit : 20.0f / (float)a.R[p]);  // (r / R - 1) / 0.05
+    int b = (int)tb;
+    if (fabsf(tb - rintf(tb)) < 2e-4f) {  // tb carries at most 5e-5
+        const double dx = dmimg(__dsub_rn((double)x, a.X[3 * p]), a.nx);
+        const double dy = dmimg(__dsub_rn((double)y, a.X[3 * p + 1]), a.ny);
+        const double dz = dmimg(__dsub_rn((double)z, a.X[3 * p + 2]), a.nz);
         const double rr = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
-        const double ratio = __ddiv_rn(rr, R[p]);
-        const int b = (int)floor(__ddiv_rn(__dsub_rn(ratio, 1.0), 0.05));
-        if (b < 0 || b >= NBIN) continue;
-        const double k = 0.5 * (u[c] * u[c] + u[N + c] * u[N + c] + u[2 * N + c] * u[2 * N + c]);
-        atomicAdd(&sk[b], k);
-        atomicAdd(&se[b], (eps_o && eps_o[c] >= 0.f) ? (double)eps_o[c] : cell_eps(u, x, y, z, nx, ny, nz, N, nu));
-        atomicAdd(&sc[b], 1.0);
+        b = (int)floor(__ddiv_rn(__dsub_rn(__ddiv_rn(rr, a.R[p]), 1.0), 0.05));
     }
-    __syncthreads();
-    for (int b = threadIdx.x; b < NBIN; b += SB) {
-        bpart[blockIdx.x * 3 * NBIN + b] = sk[b];
-        bpart[blockIdx.x * 3 * NBIN + NBIN + b] = se[b];
-        bpart[blockIdx.x * 3 * NBIN + 2 * NBIN + b] = sc[b];
+    return b >= 0 && b < NBIN ? b : -1;
+}
+
+// sum of D_aa^2 plus half the sum over a < b of (D_ab + D_ba)^2: 4 s_ij s_ij
+__device__ __forceinline__ double strain4(const double D[3][3]) {
+    const double sd = fma(D[0][0], D[0][0], fma(D[1][1], D[1][1], D[2][2] * D[2][2]));
+    const double sxy = D[0][1] + D[1][0], sxz = D[0][2] + D[2][0], syz = D[1][2] + D[2][1];
+    return fma(0.5, fma(sxy, sxy, fma(sxz, sxz, syz * syz)), sd);
+}
+
+// What a column's march gives per cell, as FP64 (V = double) or pairs (V = float2)
+template <typename V> struct Sums;
+template <> struct Sums<double> {
+    static __device__ __forceinline__ double zero() { return 0.0; }
+    static __device__ __forceinline__ double add(double a, double b) { return a + b; }
+    static __device__ __forceinline__ double mul_add(double r, double w, double s) { return fma(r, w, s); }
+    static __device__ __forceinline__ double of(double v) { return v; }
+    static __device__ __forceinline__ double value(double v) { return v; }
+};
+template <> struct Sums<float2> {
+    static __device__ __forceinline__ float2 zero() { return make_float2(0.f, 0.f); }
+    static __device__ __forceinline__ float2 add(float2 a, float2 b) { return pair_add(a, b); }
+    static __device__ __forceinline__ float2 mul_add(float r, float w, float2 s) { return pair_add(s, pair_mul(r, w)); }
+    static __device__ __forceinline__ float2 of(double v) { return pair_of(v); }
+    static __device__ __forceinline__ double value(float2 v) { return pair_value(v); }
+};
+
+template <bool BINS, typename V>
+__global__ void __launch_bounds__(ST_TB) stats_kernel(StatsArgs a) {
+    constexpr bool REC = sizeof(V) == 8 && !std::is_same<V, double>::value;
+    typedef Sums<V> M;
+    extern __shared__ double acc_raw[];  // BINS: u.u and 4 s_ij s_ij, [2][NBIN][ST_TB], then NBIN counts
+    V *acc = reinterpret_cast<V *>(acc_raw);
+    int *cnt = (int *)(acc + 2 * NBIN * ST_TB);
+    const int t = threadIdx.x;
+    if (BINS) {
+        for (int i = t; i < 2 * NBIN * ST_TB; i += ST_TB) acc[i] = M::zero();
+        for (int i = t; i < NBIN; i += ST_TB) cnt[i] = 0;
+        __syncthreads();
     }
+    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    const long long N = a.N, nxy = (long long)nx * ny;
+    const long long ntx = (nx + 31) / 32, nty = (ny + 3) / 4, ntz = (nz + ST_RUN - 1) / ST_RUN;
+    const double to_eps = 0.5 * a.nu, from_eps = 1.0 / to_eps;  // 2 nu s_ij s_ij = (nu / 2) 4 s_ij s_ij
+    double v[10];
+    for (int k = 0; k < 10; k++) v[k] = 0.0;
+    int nf = 0;
+    for (long long tile = blockIdx.x; tile < ntx * nty * ntz; tile += gridDim.x) {
+        const int x = (int)(tile % ntx) * 32 + (t & 31), y = (int)((tile / ntx) % nty) * 4 + (t >> 5);
+        if (x >= nx || y >= ny) continue;
+        const int z0 = (int)(tile / (ntx * nty)) * ST_RUN, z1 = min(nz, z0 + ST_RUN), zb = z0 == 0 ? nz - 1 : z0 - 1;
+        const long long c = x + (long long)nx * y;
+        const int oxm = x == 0 ? nx - 1 : -1, oxp = x == nx - 1 ? 1 - nx : 1;
+        const long long oym = y == 0 ? (long long)nx * (ny - 1) : -nx, oyp = y == ny - 1 ? -(long long)nx * (ny - 1) : nx;
+        const double *u = a.u + c;
+        const float4 *rec = a.rec + c, *lo = (const float4 *)a.u + c;
+        double um[3], uc[3];
+        float4 fm = make_float4(0.f, 0.f, 0.f, 0.f), fc = fm;
+        if constexpr (REC) {
+            fm = rec[nxy * zb];
+            fc = rec[nxy * z0];
+        } else {
+            for (int d = 0; d < 3; d++) {
+                um[d] = u[d * N + nxy * zb];
+                uc[d] = u[d * N + nxy * z0];
+            }
+        }
+        V s[8];
+        for (int k = 0; k < 8; k++) s[k] = M::zero();
+        V suz = M::zero();
+        // the loads of a plane are issued one plane ahead (few warps fit beside the bins)
+        float4 nb[5];
+        unsigned char nfl;
+        float neo = -1.f;
+        unsigned long long nkey = NEAR_EMPTY;
+        auto fetch = [&](int z) {
+            const long long e = nxy * z;
+            if constexpr (REC) {
+                nb[0] = rec[e + oxp];
+                nb[1] = rec[e + oxm];
+                nb[2] = rec[e + oyp];
+                nb[3] = rec[e + oym];
+                nb[4] = rec[z == nz - 1 ? 0 : e + nxy];
+            }
+            nfl = a.flags[c + e];
+            if (a.eps_o) neo = a.eps_o[c + e];
+            if (BINS) nkey = a.near_key[c + e];
+        };
+        fetch(z0);
+        for (int z = z0; z < z1; z++) {
+            const long long e = nxy * z, ep = z == nz - 1 ? 0 : e + nxy, em = z == 0 ? nxy * (nz - 1) : e - nxy;
+            const bool solid = nfl & FL_SOLID;
+            const float eo = neo;
+            const unsigned long long key = nkey;
+            const float4 xp = nb[0], xm = nb[1], yp = nb[2], ym = nb[3], zp = nb[4];
+            if (z + 1 < z1) fetch(z + 1);
+            V kk, ss;  // u.u, 4 s_ij s_ij
+            if constexpr (REC) {
+                if (fminf(fminf(fminf(xp.w, xm.w), fminf(yp.w, ym.w)), fminf(fminf(zp.w, fm.w), fc.w)) == MASKED) {
+                    // a masked particle cell among them: its velocity has a low part
+                    auto low = [&](const float4 &f, long long o) -> float4 {
+                        return f.w == MASKED ? lo[o] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    };
+                    const float4 lxp = low(xp, e + oxp), lxm = low(xm, e + oxm), lyp = low(yp, e + oyp),
+                                 lym = low(ym, e + oym), lzp = low(zp, ep), lzm = low(fm, em), lc = low(fc, e);
+                    auto diff = [](float a, float b, float la, float lb) -> float2 {
+                        return pair_add(pair_diff(a, b), make_float2(la - lb, 0.f));
+                    };
+                    kk = pair_add(pair_add(pair_square(make_float2(fc.x, lc.x)), pair_square(make_float2(fc.y, lc.y))),
+                                  pair_square(make_float2(fc.z, lc.z)));
+                    const float2 sxy = pair_add(diff(yp.x, ym.x, lyp.x, lym.x), diff(xp.y, xm.y, lxp.y, lxm.y)),
+                                 sxz = pair_add(diff(zp.x, fm.x, lzp.x, lzm.x), diff(xp.z, xm.z, lxp.z, lxm.z)),
+                                 syz = pair_add(diff(zp.y, fm.y, lzp.y, lzm.y), diff(yp.z, ym.z, lyp.z, lym.z));
+                    const float2 off = pair_add(pair_add(pair_square(sxy), pair_square(sxz)), pair_square(syz));
+                    ss = pair_add(pair_add(pair_square(diff(xp.x, xm.x, lxp.x, lxm.x)),
+                                           pair_square(diff(yp.y, ym.y, lyp.y, lym.y))),
+                                  pair_add(pair_square(diff(zp.z, fm.z, lzp.z, lzm.z)),
+                                           make_float2(0.5f * off.x, 0.5f * off.y)));
+                } else {
+                    kk = pair_add(pair_add(pair_mul(fc.x, fc.x), pair_mul(fc.y, fc.y)), pair_mul(fc.z, fc.z));
+                    const float2 sxy = pair_add(pair_diff(yp.x, ym.x), pair_diff(xp.y, xm.y)),
+                                 sxz = pair_add(pair_diff(zp.x, fm.x), pair_diff(xp.z, xm.z)),
+                                 syz = pair_add(pair_diff(zp.y, fm.y), pair_diff(yp.z, ym.z));
+                    const float2 off = pair_add(pair_add(pair_square(sxy), pair_square(sxz)), pair_square(syz));
+                    ss = pair_add(pair_add(pair_square(pair_diff(xp.x, xm.x)), pair_square(pair_diff(yp.y, ym.y))),
+                                  pair_add(pair_square(pair_diff(zp.z, fm.z)), make_float2(0.5f * off.x, 0.5f * off.y)));
+                }
+                fm = fc;
+                fc = zp;
+            } else {
+                double D[3][3], w[3];  // differences: twice the gradients
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    const double *ud = u + d * N;
+                    const double up = ud[ep];
+                    D[d][0] = ud[e + oxp] - ud[e + oxm];
+                    D[d][1] = ud[e + oyp] - ud[e + oym];
+                    D[d][2] = up - um[d];
+                    w[d] = uc[d];
+                    um[d] = uc[d];
+                    uc[d] = up;
+                }
+                kk = fma(w[0], w[0], fma(w[1], w[1], w[2] * w[2]));
+                ss = strain4(D);
+            }
+            if (eo >= 0.f) ss = M::of((double)eo * from_eps);
+            if (solid) {
+                s[ST_KS] = M::add(s[ST_KS], kk);
+                s[ST_ES] = M::add(s[ST_ES], ss);
+                if (!a.raw) continue;
+            }
+            if (!solid || (a.raw && !a.ibb)) {
+                if constexpr (REC) {  // fm: this cell now
+                    s[ST_MASS] = M::add(s[ST_MASS], make_float2(fm.w, 0.f));
+                    s[ST_MX] = M::mul_add(fm.w, fm.x, s[ST_MX]);
+                    s[ST_MY] = M::mul_add(fm.w, fm.y, s[ST_MY]);
+                    s[ST_MZ] = M::mul_add(fm.w, fm.z, s[ST_MZ]);
+                } else {
+                    const double r = a.rho[c + e];
+                    s[ST_MASS] = M::add(s[ST_MASS], r);
+                    s[ST_MX] = M::mul_add(r, um[0], s[ST_MX]);
+                    s[ST_MY] = M::mul_add(r, um[1], s[ST_MY]);
+                    s[ST_MZ] = M::mul_add(r, um[2], s[ST_MZ]);
+                }
+            }
+            if (solid) continue;
+            s[ST_KF] = M::add(s[ST_KF], kk);
+            s[ST_EF] = M::add(s[ST_EF], ss);
+            nf++;
+            if (a.pipe) {
+                if constexpr (REC) suz = M::add(suz, make_float2(fm.z, 0.f));
+                else suz = M::add(suz, um[2]);
+            }
+            if (BINS) {
+                const int b = radial_bin(a, key, x, y, z);
+                if (b < 0) continue;
+                acc[b * ST_TB + t] = M::add(acc[b * ST_TB + t], kk);
+                acc[(NBIN + b) * ST_TB + t] = M::add(acc[(NBIN + b) * ST_TB + t], ss);
+                atomicAdd(cnt + b, 1);
+            }
+        }
+        for (int k = 0; k < 8; k++) v[k] += M::value(s[k]);
+        v[ST_UZ] += M::value(suz);
+    }
+    v[ST_NF] = (double)nf;
+    v[ST_EF] *= to_eps;
+    v[ST_ES] *= to_eps;
+    __shared__ double sh[10 * (ST_TB / 32)];
+    sblock_sum<10, ST_TB>(v, sh);
+    if (t == 0)
+        for (int k = 0; k < 10; k++) a.part[blockIdx.x * NP + k] = v[k];
+    if (BINS) {
+        __syncthreads();
+        // one warp per bin and quantity in turn: fixed order
+        for (int i = t >> 5; i < 2 * NBIN; i += ST_TB / 32) {
+            double q = 0.0;
+            for (int k = t & 31; k < ST_TB; k += 32) q += M::value(acc[i * ST_TB + k]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            if ((t & 31) == 0) a.bpart[blockIdx.x * 3 * NBIN + i] = i < NBIN ? q : q * to_eps;
+        }
+        for (int i = t; i < NBIN; i += ST_TB) a.bpart[blockIdx.x * 3 * NBIN + 2 * NBIN + i] = (double)cnt[i];
+    }
+}
+
+// the blocks' sums added in a fixed order: column blockIdx.x of nblk rows
+__global__ void __launch_bounds__(SB) stats_reduce_kernel(const double *part, const double *bpart, int nblk, int mblk,
+                                                          double *out) {
+    const int k = blockIdx.x;
+    double v[1] = {0.0};
+    if (k < NP) {
+        const int n = k >= ST_SMASS ? mblk : nblk;
+        for (int b = threadIdx.x; b < n; b += SB) v[0] += part[(size_t)b * NP + k];
+    } else {
+        for (int b = threadIdx.x; b < nblk; b += SB) v[0] += bpart[(size_t)b * 3 * NBIN + (k - NP)];
+    }
+    __shared__ double sh[SB / 32];
+    sblock_sum<1, SB>(v, sh);
+    if (threadIdx.x == 0) out[k] = v[0];
 }
 
 __global__ void fill_u64(unsigned long long *p, unsigned long long v, long long n) {
@@ -373,37 +644,58 @@ __global__ void closure_target_kernel(const double *u, const uint8_t *flags, con
 
 // the near-surface fluid nodes of the fused closure dissipation: cell and
 // nearest particle (distance to the surface in (0, 2]); order not fixed
-// One slot range per block and 256 consecutive cells, filled in cell
+// One slot range per block and 1024 consecutive cells, filled in cell
 // order, so that neighbouring samples of the list are mostly neighbouring
 // cells (their stencils share lines in the inference kernel's gather).
+// (four cells per thread: 119 us per call at 256^3 with one)
 __global__ void __launch_bounds__(256) closure_list_kernel(const uint8_t *flags, const unsigned long long *near_key,
                                                            long long N, int *cells, int *pids, long long *count,
                                                            long long cap) {
     __shared__ unsigned wcnt[8];
     __shared__ unsigned long long base;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long span = (long long)gridDim.x * blockDim.x;
-    for (long long c0 = (long long)blockIdx.x * blockDim.x; c0 < N; c0 += span) {
-        const long long c = c0 + threadIdx.x;
-        const unsigned long long key = c < N && !(flags[c] & FL_SOLID) ? near_key[c] : NEAR_EMPTY;
-        const double d = near_s_of(key);  // r - R_p of the nearest particle
-        const bool take = key != NEAR_EMPTY && d > 0.0 && d <= 2.0;
-        const unsigned m = __ballot_sync(0xffffffffu, take);
-        if (lane == 0) wcnt[warp] = (unsigned)__popc(m);
-        __syncthreads();
-        unsigned before = 0, total = 0;
-        for (int w = 0; w < 8; w++) {
-            before += w < warp ? wcnt[w] : 0u;
-            total += wcnt[w];
+    const long long c = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
+    unsigned long long key[4] = {NEAR_EMPTY, NEAR_EMPTY, NEAR_EMPTY, NEAR_EMPTY};
+    if (c + 4 <= N) {
+        const ulonglong2 k0 = *(const ulonglong2 *)(near_key + c), k1 = *(const ulonglong2 *)(near_key + c + 2);
+        key[0] = k0.x;
+        key[1] = k0.y;
+        key[2] = k1.x;
+        key[3] = k1.y;
+    } else {
+        for (int k = 0; k < 4; k++)
+            if (c + k < N) key[k] = near_key[c + k];
+    }
+    unsigned take = 0;
+    for (int k = 0; k < 4; k++) {
+        if (key[k] == NEAR_EMPTY || (flags[c + k] & FL_SOLID)) continue;
+        const double d = near_s_of(key[k]);  // r - R_p of the nearest particle
+        if (d > 0.0 && d <= 2.0) take |= 1u << k;
+    }
+    const unsigned n = __popc(take);
+    unsigned inc = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned q = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += q;
+    }
+    if (lane == 31) wcnt[warp] = inc;
+    __syncthreads();
+    unsigned before = inc - n, total = 0;
+    for (int w = 0; w < 8; w++) {
+        before += w < warp ? wcnt[w] : 0u;
+        total += wcnt[w];
+    }
+    if (threadIdx.x == 0) base = total ? atomicAdd((unsigned long long *)count, (unsigned long long)total) : 0ull;
+    __syncthreads();
+    long long at = (long long)base + before;
+    for (int k = 0; k < 4; k++) {
+        if (!((take >> k) & 1u)) continue;
+        if (at < cap) {
+            cells[at] = (int)(c + k);
+            pids[at] = near_pid_of(key[k]);
         }
-        if (threadIdx.x == 0) base = total ? atomicAdd((unsigned long long *)count, (unsigned long long)total) : 0ull;
-        __syncthreads();
-        const long long k = (long long)base + before + __popc(m & ((1u << lane) - 1u));
-        if (take && k < cap) {
-            cells[k] = (int)c;
-            pids[k] = near_pid_of(key);
-        }
-        __syncthreads();  // wcnt and base are rewritten next round
+        at++;
     }
 }
 
@@ -429,6 +721,19 @@ __global__ void fill_f32(float *p, float v, long long n) {
     if (i < n) p[i] = v;
 }
 
+
+static int mask_blocks(const Ctx &c) { return (int)std::min<long long>(SNB, (c.N + MASK_RUN - 1) / MASK_RUN); }
+static cudaError_t mask_cells(Ctx &c, double *part, float4 *rec = nullptr) {
+    if (c.np == 0 && !c.has_pipe) return cudaSuccess;  // no solid cell
+    const FastDiv fdx((unsigned)c.nx), fdxy((unsigned)(c.nx * c.ny));
+    if (rec)
+        mask_kernel<true><<<mask_blocks(c), SB, 0, c.stream>>>(rec, c.u_f, c.rho_f, c.flags, c.owner, c.X, c.U, c.W, c.nx,
+                                                               c.ny, c.nz, fdx, fdxy, c.N, part);
+    else
+        mask_kernel<false><<<mask_blocks(c), SB, 0, c.stream>>>(nullptr, c.u_f, c.rho_f, c.flags, c.owner, c.X, c.U, c.W,
+                                                                c.nx, c.ny, c.nz, fdx, fdxy, c.N, part);
+    return cudaGetLastError();
+}
 
 // nearest particle and distance to its surface of the fluid cells within
 // `reach` of a surface (key and pid; others NO_OWNER)
@@ -459,9 +764,8 @@ cudaError_t closure_samples(Ctx &c, double u_scale, float *X, int *cells, long l
 cudaError_t closure_targets(Ctx &c, const int *cells, long long n, double g_scale, float *T) {
     cudaError_t e;
     if ((e = launch_macro(c, 0)) != cudaSuccess) return e;
-    const unsigned nb = (unsigned)((c.N + 255) / 256);
     count_launch(c, G_STATS, 2);
-    mask_kernel<<<nb, 256, 0, c.stream>>>(c.u_f, c.flags, c.owner, c.X, c.U, c.W, c.nx, c.ny, c.nz, c.N);
+    if ((e = mask_cells(c, nullptr)) != cudaSuccess) return e;
     if (n > 0)
         closure_target_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(c.u_f, c.flags, cells, n, c.nx, c.ny,
                                                                               c.nz, c.N, g_scale, T);
@@ -586,9 +890,7 @@ cudaError_t launch_mask(Ctx &c) {
     // the fields of an IBB pipe on columns are zero outside it already
     if (c.zlay && c.q == 19 && c.armed_bc == LBM_BC_IBB) return cudaSuccess;
     count_launch(c, G_STATS);
-    mask_kernel<<<(unsigned)((c.N + 255) / 256), 256, 0, c.stream>>>(c.u_f, c.flags, c.owner, c.X, c.U, c.W, c.nx,
-                                                                     c.ny, c.nz, c.N);
-    return cudaGetLastError();
+    return mask_cells(c, nullptr);
 }
 
 cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
@@ -597,12 +899,13 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
     const int ibb = c.armed_bc == LBM_BC_IBB;
     const int ibm = c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B;
     const bool closure = (flags & LBM_STATS_CLOSURE) && c.np > 0 && c.cl_ready && c.max_cl > 0 && c.q == 19;
-    // the closure gathers an FP32 copy of u (16 B per cell), kept in the
-    // population buffer that the next step overwrites (19 x 2 B per cell or more)
-    float *u32 = closure ? (float *)c.fB : nullptr;
-    if ((e = launch_macro(c, 0, u32)) != cudaSuccess) return e;
+    // FP32 records of the fields (16 B per cell) in the population buffer that
+    // the next step overwrites (19 x 2 B per cell or more): all that 32- and
+    // 16-bit storage needs, and the closure's gather input
+    const bool rec = c.storage != LBM_F64;
+    float *u32 = rec || closure ? (float *)c.fB : nullptr;
+    if ((e = launch_macro(c, 0, u32, rec)) != cudaSuccess) return e;
     count_launch(c, G_STATS, 3);
-    mass_kernel<<<SNB, SB, 0, c.stream>>>(c.rho_f, c.u_f, c.flags, c.N, ibb, c.partials);
     const bool mask = !(ibm && (flags & LBM_STATS_UNMASK));
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     const double nu = (c.tau - 0.5) / 3.0;
@@ -621,7 +924,7 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
         if ((e = cudaMemsetAsync(c.d_counts + 3, 0, sizeof(long long), c.stream)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(c.d_status + 1, 0, sizeof(unsigned), c.stream)) != cudaSuccess) return e;
         int *pids = (int *)c.cl_X;  // the feature buffer is not needed by the fused path
-        closure_list_kernel<<<nb, 256, 0, c.stream>>>(c.flags, c.near_key, c.N, c.cl_cells, pids, c.d_counts + 3,
+        closure_list_kernel<<<(unsigned)((c.N + 1023) / 1024), 256, 0, c.stream>>>(c.flags, c.near_key, c.N, c.cl_cells, pids, c.d_counts + 3,
                                                       c.max_cl);
         if ((e = mlp_pack_device(c.cl_w, c.cl_pk, c.stream)) != cudaSuccess) return e;
         cudaEvent_t t0 = prof_event(c);
@@ -632,22 +935,28 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
         prof_span(c, G_CLOSURE, t0, prof_event(c));
         eps_o = c.cl_eps;
     }
-    if (mask) mask_kernel<<<nb, 256, 0, c.stream>>>(c.u_f, c.flags, c.owner, c.X, c.U, c.W, c.nx, c.ny, c.nz, c.N);
-    energy_kernel<<<SNB, SB, 0, c.stream>>>(c.u_f, c.flags, c.nx, c.ny, c.nz, c.N, nu, c.has_pipe, c.partials, eps_o);
-    double *bpart = c.partials + SNB * NP;
-    if (bins) {
-        count_launch(c, G_STATS);
-        bins_kernel<<<SNB, SB, 0, c.stream>>>(c.u_f, c.flags, c.near_key, c.X, c.R, c.nx, c.ny, c.nz, c.N, nu, bpart,
-                                              eps_o);
-    }
+    // what the masked solid cells held counts in mass and momentum unless the wall is IBB
+    const bool solid_held = mask && !ibb;
+    double *bpart = c.partials + (size_t)SNB * NP, *res = bpart + (size_t)SNB * 3 * NBIN;
+    if (mask && !(c.zlay && c.q == 19 && ibb))
+        if ((e = mask_cells(c, solid_held ? c.partials : nullptr, rec ? (float4 *)u32 : nullptr)) != cudaSuccess) return e;
+    const int mblk = solid_held && (c.np > 0 || c.has_pipe) ? mask_blocks(c) : 0;
+    StatsArgs a{c.u_f, c.rho_f, rec ? (const float4 *)u32 : nullptr, c.flags, c.near_key, c.X, c.R,
+                c.same_radius ? 20.0f / (float)c.max_radius : 0.f, eps_o, c.nx, c.ny, c.nz, c.N, nu, c.has_pipe, ibb, !mask,
+                c.partials, bpart};
+    const long long tiles = (long long)((c.nx + 31) / 32) * ((c.ny + 3) / 4) * ((c.nz + ST_RUN - 1) / ST_RUN);
+    const int nblk = (int)std::min<long long>(tiles, SNB);
+    const size_t smem = bins ? sizeof(double) * 2 * NBIN * ST_TB + sizeof(int) * NBIN : 0;
+    void (*kernel)(StatsArgs) = bins ? (rec ? stats_kernel<true, float2> : stats_kernel<true, double>)
+                                     : (rec ? stats_kernel<false, float2> : stats_kernel<false, double>);
+    if (bins && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
+    kernel<<<nblk, ST_TB, smem, c.stream>>>(a);
+    const int ncol = NP + (bins ? 3 * NBIN : 0);
+    stats_reduce_kernel<<<ncol, SB, 0, c.stream>>>(c.partials, bpart, nblk, mblk, res);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    std::vector<double> part((size_t)SNB * NP), bp(bins ? (size_t)SNB * 3 * NBIN : 0);
-    if ((e = cudaMemcpyAsync(part.data(), c.partials, sizeof(double) * part.size(), cudaMemcpyDeviceToHost,
-                             c.stream)) != cudaSuccess)
-        return e;
-    if (bins && (e = cudaMemcpyAsync(bp.data(), bpart, sizeof(double) * bp.size(), cudaMemcpyDeviceToHost,
-                                     c.stream)) != cudaSuccess)
-        return e;
+    double s[NP + 3 * NBIN] = {0};
+    if ((e = cudaMemcpyAsync(s, res, sizeof(double) * ncol, cudaMemcpyDeviceToHost, c.stream)) != cudaSuccess) return e;
     std::vector<double> P(3 * c.np), Uh(3 * c.np), Wh(3 * c.np), Fh(3 * c.np), Th(3 * c.np), mass(c.np), inertia(c.np);
     if (c.np > 0) {
         cudaMemcpyAsync(Uh.data(), c.U, sizeof(double) * 3 * c.np, cudaMemcpyDeviceToHost, c.stream);
@@ -663,19 +972,14 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
         return e;
     if ((e = cudaStreamSynchronize(c.stream)) != cudaSuccess) return e;
     if (tc_err) return cudaErrorLaunchTimeout;  // a tensor-core wait of the closure ran out
-    double s[NP] = {0};
-    for (int b = 0; b < SNB; b++)
-        for (int k = 0; k < 11; k++) s[k] += part[(size_t)b * NP + k];
-    o->mass = s[0];
-    o->momentum[0] = s[1];
-    o->momentum[1] = s[2];
-    o->momentum[2] = s[3];
-    o->kinetic_energy = s[4] / (double)c.N;
-    o->dissipation = s[5] / (double)c.N;
-    o->nfluid = (long long)s[8];
-    o->kinetic_energy_fluid = s[8] > 0 ? s[6] / s[8] : 0.0;
-    o->dissipation_fluid = s[8] > 0 ? s[7] / s[8] : 0.0;
-    o->bulk_velocity = s[10] > 0 ? s[9] / s[10] : 0.0;
+    o->mass = s[ST_MASS] + s[ST_SMASS];
+    for (int d = 0; d < 3; d++) o->momentum[d] = s[ST_MX + d] + s[ST_SX + d];
+    o->kinetic_energy = 0.5 * (s[ST_KF] + s[ST_KS]) / (double)c.N;
+    o->dissipation = (s[ST_EF] + s[ST_ES]) / (double)c.N;
+    o->nfluid = (long long)s[ST_NF];
+    o->kinetic_energy_fluid = s[ST_NF] > 0 ? 0.5 * s[ST_KF] / s[ST_NF] : 0.0;
+    o->dissipation_fluid = s[ST_NF] > 0 ? s[ST_EF] / s[ST_NF] : 0.0;
+    o->bulk_velocity = c.has_pipe && s[ST_NF] > 0 ? s[ST_UZ] / s[ST_NF] : 0.0;
     for (int p = 0; p < c.np; p++) {
         double U2 = 0, W2 = 0;
         for (int d = 0; d < 3; d++) {
@@ -688,13 +992,7 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
         o->particle_ake += 0.5 * inertia[p] * W2;
     }
     if (bins) {
-        double sk[NBIN] = {0}, se[NBIN] = {0}, sc[NBIN] = {0};
-        for (int b = 0; b < SNB; b++)
-            for (int k = 0; k < NBIN; k++) {
-                sk[k] += bp[(size_t)b * 3 * NBIN + k];
-                se[k] += bp[(size_t)b * 3 * NBIN + NBIN + k];
-                sc[k] += bp[(size_t)b * 3 * NBIN + 2 * NBIN + k];
-            }
+        const double *sk = s + NP, *se = sk + NBIN, *sc = se + NBIN;
         o->nbins = NBIN;
         for (int k = 0; k < NBIN; k++) {
             o->bin_r[k] = 1.0 + 0.05 * (k + 0.5);
@@ -702,7 +1000,7 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
             if (sc[k] > 0) {
                 const double kf = o->kinetic_energy_fluid > 0 ? o->kinetic_energy_fluid : 1.0;
                 const double ef = o->dissipation_fluid > 0 ? o->dissipation_fluid : 1.0;
-                o->bin_tke[k] = sk[k] / sc[k] / kf;
+                o->bin_tke[k] = 0.5 * sk[k] / sc[k] / kf;
                 o->bin_eps[k] = se[k] / sc[k] / ef;
             }
         }
@@ -713,6 +1011,6 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
     return cudaSuccess;
 }
 
-size_t stats_partials_doubles() { return (size_t)SNB * NP + (size_t)SNB * 3 * NBIN; }
+size_t stats_partials_doubles() { return (size_t)(SNB + 1) * (NP + 3 * NBIN); }
 
 }  // namespace lbmgb

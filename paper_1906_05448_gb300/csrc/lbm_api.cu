@@ -918,6 +918,7 @@ lbm_status lbm_add_spheres(lbm_ctx *h, int n, const double *xyz, const double *r
     c.np = n;
     c.max_radius = 0.0;
     for (int p = 0; p < n; p++) c.max_radius = R[p] > c.max_radius ? R[p] : c.max_radius;
+    c.same_radius = *std::min_element(R.begin(), R.end()) == c.max_radius;
     c.fixed = fixed != 0;
     c.dens = density_ratio;
     const size_t b3 = sizeof(double) * 3 * n, b1 = sizeof(double) * n;

@@ -84,6 +84,7 @@ struct Ctx {
     int *mpid, *m_first;
     double rd;  // marker retraction (IBM-B: 0.4)
     double max_radius;
+    bool same_radius;  // every particle has max_radius
     // pipe IBM: ring markers per plane and, per (x, y) column, the ring
     // markers whose 4x4 footprint covers it with their x-y weights
     int pipe_nc;
@@ -151,7 +152,7 @@ cudaError_t launch_column_sweep(Ctx &c);  // sweep_columns.cu: the pipe's IBB st
 // c.rho_f, the macroscopic fields
 cudaError_t convert_columns(Ctx &c, const void *src, void *dst, bool to_x, bool zero_solid);
 cudaError_t column_plane_copy(Ctx &c, int i, double w, bool to_f64);
-cudaError_t launch_column_macro(Ctx &c);
+cudaError_t launch_column_macro(Ctx &c, float4 *rec);  // rec: FP32 records instead of c.rho_f, c.u_f
 // ibm_columns.cu: the pipe's IBM step, and its forces in the order of the ABI
 cudaError_t launch_ibm_columns_sweep(Ctx &c);
 cudaError_t launch_ibm_columns_passes(Ctx &c);
@@ -176,7 +177,9 @@ cudaError_t launch_support_mark(Ctx &c);
 cudaError_t launch_ibm_passes(Ctx &c);
 cudaError_t launch_ibm_particle_sums(Ctx &c, bool init_only);
 cudaError_t launch_ibm_rigid_overwrite(Ctx &c);
-cudaError_t launch_macro(Ctx &c, int mask_mode, float *u32 = nullptr);
+// rho and u into c.rho_f and c.u_f (FP64); u32, if not null, receives FP32
+// records (ux, uy, uz, rho) per cell, alone with rec_only (32- and 16-bit storage)
+cudaError_t launch_macro(Ctx &c, int mask_mode, float *u32 = nullptr, bool rec_only = false);
 cudaError_t launch_mask(Ctx &c);  // statistics velocity: solid cells take the rigid-body velocity
 cudaError_t run_spectrum(Ctx &c, int flags, int nbins, double *E, double *D);
 cudaError_t run_pipe_profiles(Ctx &c, int flags, int nbins, double *out);
@@ -186,7 +189,7 @@ cudaError_t run_tke_budget(Ctx &c, int flags, int nbins, double *out);
 cudaError_t launch_q27_step(Ctx &c);
 cudaError_t launch_q27_init(Ctx &c, const double *u_dev, double rho0);
 cudaError_t q27_plane_copy(Ctx &c, int i, bool to_f64);
-cudaError_t launch_q27_macro(Ctx &c);
+cudaError_t launch_q27_macro(Ctx &c, float4 *rec);
 void q27_pipe_colmask(const Ctx &c, std::vector<unsigned> &mask);
 cudaError_t launch_q27_coef(Ctx &c);
 size_t tke_budget_scratch_bytes(int nbins);

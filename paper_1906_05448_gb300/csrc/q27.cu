@@ -59,7 +59,7 @@ __global__ void q27_plane_kernel(void *A, double *v, long long N, int i, int to_
 
 // rho and u of the post-collision state: sum f c = rho u + F/2
 template <int S>
-__global__ void q27_macro_kernel(const void *A, double *rho_o, double *u_o, long long N, double F0, double F1,
+__global__ void q27_macro_kernel(const void *A, float4 *rec, double *rho_o, double *u_o, long long N, double F0, double F1,
                                  double F2) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
@@ -76,6 +76,11 @@ __global__ void q27_macro_kernel(const void *A, double *rho_o, double *u_o, long
         j2 += g * R(q27z(i));
     }
     const R rho = R(1) + r, ir = R(1) / rho;
+    if (rec) {
+        rec[c] = make_float4(float((j0 - R(0.5) * R(F0)) * ir), float((j1 - R(0.5) * R(F1)) * ir),
+                             float((j2 - R(0.5) * R(F2)) * ir), float(rho));
+        return;
+    }
     rho_o[c] = double(rho);
     u_o[c] = double((j0 - R(0.5) * R(F0)) * ir);
     u_o[N + c] = double((j1 - R(0.5) * R(F1)) * ir);
@@ -84,7 +89,7 @@ __global__ void q27_macro_kernel(const void *A, double *rho_o, double *u_o, long
 
 // the same on the column layout (columns.cuh): read along z, written along x
 template <int S>
-__global__ void __launch_bounds__(256) q27_column_macro_kernel(const void *A, double *rho_o, double *u_o, int nx, int ny,
+__global__ void __launch_bounds__(256) q27_column_macro_kernel(const void *A, float4 *rec, double *rho_o, double *u_o, int nx, int ny,
                                                                int nz, int zp, long long N, long long Np, double F0,
                                                                double F1, double F2) {
     typedef typename Store<S>::T T;
@@ -112,6 +117,10 @@ __global__ void __launch_bounds__(256) q27_column_macro_kernel(const void *A, do
             },
             [&](int x, int z, const V &v) {
                 const long long c = x + (long long)nx * (y + (long long)ny * z);
+                if (rec) {
+                    rec[c] = make_float4(float(v.ux), float(v.uy), float(v.uz), float(v.rho));
+                    return;
+                }
                 rho_o[c] = double(v.rho);
                 u_o[c] = double(v.ux);
                 u_o[N + c] = double(v.uy);
@@ -467,11 +476,11 @@ cudaError_t q27_plane_copy(Ctx &c, int i, bool to_f64) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_q27_macro(Ctx &c) {
+cudaError_t launch_q27_macro(Ctx &c, float4 *rec) {
     count_launch(c, G_STATS);
     if (c.zlay) {
 #define MK(S)                                                                                                      \
-    q27_column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, c.rho_f, c.u_f, c.nx, c.ny, c.nz, c.zp, c.N, \
+    q27_column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, rec, c.rho_f, c.u_f, c.nx, c.ny, c.nz, c.zp, c.N, \
                                                                     c.Np, c.F[0], c.F[1], c.F[2])
         if (c.storage == LBM_F64) MK(LBM_F64);
         else MK(LBM_F32);
@@ -480,9 +489,9 @@ cudaError_t launch_q27_macro(Ctx &c) {
     }
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     if (c.storage == LBM_F64)
-        q27_macro_kernel<LBM_F64><<<nb, 256, 0, c.stream>>>(c.fA, c.rho_f, c.u_f, c.N, c.F[0], c.F[1], c.F[2]);
+        q27_macro_kernel<LBM_F64><<<nb, 256, 0, c.stream>>>(c.fA, rec, c.rho_f, c.u_f, c.N, c.F[0], c.F[1], c.F[2]);
     else
-        q27_macro_kernel<LBM_F32><<<nb, 256, 0, c.stream>>>(c.fA, c.rho_f, c.u_f, c.N, c.F[0], c.F[1], c.F[2]);
+        q27_macro_kernel<LBM_F32><<<nb, 256, 0, c.stream>>>(c.fA, rec, c.rho_f, c.u_f, c.N, c.F[0], c.F[1], c.F[2]);
     return cudaGetLastError();
 }
 

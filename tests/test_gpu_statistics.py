@@ -1,0 +1,83 @@
+"""lbm_stats against its numpy statement on the library's own fields: FP64 and
+FP32 fields (sums of float pairs), spheres of one and of several radii across
+the box faces, odd boxes, plane counts around the 64-plane run, masked and raw
+solid cells."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1906_05448_gb300 import build, lbm as L
+    build.build()
+    L.load()
+    return L
+
+
+def expected(u, rho, flags, P, R, shape, nu):
+    """Energies, dissipation and radial bins of the masked velocity."""
+    nz, ny, nx = shape
+    n = np.array([nx, ny, nz])
+    z, y, x = np.meshgrid(np.arange(nz), np.arange(ny), np.arange(nx), indexing="ij")
+    pos = np.stack([x, y, z], -1).reshape(-1, 3).astype(float)
+    solid = (flags & 1).astype(bool)
+    s = np.full(len(pos), np.inf)
+    near = np.zeros(len(pos), dtype=int)
+    for p in range(len(R)):
+        d = pos - P["X"][p]
+        d -= n * np.rint(d / n)
+        sp = np.sqrt((d * d).sum(1)) - R[p]
+        m = sp < s
+        s[m], near[m] = sp[m], p
+    d = pos - P["X"][near]
+    d -= n * np.rint(d / n)
+    rigid = P["U"][near] + np.cross(P["W"][near], d)
+    v = np.where(solid[:, None], rigid, u.T).T.reshape(3, nz, ny, nx)
+    G = [[0.5 * (np.roll(v[a], -1, k) - np.roll(v[a], 1, k)) for k in (2, 1, 0)] for a in range(3)]
+    eps = (2 * nu * sum((0.5 * (G[a][b] + G[b][a])) ** 2 for a in range(3) for b in range(3))).reshape(-1)
+    ke = 0.5 * (v ** 2).sum(0).reshape(-1)
+    fl = ~solid
+    b = np.floor((s / R[near]) / 0.05).astype(int)
+    ok = fl & (s > 0) & (b < 40)  # a cell on the surface to the last bit has no bin
+    cnt = np.bincount(b[ok], minlength=40)[:40]
+    per = [np.bincount(b[ok], weights=q[ok], minlength=40)[:40] / np.maximum(cnt, 1) for q in (ke, eps)]
+    return dict(mass=rho.sum(), momentum=(u * rho).sum(1), kinetic_energy=ke.mean(), dissipation=eps.mean(),
+                kinetic_energy_fluid=ke[fl].mean(), dissipation_fluid=eps[fl].mean(), nfluid=int(fl.sum()),
+                bin_count=cnt, bin_tke=per[0] / ke[fl].mean(), bin_eps=per[1] / eps[fl].mean())
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+@pytest.mark.parametrize("shape,R", [((33, 37, 41), [4.0, 4.0, 4.0]), ((65, 30, 33), [3.0, 4.5, 2.2])])
+def test_stats_of_a_snapshot(lbm, storage, shape, R):
+    nz, ny, nx = shape
+    R = np.array(R)
+    X = np.array([[1.3, 2.1, 0.7], [nx / 2 + 0.2, ny / 2, 12.4], [nx - 9.5, 9.1, nz - 9.6]])
+    rng = np.random.default_rng(3)
+    U, W = rng.normal(0, 0.01, (3, 3)), rng.normal(0, 0.002, (3, 3))
+    g = lbm.Lattice(nx, ny, nz, 0.56, storage=storage, max_particles=3)
+    g.init_velocity(workloads.noise_velocity(shape, 0.02, seed=4) + 0.01)
+    g.add_spheres(X, R, U=U, W=W)
+    got = g.stats(lbm.STATS_BINS)
+    rho, u = g.macro()
+    ref = expected(u, rho, g.flags(), g.particles(), R, shape, 0.06 / 3)
+    assert got["nfluid"] == ref["nfluid"]
+    assert np.array_equal(got["bin_count"], ref["bin_count"])
+    # sums of N terms in FP64, or as pairs of 48 bits: far below 1e-12 of the result
+    for k in ("mass", "kinetic_energy", "dissipation", "kinetic_energy_fluid", "dissipation_fluid"):
+        assert got[k] == pytest.approx(ref[k], rel=1e-12), k
+    for k in ("momentum", "bin_tke", "bin_eps"):
+        assert np.allclose(got[k], ref[k], rtol=1e-11, atol=0), k
+    g.step(2, lbm.BC_IBM_B)  # raw statistics count the fluid inside the particles
+    raw = g.stats(lbm.STATS_UNMASK)
+    rho, u = g.macro()
+    ke = 0.5 * (u ** 2).sum(0)
+    assert raw["kinetic_energy"] == pytest.approx(ke.mean(), rel=1e-12)
+    assert np.allclose(raw["momentum"], (u * rho).sum(1), rtol=1e-11, atol=0)
+    g.close()
