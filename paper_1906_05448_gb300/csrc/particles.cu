@@ -653,12 +653,11 @@ __global__ void __launch_bounds__(256) ibm_spread_particle_kernel(ParticleSpread
         if (lane < 12) phi = peskin_r<R>(R((lane & 3) - 1) - E[lane >> 2]);
         const R w = __shfl_sync(0xffffffffu, phi, kx) * __shfl_sync(0xffffffffu, phi, 4 + ky) *
                     __shfl_sync(0xffffffffu, phi, 8 + kz);
-        // box-local node index; the marker base is wrapped, so unwrap the difference
-        int i0 = a.mB[3 * l] + kx - o0, i1 = a.mB[3 * l + 1] + ky - o1, i2 = a.mB[3 * l + 2] + kz - o2;
-        i0 = i0 < -a.nx / 2 ? i0 + a.nx : (i0 >= a.nx / 2 ? i0 - a.nx : i0);
-        i1 = i1 < -a.ny / 2 ? i1 + a.ny : (i1 >= a.ny / 2 ? i1 - a.ny : i1);
-        i2 = i2 < -a.nz / 2 ? i2 + a.nz : (i2 >= a.nz / 2 ? i2 - a.nz : i2);
-        if (i0 < 0 || i1 < 0 || i2 < 0 || i0 >= W || i1 >= W || i2 >= W) continue;
+        // box-local node index modulo the grid, for the marker base is wrapped:
+        // a box may be wider than half the grid (or than the grid itself)
+        const int i0 = pwrap(a.mB[3 * l] + kx - o0, a.nx), i1 = pwrap(a.mB[3 * l + 1] + ky - o1, a.ny),
+                  i2 = pwrap(a.mB[3 * l + 2] + kz - o2, a.nz);
+        if (i0 >= W || i1 >= W || i2 >= W) continue;
         const int bi = i0 + W * (i1 + W * i2);
         atomicAdd(&box[3 * bi], mFr[3 * l] * w);
         atomicAdd(&box[3 * bi + 1], mFr[3 * l + 1] * w);
