@@ -333,7 +333,6 @@ struct SiteArgs {
     int nx, ny, nz;
     long long N;
     double pcx, pcy, pR;
-    int mode;
     long long *blk_sites, *blk_links;
     long long *counts;
     int *site_cell, *site_first;
@@ -378,15 +377,11 @@ __device__ __forceinline__ void cell_info(const SiteArgs &a, long long c, bool &
     mask = 0;
     if (c >= a.N) return;
     const uint8_t fl = a.flags[c];
-    if (a.mode == 1) {
-        if (fl & FL_SOLID) return;
-        const unsigned zq = a.dxy.div((unsigned)c), rem = (unsigned)c - zq * (unsigned)(a.nx * a.ny);
-        const unsigned yq = a.dx.div(rem);
-        mask = solid_mask(a, (int)(rem - yq * (unsigned)a.nx), (int)yq, (int)zq);
-        site = mask != 0;
-    } else {
-        site = (fl & FL_SUP) != 0;
-    }
+    if (fl & FL_SOLID) return;
+    const unsigned zq = a.dxy.div((unsigned)c), rem = (unsigned)c - zq * (unsigned)(a.nx * a.ny);
+    const unsigned yq = a.dx.div(rem);
+    mask = solid_mask(a, (int)(rem - yq * (unsigned)a.nx), (int)yq, (int)zq);
+    site = mask != 0;
 }
 
 // The CPT = 4 consecutive cells of a thread at once (mode 1, nx a multiple
@@ -496,7 +491,7 @@ __global__ void __launch_bounds__(CT) site_count_kernel(SiteArgs a) {
     __shared__ long long sh[CT / 32];
     const long long base = (long long)blockIdx.x * TILE + (long long)threadIdx.x * CPT;
     long long ns = 0, nl = 0;
-    if (a.mode == 1 && a.nx % 4 == 0 && base < a.N) {
+    if (a.nx % 4 == 0 && base < a.N) {
         unsigned v[19], any = 0;
         link_bits4(a, base, v);
 #pragma unroll
@@ -706,7 +701,7 @@ __global__ void __launch_bounds__(CT) site_emit_kernel(SiteArgs a) {
     bool site[CPT];
     unsigned mask[CPT];
     long long ns = 0, nl = 0;
-    if (a.mode == 1 && a.nx % 4 == 0 && base < a.N) {
+    if (a.nx % 4 == 0 && base < a.N) {
         cell_info4(a, base, site, mask);
     } else {
         for (int k = 0; k < CPT; k++) cell_info(a, base + k, site[k], mask[k]);
@@ -726,27 +721,21 @@ __global__ void __launch_bounds__(CT) site_emit_kernel(SiteArgs a) {
         // otherwise the status word reports the overflow and the cell keeps
         // no BND flag, so no kernel reads a slot or link that was not written
         const bool fits = site[k] && s0 < a.max_sites && l0 + nl_c <= a.max_links;
-        if (a.mode == 1) {
-            const uint8_t fl = a.flags[c];
-            const uint8_t nf = fits ? (uint8_t)(fl | FL_BND) : (uint8_t)(fl & ~FL_BND);
-            if (nf != fl) a.flags[c] = nf;
-        }
+        const uint8_t fl = a.flags[c];
+        const uint8_t nf = fits ? (uint8_t)(fl | FL_BND) : (uint8_t)(fl & ~FL_BND);
+        if (nf != fl) a.flags[c] = nf;
         if (!site[k]) continue;
         if (fits) {
             a.site_cell[s0] = (int)c;
             a.site_first[s0] = (int)l0;
             a.site_mask[s0] = mask[k];
             a.aux[c] = (int)s0;
-            if (a.mode == 1) {
-                // cell and direction only; link_geom_kernel fills in q, owner and scheme
-                long long lk = l0;
-                for (unsigned mm = mask[k] & ~1u; mm; mm &= mm - 1u, lk++) {  // set bits, ascending
-                    a.link_cell[lk] = (int)c;
-                    a.link_dir[lk] = (int8_t)(__ffs(mm) - 1);
-                }
+            // cell and direction only; link_geom_kernel fills in q, owner and scheme
+            long long lk = l0;
+            for (unsigned mm = mask[k] & ~1u; mm; mm &= mm - 1u, lk++) {  // set bits, ascending
+                a.link_cell[lk] = (int)c;
+                a.link_dir[lk] = (int8_t)(__ffs(mm) - 1);
             }
-        } else if (a.mode == 2) {
-            a.aux[c] = -1;  // support cell without a slot: skipped by every reader
         }
         l0 += nl_c;
         s0++;
@@ -871,6 +860,8 @@ __device__ __forceinline__ void load_flags16(const SiteArgs &a, long long base, 
     }
 }
 
+// FLAG: FL_BND (cells with links, their masks in aux) or FL_SUP (support cells, no links)
+template <uint8_t FLAG>
 __global__ void __launch_bounds__(CT) bnd_count_kernel(SiteArgs a) {
     __shared__ long long sh[CT / 32];
     const long long base = (long long)blockIdx.x * VTILE + (long long)threadIdx.x * VT;
@@ -880,14 +871,14 @@ __global__ void __launch_bounds__(CT) bnd_count_kernel(SiteArgs a) {
         load_flags16(a, base, f);
 #pragma unroll
         for (int k = 0; k < VT; k++)
-            if (f[k] & FL_BND) {
+            if (f[k] & FLAG) {
                 ns++;
-                nl += __popc((unsigned)a.aux[base + k]);
+                if (FLAG == FL_BND) nl += __popc((unsigned)a.aux[base + k]);
             }
     }
-    long long ts, tl;
+    long long ts, tl = 0;
     block_exclusive_scan<long long>(ns, sh, ts);
-    block_exclusive_scan<long long>(nl, sh, tl);
+    if (FLAG == FL_BND) block_exclusive_scan<long long>(nl, sh, tl);
     if (threadIdx.x == 0) {
         a.blk_sites[blockIdx.x] = ts;
         a.blk_links[blockIdx.x] = tl;
@@ -940,6 +931,31 @@ __global__ void __launch_bounds__(CT) bnd_emit_kernel(SiteArgs a) {
     }
 }
 
+// the support cells in cell order: cell of a site, site of a cell
+__global__ void __launch_bounds__(CT) sup_emit_kernel(SiteArgs a) {
+    __shared__ long long sh[CT / 32];
+    const long long base = (long long)blockIdx.x * VTILE + (long long)threadIdx.x * VT;
+    unsigned sup = 0;
+    if (base < a.N) {
+        uint8_t f[VT];
+        load_flags16(a, base, f);
+#pragma unroll
+        for (int k = 0; k < VT; k++)
+            if (f[k] & FL_SUP) sup |= 1u << k;
+    }
+    long long ts;
+    long long s0 = block_exclusive_scan<long long>((long long)__popc(sup), sh, ts) + a.blk_sites[blockIdx.x];
+    for (; sup; sup &= sup - 1, s0++) {
+        const long long c = base + __ffs(sup) - 1;
+        if (s0 < a.max_sites) {
+            a.site_cell[s0] = (int)c;
+            a.aux[c] = (int)s0;
+        } else {
+            a.aux[c] = -1;  // a support cell without a slot is skipped by every reader
+        }
+    }
+}
+
 // Build the compact site list. mode 1: IBB boundary cells and their links
 // (BND flags refreshed); mode 2: IBM support cells (SUP flags set before).
 cudaError_t build_sites(Ctx &c, int mode) {
@@ -956,7 +972,6 @@ cudaError_t build_sites(Ctx &c, int mode) {
     a.pcx = c.pipe_cx;
     a.pcy = c.pipe_cy;
     a.pR = c.pipe_R;
-    a.mode = mode;
     a.blk_sites = c.blk_sites;
     a.blk_links = c.blk_links;
     a.counts = c.d_counts;
@@ -994,12 +1009,18 @@ cudaError_t build_sites(Ctx &c, int mode) {
         const int T = 2 * ((int)ceil(c.max_radius) + 2) + 4;
         if ((long long)T * T * T <= 32768) bnd_mark_tile_kernel<<<c.np, 256, (size_t)T * T * T, c.stream>>>(a, T);
         else bnd_mark_kernel<<<c.np, 256, 0, c.stream>>>(a);
-        bnd_count_kernel<<<nblk, CT, 0, c.stream>>>(a);
+        bnd_count_kernel<FL_BND><<<nblk, CT, 0, c.stream>>>(a);
         site_scan_kernel<<<1, ST, 0, c.stream>>>(a, nblk);
         bnd_emit_kernel<<<nblk, CT, 0, c.stream>>>(a);
+    } else if (mode == 2) {
+        const int nblk = (int)((c.N + VTILE - 1) / VTILE);
+        count_launch(c, G_GEOM, 3);
+        bnd_count_kernel<FL_SUP><<<nblk, CT, 0, c.stream>>>(a);
+        site_scan_kernel<<<1, ST, 0, c.stream>>>(a, nblk);
+        sup_emit_kernel<<<nblk, CT, 0, c.stream>>>(a);
     } else {
         const int nblk = (int)((c.N + TILE - 1) / TILE);
-        count_launch(c, G_GEOM, mode == 1 ? 4 : 3);
+        count_launch(c, G_GEOM, 4);
         site_count_kernel<<<nblk, CT, 0, c.stream>>>(a);
         site_scan_kernel<<<1, ST, 0, c.stream>>>(a, nblk);
         site_emit_kernel<<<nblk, CT, 0, c.stream>>>(a);
