@@ -61,10 +61,22 @@ __global__ void mlp_pack2_kernel(const float *w, __nv_bfloat16 *pk) {
 
 // sum the per-block gradients in block order; Adam on the FP32 master
 __global__ void mlp_adam_kernel(float *w, float *m, float *v, const float *gpart, int nblk, int step, float lr,
-                                float b1, float b2, float eps, __nv_bfloat16 *pk, float *gout) {
+                                float b1, float b2, float eps, __nv_bfloat16 *pk, float *gout, const float *lpart,
+                                double *loss) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= NPARAM) return;
+    if (p >= NPARAM) {
+        // the last thread adds the batch's loss partials to the epoch's sum,
+        // in block order (reading them back after each batch cost a stop of
+        // the stream per batch)
+        if (loss && threadIdx.x == blockDim.x - 1 && blockIdx.x == gridDim.x - 1) {
+            double l = *loss;
+            for (int b = 0; b < nblk; b++) l += lpart[b];
+            *loss = l;
+        }
+        return;
+    }
     float g = 0.f;
+#pragma unroll 8
     for (int b = 0; b < nblk; b++) g += gpart[(size_t)b * NPARAM + p];
     if (gout) {
         gout[p] = g;
@@ -91,6 +103,7 @@ struct MlpWs {
     __nv_bfloat16 *pk;
     float *m, *v, *gpart, *lpart;
     int *err;  // set by the tensor-core forward when a wait runs out
+    double *loss;  // sum of the last epoch's squared errors (in the pad behind err)
 };
 size_t mlp_ws_bytes() {
     return (((size_t)PK_TOTAL * 2 + 255) / 256) * 256 + 2 * (((size_t)NPARAM * 4 + 255) / 256) * 256 +
@@ -111,6 +124,7 @@ MlpWs mlp_ws(void *ws) {
     W.lpart = (float *)(b + o);
     o += 256 * 4;
     W.err = (int *)(b + o);
+    W.loss = (double *)(((uintptr_t)(b + o + 64) + 7) / 8 * 8);
     return W;
 }
 cudaError_t mlp_pack(const float *w, __nv_bfloat16 *pk, cudaStream_t s) {
@@ -159,7 +173,7 @@ lbm_status lbm_mlp_loss_grad(const float *X_dev, const float *T_dev, long long n
         mlp_train_tc(X_dev, T_dev, 0, n, w_dev, W.pk, W.gpart, W.lpart, TRAIN_BLOCKS, W.err, s, &nblk) != cudaSuccess)
         return LBM_ECUDA;
     mlp_adam_kernel<<<(NPARAM + 255) / 256, 256, 0, s>>>(nullptr, nullptr, nullptr, W.gpart, nblk, 1, 0.f, 0.f, 0.f,
-                                                         0.f, W.pk, grad_dev);
+                                                         0.f, W.pk, grad_dev, nullptr, nullptr);
     if (cudaGetLastError() != cudaSuccess) return LBM_ECUDA;
     float lp[TRAIN_BLOCKS];
     int err = 0;
@@ -187,11 +201,11 @@ lbm_status lbm_mlp_train(const float *X_dev, const float *T_dev, long long n, in
         cudaMemsetAsync(W.v, 0, sizeof(float) * NPARAM, s) != cudaSuccess || mlp_pack(w_dev, W.pk, s) != cudaSuccess)
         return LBM_ECUDA;
     int step = 0;
+    static_assert(NPARAM % 256 != 0, "the last block of the Adam kernel has a spare thread");
     double epoch_loss = 0.0;
-    std::vector<float> lp(TRAIN_BLOCKS);
+    if (cudaMemsetAsync(W.loss, 0, sizeof(double), s) != cudaSuccess) return LBM_ECUDA;
     for (int ep = 0; ep < epochs; ep++) {
         const bool last = ep == epochs - 1;
-        epoch_loss = 0.0;
         for (long long s0 = 0; s0 < n; s0 += batch) {
             const long long s1 = s0 + batch < n ? s0 + batch : n;
             int nblk = 0;
@@ -200,18 +214,14 @@ lbm_status lbm_mlp_train(const float *X_dev, const float *T_dev, long long n, in
                 return LBM_ECUDA;
             step++;
             mlp_adam_kernel<<<(NPARAM + 255) / 256, 256, 0, s>>>(w_dev, W.m, W.v, W.gpart, nblk, step, (float)lr,
-                                                                 0.9f, 0.999f, 1e-8f, W.pk, nullptr);
-            if (last) {
-                if (cudaMemcpyAsync(lp.data(), W.lpart, sizeof(float) * nblk, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-                    cudaStreamSynchronize(s) != cudaSuccess)
-                    return LBM_ECUDA;
-                for (int b = 0; b < nblk; b++) epoch_loss += lp[b];
-            }
+                                                                 0.9f, 0.999f, 1e-8f, W.pk, nullptr, W.lpart,
+                                                                 last ? W.loss : nullptr);
         }
     }
     if (cudaGetLastError() != cudaSuccess) return LBM_ECUDA;
     int err = 0;
     if (cudaMemcpyAsync(&err, W.err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaMemcpyAsync(&epoch_loss, W.loss, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return LBM_ECUDA;
     if (err) return LBM_ETIMEOUT;  // a tensor-core wait ran out
