@@ -557,7 +557,7 @@ __global__ void clear_sup_kernel(uint8_t *flags, long long N) {
 // floor(X) + ceil(R) + 2 in shared memory (a word per x-row, W <= 32), then
 // one flag update per four cells. Marker by marker and cell by cell on the
 // grid, with the overlap test in FP64 throughout, the two passes took 107 and
-// 189 us at 256^3 with 2000 spheres; this takes 48.
+// 189 us at 256^3 with 2000 spheres; this takes 43.
 __global__ void __launch_bounds__(256) mark_support_kernel(uint8_t *flags, const double *mX, const int *m_first,
                                                            const double *X, const double *R, int nx, int ny, int nz) {
     __shared__ unsigned row[32 * 32];
@@ -887,7 +887,7 @@ __global__ void __launch_bounds__(256) ibm_spread_particle_kernel(ParticleSpread
 // node visits per marker. With a warp per marker reading 64 nodes through the
 // cell index (780 MB from L2 per pass) and a second kernel spreading, a pass
 // took 147 + 170 us at 256^3 with 2000 spheres of radius 4; a warp per marker
-// on the box 215; this takes 121.
+// on the box 215; this takes 118.
 //
 // FP32: the box of forces is in integers, scaled by the power of two that
 // puts the largest |F_l dV_l| of the particle at 2^28 .. 2^29. Shared-memory
