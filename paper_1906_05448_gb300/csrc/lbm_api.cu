@@ -1,6 +1,7 @@
 // C ABI of the library (declared in include/lbm.h): workspace layout, set-up
 // of the geometry, the per-step kernel sequence and host-side checks.
 #include "lbm_internal.cuh"
+#include "spectra_scratch.h"
 
 #include <cmath>
 #include <ctime>

@@ -193,7 +193,6 @@ cudaError_t launch_q27_macro(Ctx &c, float4 *rec);
 void q27_pipe_colmask(const Ctx &c, std::vector<unsigned> &mask);
 cudaError_t launch_q27_coef(Ctx &c);
 size_t tke_budget_scratch_bytes(int nbins);
-size_t spectrum_scratch_bytes(long long N, int nbins);
 cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *out);
 cudaError_t closure_samples(Ctx &c, double u_scale, float *X, int *cells, long long cap, long long *n_out);
 cudaError_t closure_targets(Ctx &c, const int *cells, long long n, double g_scale, float *T);

@@ -30,12 +30,11 @@
 // two complex fields (16 bytes per cell of its 38 or more) and the
 // per-block sums, so the entry point needs no memory of its own.
 #include "lbm_internal.cuh"
+#include "spectra_scratch.h"
 
 #include <vector>
 
 namespace lbmgb {
-
-constexpr int SP_BLOCKS = 304;  // blocks of the z pass that own a set of bins, at most
 
 // lines per block: runs of 128 bytes, and at most 1024 threads of 8 points
 __host__ __device__ constexpr int fft_lines(int logn) { return logn <= 8 ? 16 : 8; }
@@ -282,9 +281,9 @@ static cudaError_t spectrum_t(Ctx &c, int nbins, float2 *field, double *part, do
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fft_z_bins_kernel<LOGN>, TZ, smz);
-    blocks = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
-    if (blocks > SP_BLOCKS) blocks = SP_BLOCKS;
-    if (blocks > n * (n / 2) / (L / 2)) blocks = n * (n / 2) / (L / 2);
+    blocks = spectrum_blocks((size_t)c.q * (size_t)c.N * storage_bytes(c.storage), c.N, n, L / 2, nbins,
+                             (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1));
+    if (blocks < 1) return cudaErrorInvalidValue;  // refused by the caller already
     count_launch(c, G_STATS, 3);
     fft_x_kernel<LOGN><<<dim3((unsigned)(n * n / Lx), 2), TB, smx, c.stream>>>(c.u_f, field, c.N);
     fft_y_kernel<LOGN><<<dim3((unsigned)(n * n / L), 2), TZ, smy, c.stream>>>(field, c.N);
@@ -299,7 +298,7 @@ cudaError_t run_spectrum(Ctx &c, int flags, int nbins, double *E, double *D) {
     while ((1 << logn) < n) logn++;
     const long long N = c.N;
     float2 *field = (float2 *)c.fB;
-    double *part = (double *)((char *)c.fB + 2 * (size_t)N * sizeof(float2));
+    double *part = (double *)((char *)c.fB + spectrum_bins_offset(N));
     if ((e = launch_macro(c, 0)) != cudaSuccess) return e;
     const int ibm = c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B;
     if (!(ibm && (flags & LBM_STATS_UNMASK)))
@@ -331,11 +330,6 @@ cudaError_t run_spectrum(Ctx &c, int flags, int nbins, double *E, double *D) {
         D[k] = sd;
     }
     return cudaSuccess;
-}
-
-// what the call asks of the idle population buffer (a limit of the ABI)
-size_t spectrum_scratch_bytes(long long N, int nbins) {
-    return ((size_t)N * sizeof(float2) + 255) / 256 * 256 + sizeof(double) * 2 * (size_t)nbins * 304;
 }
 
 }  // namespace lbmgb

@@ -106,3 +106,28 @@ def test_every_transform_length_on_noise(lbm, n):
     okD, eD = close(Dg, Do)
     assert okE and okD, (eE, eD)
     g.close()
+
+
+@pytest.mark.parametrize("storage", ["f16s", "bf16s"])
+def test_most_bins_of_a_small_cube_stay_in_the_scratch(lbm, storage):
+    """64^3 in 16-bit storage with the most bins the call accepts and no slack
+    behind the populations: the sums match the oracle, and neither the flags
+    nor the next steps notice that the statistics were taken."""
+    n, nb = 64, 1616
+    u = workloads.noise_velocity((n, n, n), 0.02, seed=6)
+    pair = [lbm.Lattice(n, n, n, 0.6, storage=storage, max_sites=1, max_links=1, max_markers=1) for _ in range(2)]
+    for g in pair:
+        g.init_velocity(u)
+    E, D = pair[0].spectrum(nb)
+    Eo, Do = spectra.spectra(pair[1].macro()[1], n, 0.1 / 3, nb)
+    okE, eE = close(E, Eo)
+    okD, eD = close(D, Do)
+    assert okE and okD, (eE, eD)
+    for g in pair:
+        assert not g.flags().any()
+        g.step(3)
+    assert np.array_equal(pair[0].populations(), pair[1].populations())
+    with pytest.raises(lbm.LbmError):
+        pair[0].spectrum(nb + 1)
+    for g in pair:
+        g.close()
