@@ -12,25 +12,29 @@
 // the kernels here convert.
 #pragma once
 
+#include "column_index.h"
 #include "lbm_internal.cuh"
 
 namespace lbmgb {
 
 // Addresses of a D3Q19 sweep on columns: the pull of direction i for element
-// e = z + zp * column of a plane is Ap[i][e], its store Bp[i][e] (one
+// e = z + zp * column of a plane is Ap[i][e + bias], its store Bp[i][e] (one
 // address operation per access); pulls across the ends of z, and of x and y
-// where columns on the box faces are swept, add a correction.
+// where columns on the box faces are swept, add a correction
+// (column_index.h).
 struct ColumnPtrs {
-    const void *Ap[19];  // A + i Np - (c_z + zp (c_x + nx c_y))
+    const void *Ap[19];  // A + i Np - (c_z + zp (c_x + nx c_y)) - bias
     void *Bp[19];        // B + i Np
     int nx, ny, nz, zp;
+    unsigned bias;
     FastDiv fd_nx;
 };
 
 inline void column_ptrs(const Ctx &c, ColumnPtrs &p) {
     const long long sb = (long long)storage_bytes(c.storage);
+    p.bias = column_bias(c.nx, c.zp);
     for (int i = 0; i < 19; i++) {
-        const long long off = cz(i) + (long long)c.zp * (cx(i) + (long long)c.nx * cy(i));
+        const long long off = cz(i) + (long long)c.zp * (cx(i) + (long long)c.nx * cy(i)) + p.bias;
         p.Ap[i] = (const void *)((const char *)c.fA + sb * (i * c.Np - off));
         p.Bp[i] = (void *)((char *)c.fB + sb * (i * c.Np));
     }
@@ -45,24 +49,15 @@ inline void column_ptrs(const Ctx &c, ColumnPtrs &p) {
 // column may lie on an x or y face of the box
 template <typename T, bool WRAP, typename R, typename Ld>
 __device__ __forceinline__ void column_pull(R g[19], const ColumnPtrs &p, int col, int z, Ld ld) {
-    const int e = col * p.zp + z;
-    const int zlo = z == 0 ? p.nz : 0, zhi = z == p.nz - 1 ? p.nz : 0;
-    int xlo = 0, xhi = 0, ylo = 0, yhi = 0;
+    const unsigned e = (unsigned)(col * p.zp + z) + p.bias;
+    int x = 1, y = 1;  // no face unless WRAP
     if constexpr (WRAP) {
-        const int y = (int)p.fd_nx.div((unsigned)col), x = col - y * p.nx;
-        const int row = p.nx * p.zp;
-        xlo = x == 0 ? row : 0;
-        xhi = x == p.nx - 1 ? row : 0;
-        ylo = y == 0 ? row * p.ny : 0;
-        yhi = y == p.ny - 1 ? row * p.ny : 0;
+        y = (int)p.fd_nx.div((unsigned)col);
+        x = col - y * p.nx;
     }
+    const ColumnWrap w = column_wrap(x, y, z, WRAP ? p.nx : 4, WRAP ? p.ny : 4, p.nz, p.zp);
 #pragma unroll
-    for (int i = 0; i < 19; i++) {
-        int o = e + (cz(i) > 0 ? zlo : 0) - (cz(i) < 0 ? zhi : 0);
-        if constexpr (WRAP)
-            o += (cx(i) > 0 ? xlo : 0) - (cx(i) < 0 ? xhi : 0) + (cy(i) > 0 ? ylo : 0) - (cy(i) < 0 ? yhi : 0);
-        g[i] = ld((const T *)p.Ap[i] + o);
-    }
+    for (int i = 0; i < 19; i++) g[i] = ld((const T *)p.Ap[i] + column_offset(e, w, cx(i), cy(i), cz(i)));
 }
 
 constexpr int COL_TILE = 32;  // x by z tile of the conversions, at one y
