@@ -332,9 +332,10 @@ __global__ void __launch_bounds__(256, q27_min_blocks(S)) q27_columns_kernel(Q27
             const int j = q27opp(i);
             const Q27Coef<R> k = kc[i];
             const R fi = Store<S>::ld(A + (i * N + (size_t)c));  // f*_i(x_f)
-            // q < 1/2: f*_i(x_f - c_i), the regular pull of direction i
-            // (weight 0 for the halfway fallback); q >= 1/2: f*_j(x_f)
-            const R second = ((h >> i) & 1u) ? Store<S>::ld(A + (j * N + (size_t)c)) : g[i];
+            // q < 1/2: f*_i(x_f - c_i), the regular pull of direction i;
+            // q >= 1/2: f*_j(x_f). The halfway fallback (weight 0) has no
+            // second value: its pull is a solid cell's, which may hold anything
+            const R second = ((h >> i) & 1u) ? Store<S>::ld(A + (j * N + (size_t)c)) : (k.k2 == R(0) ? R(0) : g[i]);
             // the bounce-back acts on f, the storage holds g = f - w with w_i = w_j
             g[j] = k.k1 * fi + k.k2 * second;
         }

@@ -135,3 +135,29 @@ def test_d3q27_refuses_what_it_does_not_build(lbm):
     g.close()
     with pytest.raises(ValueError):
         lbm.Lattice(16, 16, 16, 0.6, storage=lbm.F16S, lattice=27)
+
+
+@pytest.mark.parametrize("lattice,storage", [(27, "f64"), (27, "f32"), (19, "f64"), (19, "f32"), (19, "f16s"),
+                                             (19, "bf16s")])
+def test_what_solid_cells_hold_never_reaches_the_fluid(lbm, lattice, storage):
+    """A wall with the schemes for walls one cell apart (the 6.4 radius in a
+    16 x 15 section): a context whose solid cells hold NaN steps the fluid bit
+    for bit as one whose solid cells hold the state at rest."""
+    nx, ny, nz, R = 16, 15, 5, 6.4
+    u = workloads.pipe_velocity(nx, ny, nz, R, 0.02, perturbation=0.1, seed=3)
+    runs = []
+    for fill in (None, np.nan):
+        g = lbm.Lattice(nx, ny, nz, 0.62, force=(0.0, 0.0, 3e-6), storage=storage, lattice=lattice)
+        g.init_velocity(u)
+        g.set_pipe(R)
+        g.step(1, lbm.BC_IBB)
+        solid = (g.flags() & 1) != 0 if lattice == 19 else q27.pipe_solid(nx, ny, nz, R).reshape(-1)
+        f = g.populations()
+        if fill is not None:
+            f[:, solid] = fill
+        g.set_populations(f)
+        g.step(3, lbm.BC_IBB)
+        runs.append((g.populations()[:, ~solid], g.stats()["kinetic_energy"]))
+        g.close()
+    assert np.array_equal(runs[0][0], runs[1][0])
+    assert np.isfinite(runs[1][1]) and runs[0][1] == runs[1][1]
