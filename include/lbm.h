@@ -253,7 +253,9 @@ lbm_status lbm_tke_budget(lbm_ctx *ctx, int flags, int nbins, double *out);
 #define LBM_FIELD_IBM_FORCE 4 /* 3N doubles: IBM force of the last step */
 
 /* Copy a field to host memory dst of `bytes` bytes. Syncs. Populations of
- * solid cells under IBB are undefined; rho and u report 0 there. */
+ * solid cells under IBB are undefined (they are never swept, and calls that
+ * name the population buffer as their scratch leave its bytes there); rho
+ * and u report 0 there, on D3Q27 the state at rest: rho = 1, u = -F/2. */
 lbm_status lbm_get_field(lbm_ctx *ctx, int which, void *dst, size_t bytes);
 
 /* Number of IBB boundary links of the current geometry. */

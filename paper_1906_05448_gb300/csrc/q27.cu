@@ -87,11 +87,14 @@ __global__ void q27_macro_kernel(const void *A, float4 *rec, double *rho_o, doub
     u_o[2 * N + c] = double((j2 - R(0.5) * R(F2)) * ir);
 }
 
-// the same on the column layout (columns.cuh): read along z, written along x
+// the same on the column layout (columns.cuh): read along z, written along x.
+// Solid columns are never swept and their populations are undefined (calls
+// that use the idle buffer as scratch leave their bytes there): they report
+// the state at rest, g = 0.
 template <int S>
-__global__ void __launch_bounds__(256) q27_column_macro_kernel(const void *A, float4 *rec, double *rho_o, double *u_o, int nx, int ny,
-                                                               int nz, int zp, long long N, long long Np, double F0,
-                                                               double F1, double F2) {
+__global__ void __launch_bounds__(256) q27_column_macro_kernel(const void *A, const unsigned *colmask, float4 *rec, double *rho_o,
+                                                               double *u_o, int nx, int ny, int nz, int zp, long long N,
+                                                               long long Np, double F0, double F1, double F2) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
     struct V {
@@ -104,13 +107,15 @@ __global__ void __launch_bounds__(256) q27_column_macro_kernel(const void *A, fl
             [&](int x, int z) {
                 const T *P = (const T *)A + (size_t)(x + nx * y) * zp + z;
                 R r = R(0), j0 = R(0), j1 = R(0), j2 = R(0);
+                if (!(__ldg(colmask + x + nx * y) & 1u)) {
 #pragma unroll
-                for (int i = 0; i < Q27; i++) {
-                    const R g = Store<S>::ld(P + i * Np);
-                    r += g;
-                    j0 += g * R(q27x(i));
-                    j1 += g * R(q27y(i));
-                    j2 += g * R(q27z(i));
+                    for (int i = 0; i < Q27; i++) {
+                        const R g = Store<S>::ld(P + i * Np);
+                        r += g;
+                        j0 += g * R(q27x(i));
+                        j1 += g * R(q27y(i));
+                        j2 += g * R(q27z(i));
+                    }
                 }
                 const R rho = R(1) + r, ir = R(1) / rho;
                 return V{rho, (j0 - R(0.5) * R(F0)) * ir, (j1 - R(0.5) * R(F1)) * ir, (j2 - R(0.5) * R(F2)) * ir};
@@ -481,8 +486,8 @@ cudaError_t launch_q27_macro(Ctx &c, float4 *rec) {
     count_launch(c, G_STATS);
     if (c.zlay) {
 #define MK(S)                                                                                                      \
-    q27_column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, rec, c.rho_f, c.u_f, c.nx, c.ny, c.nz, c.zp, c.N, \
-                                                                    c.Np, c.F[0], c.F[1], c.F[2])
+    q27_column_macro_kernel<S><<<column_tiles(c), 256, 0, c.stream>>>(c.fA, c.q27_colmask, rec, c.rho_f, c.u_f, c.nx, c.ny, c.nz, \
+                                                                    c.zp, c.N, c.Np, c.F[0], c.F[1], c.F[2])
         if (c.storage == LBM_F64) MK(LBM_F64);
         else MK(LBM_F32);
 #undef MK

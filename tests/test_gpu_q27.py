@@ -161,3 +161,35 @@ def test_what_solid_cells_hold_never_reaches_the_fluid(lbm, lattice, storage):
         g.close()
     assert np.array_equal(runs[0][0], runs[1][0])
     assert np.isfinite(runs[1][1]) and runs[0][1] == runs[1][1]
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_solid_cells_report_rest_after_statistics(lbm, storage, tmp_path):
+    """Calls that use the idle population buffer (statistics, profiles, the
+    budget, a checkpoint) do not show in the fields of later steps: solid
+    cells report the state at rest, fluid cells what an undisturbed run does."""
+    nx, ny, nz, R, F = 26, 25, 9, 11.3, (0.0, 0.0, 4e-6)
+    solid = q27.pipe_solid(nx, ny, nz, R).reshape(-1)
+    u = workloads.pipe_velocity(nx, ny, nz, R, 0.02, perturbation=0.1, seed=4)
+    runs = []
+    for disturbed in (False, True):
+        g = lbm.Lattice(nx, ny, nz, 0.6, force=F, storage=storage, lattice=27)
+        g.init_velocity(u)
+        g.set_pipe(R)
+        for _ in range(3):
+            g.step(1, lbm.BC_IBB)
+            if disturbed:
+                g.stats()
+                g.pipe_profiles(2)
+                g.tke_budget(2)
+                g.checkpoint(str(tmp_path / "c.bin"))
+                g.stats()
+        rho, v = g.macro()
+        rest = np.array(F) * (-0.5 if storage == "f64" else np.float32(-0.5))
+        rest = rest.astype(np.float32 if storage == "f32" else np.float64)
+        assert np.all(rho[solid] == 1.0)
+        assert np.all(v[:, solid] == rest.astype(np.float64)[:, None])
+        runs.append((rho, v, g.populations()[:, ~solid]))
+        g.close()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
