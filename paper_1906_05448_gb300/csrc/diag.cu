@@ -323,8 +323,8 @@ constexpr int ST_TB = 128;   // threads: 32 x 4 columns
 constexpr int ST_RUN = 64;   // planes per tile
 
 struct StatsArgs {
-    const double *u, *rho;  // FP64 fields; with records: u holds the low parts of masked particle cells' velocities
-    const float4 *rec;      // FP32 records, or null
+    const double *u, *rho;  // FP64 fields
+    const float4 *rec, *low;  // or FP32 records, and the low parts of masked particle cells' velocities
     const uint8_t *flags;
     const unsigned long long *near_key;
     const double *X, *R;
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(ST_TB) stats_kernel(StatsArgs a) {
         const int oxm = x == 0 ? nx - 1 : -1, oxp = x == nx - 1 ? 1 - nx : 1;
         const long long oym = y == 0 ? (long long)nx * (ny - 1) : -nx, oyp = y == ny - 1 ? -(long long)nx * (ny - 1) : nx;
         const double *u = a.u + c;
-        const float4 *rec = a.rec + c, *lo = (const float4 *)a.u + c;
+        const float4 *rec = a.rec + c, *lo = a.low + c;
         double um[3], uc[3];
         float4 fm = make_float4(0.f, 0.f, 0.f, 0.f), fc = fm;
         if constexpr (REC) {
@@ -727,8 +727,8 @@ static cudaError_t mask_cells(Ctx &c, double *part, float4 *rec = nullptr) {
     if (c.np == 0 && !c.has_pipe) return cudaSuccess;  // no solid cell
     const FastDiv fdx((unsigned)c.nx), fdxy((unsigned)(c.nx * c.ny));
     if (rec)
-        mask_kernel<true><<<mask_blocks(c), SB, 0, c.stream>>>(rec, c.u_f, c.rho_f, c.flags, c.owner, c.X, c.U, c.W, c.nx,
-                                                               c.ny, c.nz, fdx, fdxy, c.N, part);
+        mask_kernel<true><<<mask_blocks(c), SB, 0, c.stream>>>(rec, (double *)(rec + c.N), nullptr, c.flags, c.owner, c.X,
+                                                               c.U, c.W, c.nx, c.ny, c.nz, fdx, fdxy, c.N, part);
     else
         mask_kernel<false><<<mask_blocks(c), SB, 0, c.stream>>>(nullptr, c.u_f, c.rho_f, c.flags, c.owner, c.X, c.U, c.W,
                                                                 c.nx, c.ny, c.nz, fdx, fdxy, c.N, part);
@@ -899,11 +899,13 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
     const int ibb = c.armed_bc == LBM_BC_IBB;
     const int ibm = c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B;
     const bool closure = (flags & LBM_STATS_CLOSURE) && c.np > 0 && c.cl_ready && c.max_cl > 0 && c.q == 19;
-    // FP32 records of the fields (16 B per cell) in the population buffer that
-    // the next step overwrites (19 x 2 B per cell or more): all that 32- and
-    // 16-bit storage needs, and the closure's gather input
+    // FP32 records of the fields, 16 B per cell: all that 32- and 16-bit
+    // storage needs, and the closure's gather input. With such storage they
+    // lie in the place of the FP64 fields (rho_f and u_f, 32 B per cell
+    // together), the low parts of masked cells behind them; else in the
+    // population buffer that the next step overwrites.
     const bool rec = c.storage != LBM_F64;
-    float *u32 = rec || closure ? (float *)c.fB : nullptr;
+    float *u32 = rec ? (float *)c.rho_f : (closure ? (float *)c.fB : nullptr);
     if ((e = launch_macro(c, 0, u32, rec)) != cudaSuccess) return e;
     count_launch(c, G_STATS, 3);
     const bool mask = !(ibm && (flags & LBM_STATS_UNMASK));
@@ -941,7 +943,7 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
     if (mask && !(c.zlay && c.q == 19 && ibb))
         if ((e = mask_cells(c, solid_held ? c.partials : nullptr, rec ? (float4 *)u32 : nullptr)) != cudaSuccess) return e;
     const int mblk = solid_held && (c.np > 0 || c.has_pipe) ? mask_blocks(c) : 0;
-    StatsArgs a{c.u_f, c.rho_f, rec ? (const float4 *)u32 : nullptr, c.flags, c.near_key, c.X, c.R,
+    StatsArgs a{c.u_f, c.rho_f, rec ? (const float4 *)u32 : nullptr, rec ? (const float4 *)u32 + c.N : nullptr, c.flags, c.near_key, c.X, c.R,
                 c.same_radius ? 20.0f / (float)c.max_radius : 0.f, eps_o, c.nx, c.ny, c.nz, c.N, nu, c.has_pipe, ibb, !mask,
                 c.partials, bpart};
     const long long tiles = (long long)((c.nx + 31) / 32) * ((c.ny + 3) / 4) * ((c.nz + ST_RUN - 1) / ST_RUN);

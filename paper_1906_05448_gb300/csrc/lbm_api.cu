@@ -153,7 +153,7 @@ bool make_plan(const lbm_grid *g, Plan &P) {
     P.mE = L.take(24 * mm);
     P.mpid = L.take(4 * mm);
     P.mfirst = L.take(4 * (np + 1));
-    P.rho_f = L.take(8 * n);
+    P.rho_f = L.take(8 * n);  // these two stay next to each other (the statistics keep records across both)
     P.u_f = L.take(24 * n);
     P.partials = L.take(8 * stats_partials_doubles());
     P.near_key = L.take(8 * n);
@@ -1400,6 +1400,9 @@ lbm_status lbm_checkpoint(lbm_ctx *h, const char *path) {
         }
         CKS(dev_to_file(c, F.f, sF, 3 * arith_bytes(c) * (size_t)H.nsites, path));
     }
+    // the sweep of an IBB pipe never writes solid columns: none of the file's bytes stay there
+    if (c.zlay && c.armed_bc == LBM_BC_IBB)
+        CK(cudaMemsetAsync(c.fB, 0, (size_t)c.q * (size_t)c.Np * storage_bytes(c.storage), c.stream));
     if (H.nm > 0) CK(refresh_markers(c));
     if (H.nm > 0) CKS(dev_to_file(c, F.f, c.mFacc, sizeof(double) * 3 * (size_t)H.nm, path));
     if (c.cl_ready) CKS(dev_to_file(c, F.f, c.cl_w, sizeof(float) * LBM_MLP_NPARAM, path));

@@ -98,7 +98,7 @@ struct Ctx {
     void *pipe_it_w;  // arithmetic type of the storage
     int pipe_sp, pipe_max_ring;
     // statistics scratch
-    double *rho_f, *u_f, *partials;
+    double *rho_f, *u_f, *partials;  // u_f begins where rho_f ends (up to the alignment of the workspace's arrays)
     unsigned long long *near_key;  // nearest particle surface per cell (diag.cu)
     // status
     unsigned *d_status;

@@ -81,3 +81,31 @@ def test_stats_of_a_snapshot(lbm, storage, shape, R):
     assert raw["kinetic_energy"] == pytest.approx(ke.mean(), rel=1e-12)
     assert np.allclose(raw["momentum"], (u * rho).sum(1), rtol=1e-11, atol=0)
     g.close()
+
+
+@pytest.mark.parametrize("wall", ["pipe", "spheres"])
+@pytest.mark.parametrize("storage", ["f32", "f16s"])
+def test_statistics_leave_the_populations_alone(lbm, wall, storage, tmp_path):
+    """lbm_stats names no population buffer as its scratch: a run that takes
+    them (and, with a pipe, writes a checkpoint) between steps holds the same
+    populations in every cell, solid ones included, as one that does not."""
+    shape = (18, 21, 23)
+    nz, ny, nx = shape
+    u = workloads.noise_velocity(shape, 0.02, seed=4)
+    runs = []
+    for taken in (False, True):
+        g = lbm.Lattice(nx, ny, nz, 0.6, storage=storage, max_particles=1)
+        g.init_velocity(u)
+        if wall == "pipe":
+            g.set_pipe(9.3)
+        else:
+            g.add_spheres(np.array([[11.2, 9.7, 8.1]]), 4.0, U=np.full((1, 3), 0.01), W=np.zeros((1, 3)), fixed=True)
+        for _ in range(3):
+            g.step(1, lbm.BC_IBB)
+            if taken:
+                g.stats(lbm.STATS_BINS)
+                if wall == "pipe":
+                    g.checkpoint(str(tmp_path / "c.bin"))
+        runs.append(g.populations())
+        g.close()
+    assert np.array_equal(*runs)
