@@ -921,6 +921,7 @@ template <> struct SpreadSum<double> {
 // shared memory of a block: fields and forces of the box (z planes padded by
 // one cell, so that the four planes of a marker start on different banks),
 // its sites, per marker 12 kernel values, the force and the first node
+constexpr int PASS_SMEM = 220 * 1024;  // at most
 template <typename R>
 size_t pass_smem_bytes(int W, int markers) {
     const size_t nb = (size_t)W * (W * W + 1);
@@ -1103,11 +1104,13 @@ static cudaError_t ibm_passes_t(Ctx &c) {
     const int WB = 2 * (int)ceil(RLmax) + 4;
     const int mmax = RLmax > 0.0 ? (int)floor(M_PI / 3.0 * (12.0 * RLmax * RLmax + 1.0) + 0.5) : 0;  // as build_markers
     const size_t pass_smem = pass_smem_bytes<R>(WB, mmax);
-    const bool fused = !c.has_pipe && c.np > 0 && c.nm > 0 && pass_smem <= 220 * 1024 &&
+    const bool fused = !c.has_pipe && c.np > 0 && c.nm > 0 && pass_smem <= PASS_SMEM &&
                        WB <= std::min(c.nx, std::min(c.ny, c.nz));
     if (fused) {
+        // the limit, not this context's own size: the attribute is the
+        // process's, and another thread may set it before this one launches
         const cudaError_t e = cudaFuncSetAttribute(ibm_pass_particle_kernel<R>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pass_smem);
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, PASS_SMEM);
         if (e != cudaSuccess) return e;
     }
     for (int pass = 0; pass < 3; pass++) {

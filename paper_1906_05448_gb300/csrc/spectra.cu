@@ -271,11 +271,14 @@ template <int LOGN>
 static cudaError_t spectrum_t(Ctx &c, int nbins, float2 *field, double *part, double scale, double dfac, int &blocks) {
     constexpr int n = 1 << LOGN, Lx = fft_lines(LOGN), L = Lx < n ? Lx : n, TB = fft_threads(LOGN), TZ = L * n / 8;
     const size_t smx = sizeof(float2) * (size_t)(n * (Lx + 1) + n), smy = sizeof(float2) * (size_t)(n * L + n),
-                 smz = smy + sizeof(double) * 2 * (size_t)nbins;
+                 smz = smy + sizeof(double) * 2 * (size_t)nbins,
+                 // the attribute is the process's: what the most bins need,
+                 // so that no other thread's call sets it below this one's
+                 smz_most = smy + sizeof(double) * 2 * LBM_SPECTRUM_MAX_BINS;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(fft_x_kernel<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smx)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(fft_y_kernel<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smy)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(fft_z_bins_kernel<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smz)) != cudaSuccess)
+        (e = cudaFuncSetAttribute(fft_z_bins_kernel<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smz_most)) != cudaSuccess)
         return e;
     int per_sm = 0, dev = 0, sms = 0;
     cudaGetDevice(&dev);
