@@ -18,25 +18,25 @@
 namespace lbmgb {
 
 // Addresses of a D3Q19 sweep on columns: the pull of direction i for element
-// e = z + zp * column of a plane is Ap[i][e + bias], its store Bp[i][e] (one
+// e = z + zp * column of a plane is Ap[i][e], its store Bp[i][e] (one
 // address operation per access); pulls across the ends of z, and of x and y
-// where columns on the box faces are swept, add a correction
-// (column_index.h).
+// where columns on the box faces are swept, add a correction; e is shifted
+// there (column_index.h).
 struct ColumnPtrs {
-    const void *Ap[19];  // A + i Np - (c_z + zp (c_x + nx c_y)) - bias
-    void *Bp[19];        // B + i Np
-    int nx, ny, nz, zp;
-    unsigned bias;
+    const void *Ap[19];  // A + i Np - (c_z + zp (c_x + nx c_y)) + shift
+    void *Bp[19];        // B + i Np + shift
+    int nx, ny, nz, zp, shift;
     FastDiv fd_nx;
 };
 
-inline void column_ptrs(const Ctx &c, ColumnPtrs &p) {
+// wrap: for column_pull<WRAP = true>
+inline void column_ptrs(const Ctx &c, ColumnPtrs &p, bool wrap) {
     const long long sb = (long long)storage_bytes(c.storage);
-    p.bias = column_bias(c.nx, c.zp);
+    p.shift = wrap ? column_shift(c.Np) : 0;
     for (int i = 0; i < 19; i++) {
-        const long long off = cz(i) + (long long)c.zp * (cx(i) + (long long)c.nx * cy(i)) + p.bias;
+        const long long off = cz(i) + (long long)c.zp * (cx(i) + (long long)c.nx * cy(i)) - p.shift;
         p.Ap[i] = (const void *)((const char *)c.fA + sb * (i * c.Np - off));
-        p.Bp[i] = (void *)((char *)c.fB + sb * (i * c.Np));
+        p.Bp[i] = (void *)((char *)c.fB + sb * (i * c.Np + p.shift));
     }
     p.nx = c.nx;
     p.ny = c.ny;
@@ -45,19 +45,28 @@ inline void column_ptrs(const Ctx &c, ColumnPtrs &p) {
     p.fd_nx = FastDiv((unsigned)c.nx);
 }
 
+// the cell's element for the pointers above
+template <bool WRAP>
+__device__ __forceinline__ int column_element(const ColumnPtrs &p, int col, int z) {
+    return WRAP ? col * p.zp + z - p.shift : col * p.zp + z;
+}
+
 // the 19 pulls of the cell (column, z) through ld(const T *); WRAP: the
 // column may lie on an x or y face of the box
 template <typename T, bool WRAP, typename R, typename Ld>
 __device__ __forceinline__ void column_pull(R g[19], const ColumnPtrs &p, int col, int z, Ld ld) {
-    const unsigned e = (unsigned)(col * p.zp + z) + p.bias;
-    int x = 1, y = 1;  // no face unless WRAP
     if constexpr (WRAP) {
-        y = (int)p.fd_nx.div((unsigned)col);
-        x = col - y * p.nx;
-    }
-    const ColumnWrap w = column_wrap(x, y, z, WRAP ? p.nx : 4, WRAP ? p.ny : 4, p.nz, p.zp);
+        const int y = (int)p.fd_nx.div((unsigned)col), x = col - y * p.nx;
+        const int e = column_element<WRAP>(p, col, z);
+        const ColumnWrap w = column_wrap(x, y, z, p.nx, p.ny, p.nz, p.zp);
 #pragma unroll
-    for (int i = 0; i < 19; i++) g[i] = ld((const T *)p.Ap[i] + column_offset(e, w, cx(i), cy(i), cz(i)));
+        for (int i = 0; i < 19; i++) g[i] = ld((const T *)p.Ap[i] + column_offset(e, w, cx(i), cy(i), cz(i)));
+    } else {
+        const int e = column_element<WRAP>(p, col, z);
+        const int zlo = z == 0 ? p.nz : 0, zhi = z == p.nz - 1 ? p.nz : 0;
+#pragma unroll
+        for (int i = 0; i < 19; i++) g[i] = ld((const T *)p.Ap[i] + (e + (cz(i) > 0 ? zlo : 0) - (cz(i) < 0 ? zhi : 0)));
+    }
 }
 
 constexpr int COL_TILE = 32;  // x by z tile of the conversions, at one y

@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(256, ibm_column_min_blocks(S)) ibm_columns_swe
     collide<R, FORCE, SRT>(g, fs * body_force<R>(a, 0), fs * body_force<R>(a, 1), fs * body_force<R>(a, 2), a.rt, rho, ux,
                            uy, uz);
     watchdog(rho, ux, uy, uz, a.status);
-    const int e = (int)col * a.p.zp + z;
+    const int e = column_element<true>(a.p, (int)col, z);
 #pragma unroll
     for (int i = 0; i < 19; i++) Store<S>::st((T *)a.p.Bp[i] + e, g[i]);
 }
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256, ibm_column_min_blocks(S)) ibm_columns_col
     R rho, ux, uy, uz;
     collide<R, true, SRT>(g, Fx, Fy, Fz, a.rt, rho, ux, uy, uz);
     watchdog(rho, ux, uy, uz, a.status);
-    const int e = col * a.p.zp + z;
+    const int e = column_element<true>(a.p, col, z);
 #pragma unroll
     for (int i = 0; i < 19; i++) Store<S>::st((T *)a.p.Bp[i] + e, g[i]);
 }
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256) ibm_columns_spread(IbmPassArgs a) {
 
 // ------------------------------------------------------------- launchers ---
 static void fill_args(const Ctx &c, IbmColumnArgs &a, unsigned n) {
-    column_ptrs(c, a.p);
+    column_ptrs(c, a.p, true);
     a.info = c.col_ibm;
     a.sites = c.site_cell;
     a.ru = c.sup_ru;

@@ -29,7 +29,7 @@ struct ColumnCoef {
 };
 
 struct ColumnArgs {
-    const void *A;
+    const void *A;      // shifted as the pointers of the pulls
     const int2 *cols;   // fluid columns: x + nx y, index of the column's wall record (-1: no wall link)
     const uint4 *wall;  // per wall column: direction masks of its links (x), of those with q >= 1/2 (y), single-node (z)
     const void *coef;   // per wall column 19 pairs of weights (arithmetic type of the storage)
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256, column_min_blocks(S, SRT)) sweep_columns(
     const int2 col = __ldg(a.cols + ci);
     const int z = (int)(item - ci * a.nchunk) * 32 + (int)(threadIdx.x & 31);
     if (z >= a.p.nz) return;
-    const int e = col.x * a.p.zp + z;
+    const int e = column_element<WRAP>(a.p, col.x, z);
     R g[19];
     column_pull<T, WRAP>(g, a.p, col.x, z, ld);
     if (col.y >= 0) {  // uniform over the warp
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256, column_min_blocks(S, SRT)) sweep_columns(
         //   f*_l(x_f) + k2 (d_l + d_ibar)       single-node
         const uint4 w = __ldg(a.wall + col.y);
         const ColumnCoef<R> *kc = (const ColumnCoef<R> *)a.coef + 19 * (size_t)col.y;
-        const T *Ae = (const T *)a.A + e;
+        const T *Ae = (const T *)a.A + e;  // the cell's own populations
 #pragma unroll
         for (int l = 1; l < 19; l++) {
             if (!((w.x >> l) & 1u)) continue;
@@ -135,14 +135,14 @@ __global__ void __launch_bounds__(256, column_min_blocks(S, SRT)) sweep_columns(
 template <int S, bool FORCE, bool SRT>
 static cudaError_t launch_columns_t(Ctx &c) {
     ColumnArgs a{};
-    a.A = c.fA;
     a.cols = c.col_list;
     a.wall = c.col_wall;
     a.coef = c.col_coef;
     a.ncols = (unsigned)c.ncols;
     a.nchunk = (unsigned)((c.nz + 31) / 32);
     a.fd_chunk = FastDiv(a.nchunk);
-    column_ptrs(c, a.p);
+    column_ptrs(c, a.p, !c.pipe_nowrap);
+    a.A = (const char *)c.fA + (long long)storage_bytes(c.storage) * a.p.shift;
     a.Np = c.Np;
     a.status = c.d_status;
     a.pk = make_pair_k(c.rt.d_nu, c.F);
