@@ -24,7 +24,7 @@ struct Ctx {
     int storage, rates;
     int q = 19;  // velocity set: 19 (every path) or 27 (periodic box or pipe with IBB, BGK)
     unsigned *q27_colmask;  // D3Q27 pipe: per (x, y) column, the directions whose column is solid
-    unsigned *q27_hmask;    // D3Q27 pipe: per column, the wall directions with q >= 1/2
+    unsigned *q27_hmask;    // D3Q27 pipe: per column, the wall directions with q >= 1/2 or the halfway fallback
     void *q27_coef;         // D3Q27 pipe: per column and direction, the two wall weights
     Rates rt;
     cudaStream_t stream;

@@ -224,7 +224,7 @@ static_assert(q27opp(0) == 0 && q27opp(1) == 6 && q27opp(26) == 19, "opposites")
 // The weights of the two populations of each wall link are formed once, at
 // set-up (q27_coef_kernel), per column and direction: (2q, 1 - 2q) with
 // f*_i(x_f - c_i), (1, 0) for the halfway fallback, and
-// (1/(2q), (2q - 1)/(2q)) with f*_j(x_f), the last flagged in hmask.
+// (1/(2q), (2q - 1)/(2q)) with f*_j(x_f), the last two flagged in hmask.
 struct Q27PipeArgs {
     Q27Args b;
     const unsigned *colmask, *hmask;
@@ -268,6 +268,7 @@ __global__ void q27_coef_kernel(const unsigned *colmask, unsigned *hmask, void *
                 if ((m >> q27opp(i)) & 1u) {  // x_f - c_i solid too: halfway
                     k.k1 = R(1);
                     k.k2 = R(0);
+                    h |= 1u << i;
                 } else {
                     k.k1 = R(2.0 * q);
                     k.k2 = R(1.0 - 2.0 * q);
@@ -338,9 +339,9 @@ __global__ void __launch_bounds__(256, q27_min_blocks(S)) q27_columns_kernel(Q27
             const Q27Coef<R> k = kc[i];
             const R fi = Store<S>::ld(A + (i * N + (size_t)c));  // f*_i(x_f)
             // q < 1/2: f*_i(x_f - c_i), the regular pull of direction i;
-            // q >= 1/2: f*_j(x_f). The halfway fallback (weight 0) has no
-            // second value: its pull is a solid cell's, which may hold anything
-            const R second = ((h >> i) & 1u) ? Store<S>::ld(A + (j * N + (size_t)c)) : (k.k2 == R(0) ? R(0) : g[i]);
+            // q >= 1/2 and the halfway fallback (weight 0; its pull is a solid
+            // cell's, which may hold anything): f*_j(x_f)
+            const R second = ((h >> i) & 1u) ? Store<S>::ld(A + (j * N + (size_t)c)) : g[i];
             // the bounce-back acts on f, the storage holds g = f - w with w_i = w_j
             g[j] = k.k1 * fi + k.k2 * second;
         }
