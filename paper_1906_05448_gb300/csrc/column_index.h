@@ -20,6 +20,12 @@
 
 namespace lbmgb {
 
+// Whether the sweeps walk cells across the ends of the columns: 32-cell warps
+// of single columns would hold more than a tenth of idle lanes.
+LBM_HD bool column_flat(int nz) { return 10LL * nz < 9LL * ((nz + 31) / 32 * 32); }
+
+// Whether pulls that wrap in x and y need the shift.
+LBM_HD bool column_shifted(int nx, int zp, long long plane) { return plane + (long long)(nx + 2) * zp >= (1LL << 31); }
 LBM_HD int column_shift(long long plane) { return (int)(plane / 2); }
 
 // what a pull adds across the low and the high end of each axis

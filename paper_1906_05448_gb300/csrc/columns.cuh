@@ -20,8 +20,8 @@ namespace lbmgb {
 // Addresses of a D3Q19 sweep on columns: the pull of direction i for element
 // e = z + zp * column of a plane is Ap[i][e], its store Bp[i][e] (one
 // address operation per access); pulls across the ends of z, and of x and y
-// where columns on the box faces are swept, add a correction; e is shifted
-// there (column_index.h).
+// where columns on the box faces are swept, add a correction; e and the
+// pointers are shifted where that would overflow (column_index.h).
 struct ColumnPtrs {
     const void *Ap[19];  // A + i Np - (c_z + zp (c_x + nx c_y)) + shift
     void *Bp[19];        // B + i Np + shift
@@ -29,10 +29,48 @@ struct ColumnPtrs {
     FastDiv fd_nx;
 };
 
-// wrap: for column_pull<WRAP = true>
-inline void column_ptrs(const Ctx &c, ColumnPtrs &p, bool wrap) {
+// How threads walk the cells of n columns (of a list, or all of them in
+// order): a warp per 32 consecutive z of one column, so that a column's wall
+// is uniform over the warp and the accesses are whole sectors; or, where
+// such warps would hold too many idle lanes (column_flat), the cells one
+// after the other across the ends of the columns, which lie next to each
+// other then (zp = nz); that walk also takes planes so large that the pulls
+// need shifted offsets (column_shifted). us per step of the IBB pipe with warps
+// per column, and so:
+//   148 x 148 x 4    FP32 12.3 and 6.2   FP16 13.1 and 6.2   FP64 254 and 41
+//   148 x 148 x 16   FP32 12.3 and 10.3  FP16 13.5 and 10.3  FP64 254 and 131
+//   300 x 300 x 8    FP32 33.4 and 16.5  FP16 35.5 and 14.4  FP64 1033 and 274
+//   300 x 300 x 33   FP32 75.8 and 63.7  FP16 70.8 and 49.4  FP64 2044 and 1071
+//   148 x 148 x 58   FP32 37.1 and 31.3  FP16 22.1 and 20.8  FP64 505 and 456
+//   148 x 148 x 438  FP32 176.4 and 179.7, FP16 124.7 and 125.1 (14 warps of
+//                    32 for 438 cells: the wall and the sectors decide)
+// The line at nine tenths of busy lanes is where FP64, bound by its
+// arithmetic, would fall behind by more than the flat walk's ends cost FP32.
+struct ColumnItems {
+    unsigned n, run;  // run: warps, or cells, per column
+    FastDiv fd;
+    // column and z of this thread (blocks of 256); z may lie past the last plane
+    template <bool FLAT>
+    __device__ __forceinline__ bool cell(unsigned &ci, int &z) const {
+        const unsigned t = FLAT ? blockIdx.x * 256u + threadIdx.x : blockIdx.x * 8 + threadIdx.x / 32;
+        ci = fd.div(t);
+        if (ci >= n) return false;
+        z = FLAT ? (int)(t - ci * run) : (int)(t - ci * run) * 32 + (int)(threadIdx.x & 31);
+        return true;
+    }
+};
+inline ColumnItems column_items(const Ctx &c, long long n) {
+    const unsigned run = c.col_flat ? (unsigned)c.nz : (unsigned)((c.nz + 31) / 32);
+    return ColumnItems{(unsigned)n, run, FastDiv(run)};
+}
+inline unsigned column_item_blocks(const Ctx &c, const ColumnItems &it) {
+    const unsigned long long items = (unsigned long long)it.n * it.run, per = c.col_flat ? 256 : 8;
+    return (unsigned)((items + per - 1) / per);
+}
+
+inline void column_ptrs(const Ctx &c, ColumnPtrs &p) {
     const long long sb = (long long)storage_bytes(c.storage);
-    p.shift = wrap ? column_shift(c.Np) : 0;
+    p.shift = c.col_flat ? column_shift(c.Np) : 0;  // the cell-by-cell walk carries it whatever the size
     for (int i = 0; i < 19; i++) {
         const long long off = cz(i) + (long long)c.zp * (cx(i) + (long long)c.nx * cy(i)) - p.shift;
         p.Ap[i] = (const void *)((const char *)c.fA + sb * (i * c.Np - off));
@@ -46,26 +84,45 @@ inline void column_ptrs(const Ctx &c, ColumnPtrs &p, bool wrap) {
 }
 
 // the cell's element for the pointers above
-template <bool WRAP>
+template <bool SHIFT>
 __device__ __forceinline__ int column_element(const ColumnPtrs &p, int col, int z) {
-    return WRAP ? col * p.zp + z - p.shift : col * p.zp + z;
+    return SHIFT ? col * p.zp + z - p.shift : col * p.zp + z;
 }
 
 // the 19 pulls of the cell (column, z) through ld(const T *); WRAP: the
-// column may lie on an x or y face of the box
-template <typename T, bool WRAP, typename R, typename Ld>
+// column may lie on an x or y face of the box; SHIFT: with p.shift
+template <typename T, bool WRAP, bool SHIFT, typename R, typename Ld>
 __device__ __forceinline__ void column_pull(R g[19], const ColumnPtrs &p, int col, int z, Ld ld) {
-    if constexpr (WRAP) {
-        const int y = (int)p.fd_nx.div((unsigned)col), x = col - y * p.nx;
-        const int e = column_element<WRAP>(p, col, z);
-        const ColumnWrap w = column_wrap(x, y, z, p.nx, p.ny, p.nz, p.zp);
+    if constexpr (SHIFT) {
+        int x = 1, y = 1;  // no face unless WRAP
+        if constexpr (WRAP) {
+            y = (int)p.fd_nx.div((unsigned)col);
+            x = col - y * p.nx;
+        }
+        const int e = column_element<true>(p, col, z);
+        const ColumnWrap w = column_wrap(x, y, z, WRAP ? p.nx : 4, WRAP ? p.ny : 4, p.nz, p.zp);
 #pragma unroll
         for (int i = 0; i < 19; i++) g[i] = ld((const T *)p.Ap[i] + column_offset(e, w, cx(i), cy(i), cz(i)));
-    } else {
-        const int e = column_element<WRAP>(p, col, z);
-        const int zlo = z == 0 ? p.nz : 0, zhi = z == p.nz - 1 ? p.nz : 0;
+        return;
+    }
+    // (through the functions above, the same offsets without the shift take the IBM pipe 4 % longer)
+    const int e = col * p.zp + z;
+    const int zlo = z == 0 ? p.nz : 0, zhi = z == p.nz - 1 ? p.nz : 0;
+    int xlo = 0, xhi = 0, ylo = 0, yhi = 0;
+    if constexpr (WRAP) {
+        const int y = (int)p.fd_nx.div((unsigned)col), x = col - y * p.nx;
+        const int row = p.nx * p.zp;
+        xlo = x == 0 ? row : 0;
+        xhi = x == p.nx - 1 ? row : 0;
+        ylo = y == 0 ? row * p.ny : 0;
+        yhi = y == p.ny - 1 ? row * p.ny : 0;
+    }
 #pragma unroll
-        for (int i = 0; i < 19; i++) g[i] = ld((const T *)p.Ap[i] + (e + (cz(i) > 0 ? zlo : 0) - (cz(i) < 0 ? zhi : 0)));
+    for (int i = 0; i < 19; i++) {
+        int o = e + (cz(i) > 0 ? zlo : 0) - (cz(i) < 0 ? zhi : 0);
+        if constexpr (WRAP)
+            o += (cx(i) > 0 ? xlo : 0) - (cx(i) < 0 ? xhi : 0) + (cy(i) > 0 ? ylo : 0) - (cy(i) < 0 ? yhi : 0);
+        g[i] = ld((const T *)p.Ap[i] + o);
     }
 }
 

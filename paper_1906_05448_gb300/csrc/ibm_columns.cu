@@ -33,8 +33,7 @@ struct IbmColumnArgs {
     void *ru;          // (rho, u*) per site
     const void *sF;    // IBM force planes
     long long S;       // sites
-    unsigned n, nchunk;  // columns of the launch, 32-cell chunks per column
-    FastDiv fd_chunk;
+    ColumnItems items;  // of all columns, or of the support columns
     unsigned *status;
     Rates rt;
     double F[3];
@@ -67,20 +66,19 @@ __device__ __forceinline__ void ld_site4(const double *p, double q[4]) {
 // 0.3158 ms at 3, 0.3156 at 4, 0.3113 at 5, 0.3184 at 6
 constexpr int ibm_column_min_blocks(int S) { return S == LBM_F64 ? 2 : 5; }
 
-template <int S, bool FORCE, bool SRT>
+template <int S, bool FORCE, bool SRT, bool FLAT>
 __global__ void __launch_bounds__(256, ibm_column_min_blocks(S)) ibm_columns_sweep(IbmColumnArgs a) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
-    const unsigned item = blockIdx.x * 8 + threadIdx.x / 32;
-    const unsigned col = a.fd_chunk.div(item);
-    if (col >= a.n) return;
+    unsigned col;
+    int z;
+    if (!a.items.cell<FLAT>(col, z)) return;
     const int info = __ldg(a.info + col);
-    const int z = (int)(item - col * a.nchunk) * 32 + (int)(threadIdx.x & 31);
     if (z >= a.p.nz) return;
     R g[19];
-    column_pull<T, true>(g, a.p, (int)col, z, [](const T *p) -> R { return Store<S>::ld(p); });
+    column_pull<T, true, FLAT>(g, a.p, (int)col, z, [](const T *p) -> R { return Store<S>::ld(p); });
     const bool fluid = !(info & 1);
-    if (info >> 1) {  // support column (uniform over the warp)
+    if (info >> 1) {  // support column (uniform over a warp of one column)
         R drho = g[0];
 #pragma unroll
         for (int i = 1; i < 19; i++) drho += g[i];
@@ -101,23 +99,22 @@ __global__ void __launch_bounds__(256, ibm_column_min_blocks(S)) ibm_columns_swe
     collide<R, FORCE, SRT>(g, fs * body_force<R>(a, 0), fs * body_force<R>(a, 1), fs * body_force<R>(a, 2), a.rt, rho, ux,
                            uy, uz);
     watchdog(rho, ux, uy, uz, a.status);
-    const int e = column_element<true>(a.p, (int)col, z);
+    const int e = column_element<FLAT>(a.p, (int)col, z);
 #pragma unroll
     for (int i = 0; i < 19; i++) Store<S>::st((T *)a.p.Bp[i] + e, g[i]);
 }
 
-template <int S, bool SRT>
+template <int S, bool SRT, bool FLAT>
 __global__ void __launch_bounds__(256, ibm_column_min_blocks(S)) ibm_columns_collide(IbmColumnArgs a) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
-    const unsigned item = blockIdx.x * 8 + threadIdx.x / 32;
-    const unsigned k = a.fd_chunk.div(item);
-    if (k >= a.n) return;
+    unsigned k;
+    int z;
+    if (!a.items.cell<FLAT>(k, z)) return;
     const int col = __ldg(a.sites + k);
-    const int z = (int)(item - k * a.nchunk) * 32 + (int)(threadIdx.x & 31);
     if (z >= a.p.nz) return;
     R g[19];
-    column_pull<T, true>(g, a.p, col, z, [](const T *p) -> R { return Store<S>::ld(p); });
+    column_pull<T, true, FLAT>(g, a.p, col, z, [](const T *p) -> R { return Store<S>::ld(p); });
     const R fs = (__ldg(a.info + col) & 1) ? R(0) : R(1);
     const R *sF = (const R *)a.sF + (size_t)k * a.p.nz + z;
     const R Fx = fs * body_force<R>(a, 0) + sF[0];
@@ -126,7 +123,7 @@ __global__ void __launch_bounds__(256, ibm_column_min_blocks(S)) ibm_columns_col
     R rho, ux, uy, uz;
     collide<R, true, SRT>(g, Fx, Fy, Fz, a.rt, rho, ux, uy, uz);
     watchdog(rho, ux, uy, uz, a.status);
-    const int e = column_element<true>(a.p, col, z);
+    const int e = column_element<FLAT>(a.p, col, z);
 #pragma unroll
     for (int i = 0; i < 19; i++) Store<S>::st((T *)a.p.Bp[i] + e, g[i]);
 }
@@ -219,16 +216,14 @@ __global__ void __launch_bounds__(256) ibm_columns_spread(IbmPassArgs a) {
 }
 
 // ------------------------------------------------------------- launchers ---
-static void fill_args(const Ctx &c, IbmColumnArgs &a, unsigned n) {
-    column_ptrs(c, a.p, true);
+static void fill_args(const Ctx &c, IbmColumnArgs &a, long long n) {
+    column_ptrs(c, a.p);
     a.info = c.col_ibm;
     a.sites = c.site_cell;
     a.ru = c.sup_ru;
     a.sF = c.sup_F;
     a.S = (long long)c.pipe_sp * c.nz;
-    a.n = n;
-    a.nchunk = (unsigned)((c.nz + 31) / 32);
-    a.fd_chunk = FastDiv(a.nchunk);
+    a.items = column_items(c, n);
     a.status = c.d_status;
     a.rt = c.rt;
     for (int d = 0; d < 3; d++) {
@@ -237,28 +232,28 @@ static void fill_args(const Ctx &c, IbmColumnArgs &a, unsigned n) {
     }
 }
 
-template <int S>
+template <int S, bool FLAT>
 static cudaError_t sweep_t(Ctx &c) {
     IbmColumnArgs a;
-    fill_args(c, a, (unsigned)(c.nx * c.ny));
-    const unsigned nb = (unsigned)(((long long)a.n * a.nchunk + 7) / 8);
+    fill_args(c, a, (long long)c.nx * c.ny);
+    const unsigned nb = column_item_blocks(c, a.items);
     const bool force = c.F[0] != 0.0 || c.F[1] != 0.0 || c.F[2] != 0.0, srt = c.rates == LBM_RATES_SRT;
     count_launch(c, G_BULK);
-    if (srt && force) ibm_columns_sweep<S, true, true><<<nb, 256, 0, c.stream>>>(a);
-    else if (srt) ibm_columns_sweep<S, false, true><<<nb, 256, 0, c.stream>>>(a);
-    else if (force) ibm_columns_sweep<S, true, false><<<nb, 256, 0, c.stream>>>(a);
-    else ibm_columns_sweep<S, false, false><<<nb, 256, 0, c.stream>>>(a);
+    if (srt && force) ibm_columns_sweep<S, true, true, FLAT><<<nb, 256, 0, c.stream>>>(a);
+    else if (srt) ibm_columns_sweep<S, false, true, FLAT><<<nb, 256, 0, c.stream>>>(a);
+    else if (force) ibm_columns_sweep<S, true, false, FLAT><<<nb, 256, 0, c.stream>>>(a);
+    else ibm_columns_sweep<S, false, false, FLAT><<<nb, 256, 0, c.stream>>>(a);
     return cudaGetLastError();
 }
 
-template <int S>
+template <int S, bool FLAT>
 static cudaError_t collide_t(Ctx &c) {
     IbmColumnArgs a;
-    fill_args(c, a, (unsigned)c.pipe_sp);
-    const unsigned nb = (unsigned)(((long long)a.n * a.nchunk + 7) / 8);
+    fill_args(c, a, c.pipe_sp);
+    const unsigned nb = column_item_blocks(c, a.items);
     count_launch(c, G_IBMCOL);
-    if (c.rates == LBM_RATES_SRT) ibm_columns_collide<S, true><<<nb, 256, 0, c.stream>>>(a);
-    else ibm_columns_collide<S, false><<<nb, 256, 0, c.stream>>>(a);
+    if (c.rates == LBM_RATES_SRT) ibm_columns_collide<S, true, FLAT><<<nb, 256, 0, c.stream>>>(a);
+    else ibm_columns_collide<S, false, FLAT><<<nb, 256, 0, c.stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -282,18 +277,18 @@ static cudaError_t passes_t(Ctx &c) {
 
 cudaError_t launch_ibm_columns_sweep(Ctx &c) {
     switch (c.storage) {
-    case LBM_F64: return sweep_t<LBM_F64>(c);
-    case LBM_F32: return sweep_t<LBM_F32>(c);
-    case LBM_F16S: return sweep_t<LBM_F16S>(c);
-    default: return sweep_t<LBM_BF16S>(c);
+    case LBM_F64: return c.col_flat ? sweep_t<LBM_F64, true>(c) : sweep_t<LBM_F64, false>(c);
+    case LBM_F32: return c.col_flat ? sweep_t<LBM_F32, true>(c) : sweep_t<LBM_F32, false>(c);
+    case LBM_F16S: return c.col_flat ? sweep_t<LBM_F16S, true>(c) : sweep_t<LBM_F16S, false>(c);
+    default: return c.col_flat ? sweep_t<LBM_BF16S, true>(c) : sweep_t<LBM_BF16S, false>(c);
     }
 }
 cudaError_t launch_ibm_columns_collide(Ctx &c) {
     switch (c.storage) {
-    case LBM_F64: return collide_t<LBM_F64>(c);
-    case LBM_F32: return collide_t<LBM_F32>(c);
-    case LBM_F16S: return collide_t<LBM_F16S>(c);
-    default: return collide_t<LBM_BF16S>(c);
+    case LBM_F64: return c.col_flat ? collide_t<LBM_F64, true>(c) : collide_t<LBM_F64, false>(c);
+    case LBM_F32: return c.col_flat ? collide_t<LBM_F32, true>(c) : collide_t<LBM_F32, false>(c);
+    case LBM_F16S: return c.col_flat ? collide_t<LBM_F16S, true>(c) : collide_t<LBM_F16S, false>(c);
+    default: return c.col_flat ? collide_t<LBM_BF16S, true>(c) : collide_t<LBM_BF16S, false>(c);
     }
 }
 cudaError_t launch_ibm_columns_passes(Ctx &c) {

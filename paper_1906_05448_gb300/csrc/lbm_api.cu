@@ -1,6 +1,7 @@
 // C ABI of the library (declared in include/lbm.h): workspace layout, set-up
 // of the geometry, the per-step kernel sequence and host-side checks.
 #include "lbm_internal.cuh"
+#include "column_index.h"
 #include "spectra_scratch.h"
 
 #include <cmath>
@@ -81,11 +82,12 @@ bool make_plan(const lbm_grid *g, Plan &P) {
     const size_t nq = g->lattice == 27 ? 27 : 19;
     // the populations, and beside them room for the padding of the pipe's
     // columns (columns.cuh): a pitch of whole 16-cell groups where it fits,
-    // so that every column starts on a sector in every storage type
+    // so that every column starts on a sector in every storage type; none
+    // where the sweeps cross from column to column
     const size_t slack = 10 * ms;
     P.fA = L.take((nq * n + slack) * sb);
     P.fB = L.take((nq * n + slack) * sb);
-    P.zp = (g->nz + 15) / 16 * 16;
+    P.zp = column_flat(g->nz) ? g->nz : (g->nz + 15) / 16 * 16;
     P.Np = (long long)g->nx * g->ny * P.zp;
     if (nq * (size_t)P.Np > nq * n + slack || P.Np >= (1LL << 31) - 4096) {
         P.zp = g->nz;
@@ -743,6 +745,7 @@ lbm_status lbm_create(const lbm_grid *grid, double tau, const double force[3], v
     c.pipe_sp = 0;
     c.pipe_max_xy = P.max_xy;
     c.zp = P.zp;
+    c.col_flat = column_flat(c.nz) || column_shifted(c.nx, c.zp, c.Np);
     c.Np = P.Np;
     c.col_list = (int2 *)(b + P.col_list);
     c.col_wall = (uint4 *)(b + P.col_wall);

@@ -49,6 +49,7 @@ struct Ctx {
     void *link_dP, *link_dT;  // per-link momentum exchange and torque (arithmetic type of the storage)
     // column layout of the pipe (columns.cuh), in use once zlay is set
     int zlay, zp;      // zp: elements from a column to the next (>= nz)
+    int col_flat;      // the sweeps walk the cells across the ends of the columns (zp = nz)
     long long Np;      // elements of a population plane in that layout
     int2 *col_list;    // fluid columns: x + nx y, index of the column's wall record or -1
     long long ncols;

@@ -230,8 +230,7 @@ struct Q27PipeArgs {
     const unsigned *colmask, *hmask;
     const void *coef;  // per column x 27 directions: two weights in the arithmetic type
     const int2 *cols;  // fluid columns: x + nx y, nonzero if the column has wall links
-    unsigned ncols, nchunk;
-    FastDiv fd_chunk;
+    ColumnItems items;
     int zp;
     long long Np;
     // the pull of direction i for element e of a plane is Ap[i][e] (plus nz
@@ -284,8 +283,8 @@ __global__ void q27_coef_kernel(const unsigned *colmask, unsigned *hmask, void *
     hmask[col] = h;
 }
 
-// On the column layout (columns.cuh): one warp per 32 consecutive z of a
-// fluid column, the column's mask and weights uniform over the warp. What
+// On the column layout (columns.cuh): a warp takes 32 consecutive z of a
+// fluid column, whose mask and weights are uniform over it. What
 // bounds it: HBM. 0.259 ms per step on the benchmark pipe (148 x 148 x 438,
 // R = 73, FP32): 6.12 TB/s of its 216 B per fluid cell; the sweep over
 // x-fast cells, whose warps mixed fluid, wall and solid cells, took 0.386.
@@ -294,17 +293,16 @@ __global__ void q27_coef_kernel(const unsigned *colmask, unsigned *hmask, void *
 constexpr int q27_min_blocks(int S) { return S == LBM_F32 ? 4 : 2; }
 
 // WRAP: fluid columns touch an x or y face of the box
-template <int S, bool FORCE, bool WRAP>
+template <int S, bool FORCE, bool WRAP, bool FLAT>
 __global__ void __launch_bounds__(256, q27_min_blocks(S)) q27_columns_kernel(Q27PipeArgs pa) {
     typedef typename Store<S>::T T;
     typedef typename Store<S>::R R;
     const Q27Args &a = pa.b;
-    const unsigned item = blockIdx.x * 8 + threadIdx.x / 32;
-    const unsigned ci = pa.fd_chunk.div(item);
-    if (ci >= pa.ncols) return;
+    unsigned ci;
+    int z;
+    if (!pa.items.cell<FLAT>(ci, z)) return;
     const int2 col = __ldg(pa.cols + ci);
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const int z = (int)(item - ci * pa.nchunk) * 32 + (int)(threadIdx.x & 31);
     if (z >= nz) return;
     const int c = col.x * pa.zp + z;
     const int zlo = z == 0 ? nz : 0, zhi = z == nz - 1 ? nz : 0;
@@ -328,7 +326,7 @@ __global__ void __launch_bounds__(256, q27_min_blocks(S)) q27_columns_kernel(Q27
             g[i] = Store<S>::ld((const T *)pa.Ap[i] + (c + (q27z(i) > 0 ? zlo : 0) - (q27z(i) < 0 ? zhi : 0)));
     }
     const unsigned rem = (unsigned)col.x;
-    if (col.y) {  // wall column (uniform over the warp): the populations coming back from the wall
+    if (col.y) {  // wall column (uniform over a warp of one column): the populations coming back from the wall
         const unsigned m = __ldg(pa.colmask + rem);
         const unsigned h = __ldg(pa.hmask + rem);
         const Q27Coef<R> *kc = (const Q27Coef<R> *)pa.coef + (size_t)rem * Q27;
@@ -407,9 +405,7 @@ cudaError_t launch_q27_step(Ctx &c) {
         pa.hmask = c.q27_hmask;
         pa.coef = c.q27_coef;
         pa.cols = c.col_list;
-        pa.ncols = (unsigned)c.ncols;
-        pa.nchunk = (unsigned)((c.nz + 31) / 32);
-        pa.fd_chunk = FastDiv(pa.nchunk);
+        pa.items = column_items(c, c.ncols);
         pa.zp = c.zp;
         pa.Np = c.Np;
         const long long sb = (long long)storage_bytes(c.storage);
@@ -418,16 +414,19 @@ cudaError_t launch_q27_step(Ctx &c) {
             pa.Ap[i] = (const void *)((const char *)c.fA + sb * (i * c.Np - off));
             pa.Bp[i] = (void *)((char *)c.fB + sb * (i * c.Np));
         }
-        const unsigned nb = (unsigned)(((long long)pa.ncols * pa.nchunk + 7) / 8);
+        const unsigned nb = column_item_blocks(c, pa.items);
         if (nb == 0) return cudaSuccess;
-#define QC(S, W)                                                                       \
-    if (force) q27_columns_kernel<S, true, W><<<nb, 256, 0, c.stream>>>(pa);           \
-    else q27_columns_kernel<S, false, W><<<nb, 256, 0, c.stream>>>(pa)
-        if (c.storage == LBM_F64) {
-            if (c.pipe_nowrap) { QC(LBM_F64, false); } else { QC(LBM_F64, true); }
-        } else {
-            if (c.pipe_nowrap) { QC(LBM_F32, false); } else { QC(LBM_F32, true); }
-        }
+#define QC(S, W, L)                                                                    \
+    if (force) q27_columns_kernel<S, true, W, L><<<nb, 256, 0, c.stream>>>(pa);        \
+    else q27_columns_kernel<S, false, W, L><<<nb, 256, 0, c.stream>>>(pa)
+#define QS(S)                                                                          \
+    if (c.col_flat) {                                                                  \
+        if (c.pipe_nowrap) { QC(S, false, true); } else { QC(S, true, true); }         \
+    } else {                                                                           \
+        if (c.pipe_nowrap) { QC(S, false, false); } else { QC(S, true, false); }       \
+    }
+        if (c.storage == LBM_F64) { QS(LBM_F64) } else { QS(LBM_F32) }
+#undef QS
 #undef QC
         return cudaGetLastError();
     }

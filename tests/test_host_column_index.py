@@ -1,7 +1,8 @@
 """Pull offsets of the column layout (column_index.h), compiled with g++:
 every direction from every corner, face and some inner cells, on grids up to
 the largest that a context takes (nx ny nz below 2^31 - 4096), gives the
-wrapped neighbour's element without a 32-bit overflow on the way."""
+wrapped neighbour's element without a 32-bit overflow on the way, shifted or, where that is said to do,
+not."""
 import os
 import shutil
 import subprocess
@@ -22,7 +23,10 @@ int main() {
     for (auto &g : grids) {
         const long long nx = g[0], ny = g[1], nz = g[2], zp = g[3];
         if (nx * ny * zp >= (1LL << 31) - 4096) return 9;
-        const long long shift = lbmgb::column_shift(nx * ny * zp);
+        const bool big = lbmgb::column_shifted((int)nx, (int)zp, nx * ny * zp);
+        if (big != (nx * ny * zp + (nx + 2) * zp >= (1LL << 31))) return 8;
+        for (int s = big; s < 2; s++) {  // without the shift only where it is not needed
+        const long long shift = s ? lbmgb::column_shift(nx * ny * zp) : 0;
         const long long xs[] = {0, 1, nx / 2, nx - 2, nx - 1}, ys[] = {0, 1, ny / 2, ny - 2, ny - 1},
                         zs[] = {0, nz > 1 ? 1 : 0, nz / 2, nz > 1 ? nz - 2 : 0, nz - 1};
         for (long long x : xs) for (long long y : ys) for (long long z : zs)
@@ -36,6 +40,7 @@ int main() {
                     return 1;
                 }
             }
+        }
     }
     return 0;
 }
