@@ -40,8 +40,8 @@ struct Plan {
     size_t fA, fB, flags, owner, aux;
     size_t site_cell, site_first, site_mask, sup_ru, sup_F, sup_Fp;
     size_t link_cell, link_pid, link_dir, link_scheme, link_q, link_dP, link_dT;
-    size_t blk_sites, blk_links, counts, status, col_list, col_wall, col_coef, col_ibm, refill;
-    long long max_refill;
+    size_t blk_sites, blk_links, counts, status, col_wall, col_coef, refill;
+    long long max_refill, max_wall;
     int zp;
     long long Np;
     size_t xy_start, xy_j, xy_w, it_k, it_w;
@@ -116,11 +116,14 @@ bool make_plan(const lbm_grid *g, Plan &P) {
     P.max_ring = 4 * (g->nx + g->ny);
     P.it_k = L.take(4 * 16 * (size_t)P.max_ring);
     P.it_w = L.take(8 * 16 * (size_t)P.max_ring);
-    const size_t nxy = (size_t)g->nx * g->ny;
-    P.col_list = L.take(8 * nxy);
-    P.col_wall = L.take(16 * nxy);
-    P.col_coef = L.take(16 * 19 * nxy);
-    P.col_ibm = L.take(4 * nxy);
+    // The pipe's tables on the column layout lie where other treatments of a
+    // context keep theirs. The wall records and weights of the IBB pipe, for
+    // at most 4 (nx + ny) wall columns (a circle's rim has fewer than
+    // 2 (nx + ny)): in the ring tables of the IBM pipe, 1536 (nx + ny) bytes
+    // from xy_j on, which are filled when an IBM step fixes the treatment.
+    P.max_wall = std::min((long long)g->nx * g->ny, 4LL * (g->nx + g->ny));
+    P.col_wall = P.xy_j;
+    P.col_coef = P.col_wall + (16 * (size_t)P.max_wall + ALIGN - 1) / ALIGN * ALIGN;
     P.blk_sites = L.take(8 * (size_t)P.nblk);
     P.blk_links = L.take(8 * (size_t)P.nblk);
     P.counts = L.take(64);
@@ -158,7 +161,7 @@ bool make_plan(const lbm_grid *g, Plan &P) {
     P.rho_f = L.take(8 * n);  // these two stay next to each other (the statistics keep records across both)
     P.u_f = L.take(24 * n);
     P.partials = L.take(8 * stats_partials_doubles());
-    P.near_key = L.take(8 * n);
+    P.near_key = L.take(8 * n);  // with spheres only; a pipe's column list, or its IBM column records, lie there
     P.max_cl = P.max_np > 0 ? 1500LL * P.max_np : 0;
     P.cl_w = L.take(4 * 14409);
     P.cl_pk = L.take(mlp_pack_bytes());
@@ -620,6 +623,7 @@ lbm_status build_columns(Ctx &c) {
         cols.push_back(make_int2((int)cell, slot));
     }
     if (k != nl) return fail(c, LBM_EINVAL, "link list is not in cell order");
+    if ((long long)wall.size() > c.max_wall) return fail(c, LBM_ENOMEM, "wall columns exceed capacity");
     c.ncols = (long long)cols.size();
     if (!cols.empty()) CK(cudaMemcpy(c.col_list, cols.data(), sizeof(int2) * cols.size(), cudaMemcpyHostToDevice));
     if (!wall.empty()) CK(cudaMemcpy(c.col_wall, wall.data(), sizeof(uint4) * wall.size(), cudaMemcpyHostToDevice));
@@ -747,10 +751,11 @@ lbm_status lbm_create(const lbm_grid *grid, double tau, const double force[3], v
     c.zp = P.zp;
     c.col_flat = column_flat(c.nz) || column_shifted(c.nx, c.zp, c.Np);
     c.Np = P.Np;
-    c.col_list = (int2 *)(b + P.col_list);
+    c.col_list = (int2 *)(b + P.near_key);
+    c.col_ibm = (int *)(b + P.near_key);
+    c.max_wall = P.max_wall;
     c.col_wall = (uint4 *)(b + P.col_wall);
     c.col_coef = b + P.col_coef;
-    c.col_ibm = (int *)(b + P.col_ibm);
     c.nblk = P.nblk;
     c.blk_sites = (long long *)(b + P.blk_sites);
     c.blk_links = (long long *)(b + P.blk_links);

@@ -51,11 +51,11 @@ struct Ctx {
     int zlay, zp;      // zp: elements from a column to the next (>= nz)
     int col_flat;      // the sweeps walk the cells across the ends of the columns (zp = nz)
     long long Np;      // elements of a population plane in that layout
-    int2 *col_list;    // fluid columns: x + nx y, index of the column's wall record or -1
-    long long ncols;
+    int2 *col_list;    // fluid columns: x + nx y, index of the column's wall record or -1 (IBB, D3Q27)
+    long long ncols, max_wall;
     uint4 *col_wall;   // per wall column: direction masks of its links, of those with q >= 1/2, of single-node ones
     void *col_coef;    // per wall column 19 pairs of weights (arithmetic type of the storage)
-    int *col_ibm;      // IBM: per column (support index + 1) << 1 | solid
+    int *col_ibm;      // IBM: per column (support index + 1) << 1 | solid (in the place of col_list)
     int markers_stale; // IBM on columns: the marker forces of the last step are not in mFacc yet
     long long static_single;  // single-node (scheme 2) links of a plane of the wall
     int pipe_nowrap;   // no fluid cell on an x or y face: pulls wrap only in z
