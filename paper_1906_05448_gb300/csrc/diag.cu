@@ -314,8 +314,8 @@ __device__ __forceinline__ long long warp_slot(bool take, long long *count) {
 // atomics, no bank conflicts); FP64 atomics on 40 shared bins per block,
 // contended by the lanes of a warp, were most of the former bins pass. The
 // bin index is decided in FP32 from the distance in the cell's key (20 bits
-// of mantissa) away from the bin edges and by the exact FP64 quotient within
-// 2e-4 of one. A plane's loads are issued one plane ahead: only 8 warps per SM
+// of mantissa) away from the bin edges and by the exact FP64 quotient near
+// one. A plane's loads are issued one plane ahead: only 8 warps per SM
 // fit beside the bins.
 // 256^3, 2000 spheres, FP32, with bins: 0.7 ms in place of 1.57 (energies) +
 // 2.9 (bins); 1.74 ms in FP64, 1.12 without the loads ahead.
@@ -329,6 +329,7 @@ struct StatsArgs {
     const unsigned long long *near_key;
     const double *X, *R;
     float bins_per_unit;  // 1 / (0.05 R) where all particles have one radius, else 0
+    float bin_slack;      // how far a bin coordinate may be off, per unit of 1 / (0.05 R), beside 1e-4
     const float *eps_o;  // dissipation from the closure where >= 0, or null
     int nx, ny, nz;
     long long N;
@@ -344,9 +345,15 @@ __device__ __forceinline__ int radial_bin(const StatsArgs &a, unsigned long long
     // the key's distance s with the upper 20 bits of its mantissa
     const unsigned hi = (unsigned)(key >> 32);
     const float s = __uint_as_float((((hi >> 20) - 896u) << 23) | ((hi & 0xfffffu) << 3));
-    const float tb = s * (a.bins_per_unit > 0.f ? a.bins_per_unit : 20.0f / (float)a.R[p]);  // (r / R - 1) / 0.05
+    const float k = a.bins_per_unit > 0.f ? a.bins_per_unit : 20.0f / (float)a.R[p], tb = s * k;  // (r / R - 1) / 0.05
     int b = (int)tb;
-    if (fabsf(tb - rintf(tb)) < 2e-4f) {  // tb carries at most 5e-5
+    // The key's s carries the FP32 centre of near_key_kernel, rounded at the
+    // half width of its box (less than reach + R + 4, R the particle's own),
+    // at most 1.8 (reach + R + 4) 2^-24, and the rounding of distances up to
+    // 3 R, 14 R 2^-24 with the root; k s that of the 20 bits, 4e-5, and two
+    // products. With R = 20 / k: 1.1e-7 (reach + 4) k + 7e-5. A box made for a
+    // large particle's reach is coarse for the bins of a small one.
+    if (fabsf(tb - rintf(tb)) < 2e-4f + a.bin_slack * k) {
         const double dx = dmimg(__dsub_rn((double)x, a.X[3 * p]), a.nx);
         const double dy = dmimg(__dsub_rn((double)y, a.X[3 * p + 1]), a.ny);
         const double dz = dmimg(__dsub_rn((double)z, a.X[3 * p + 2]), a.nz);
@@ -944,7 +951,7 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
         if ((e = mask_cells(c, solid_held ? c.partials : nullptr, rec ? (float4 *)u32 : nullptr)) != cudaSuccess) return e;
     const int mblk = solid_held && (c.np > 0 || c.has_pipe) ? mask_blocks(c) : 0;
     StatsArgs a{c.u_f, c.rho_f, rec ? (const float4 *)u32 : nullptr, rec ? (const float4 *)u32 + c.N : nullptr, c.flags, c.near_key, c.X, c.R,
-                c.same_radius ? 20.0f / (float)c.max_radius : 0.f, eps_o, c.nx, c.ny, c.nz, c.N, nu, c.has_pipe, ibb, !mask,
+                c.same_radius ? 20.0f / (float)c.max_radius : 0.f, 2e-7f * (float)(reach + 4.0), eps_o, c.nx, c.ny, c.nz, c.N, nu, c.has_pipe, ibb, !mask,
                 c.partials, bpart};
     const long long tiles = (long long)((c.nx + 31) / 32) * ((c.ny + 3) / 4) * ((c.nz + ST_RUN - 1) / ST_RUN);
     const int nblk = (int)std::min<long long>(tiles, SNB);

@@ -109,3 +109,38 @@ def test_statistics_leave_the_populations_alone(lbm, wall, storage, tmp_path):
         runs.append(g.populations())
         g.close()
     assert np.array_equal(*runs)
+
+
+def test_bins_of_a_small_sphere_beside_a_large_one(lbm):
+    """Spheres of radius 0.6 beside one of 64: the distances of the small ones
+    are formed in the coarse coordinates of the large one's reach. The centres
+    put one cell of each within that error of a bin edge."""
+    n, r, R = 134, 0.6, 64.0
+    frac = [[0.6503087487684525, 0.2039073800978315, 0.353350778146563],
+            [0.5836530203021653, 0.6346187417687474, 0.040459510349080574],
+            [0.30313713100829887, 0.18944387380685157, 0.8637899145128074],
+            [0.576195652467419, 0.878151356172026, 0.39333355485314314],
+            [0.3109796451597333, 0.4064864649216986, 0.45511893301826944],
+            [0.29087156922514623, 0.4230262586893332, 0.9846860944370519],
+            [0.2924158302428168, 0.9461288070160094, 0.6216942062295914],
+            [0.37036860357278556, 0.42926034510139743, 0.22518122567558407]]
+    corner = [[x, y, z] for x in (4, 124) for y in (4, 124) for z in (4, 124)]
+    X = np.concatenate([np.array(corner) + np.array(frac), [[66.5, 66.5, 66.5]]])
+    radii = np.array([r] * 8 + [R])
+    g = lbm.Lattice(n, n, n, 0.6, storage="f32", max_particles=9)
+    g.add_spheres(X, radii, U=np.zeros((9, 3)), W=np.zeros((9, 3)))
+    got = g.stats(lbm.STATS_BINS)
+    z, y, x = np.meshgrid(*[np.arange(n)] * 3, indexing="ij", sparse=True)
+    near, who = np.full((n, n, n), np.inf), np.zeros((n, n, n), dtype=int)
+    for p in range(9):
+        d2 = 0.0
+        for a, c in ((x, 0), (y, 1), (z, 2)):
+            d = a - X[p, c]
+            d2 = d2 + (d - n * np.rint(d / n)) ** 2
+        s = np.sqrt(d2) - radii[p]
+        m = s < near
+        near[m], who[m] = s[m], p
+    b = np.floor(near / radii[who] / 0.05).astype(int)
+    ok = (near > 0) & (b < 40)
+    assert np.array_equal(got["bin_count"], np.bincount(b[ok], minlength=40))
+    g.close()
