@@ -6,6 +6,7 @@
 #include "columns.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 #include <vector>
@@ -900,10 +901,57 @@ cudaError_t launch_mask(Ctx &c) {
     return mask_cells(c, nullptr);
 }
 
+// The masked fields' sums into res (NP columns, then 3 NBIN of the bins).
+// rec: from the FP32 records, else from the FP64 fields (launch_macro wrote
+// the one or the other); raw: solid cells keep the virtual fluid.
+static cudaError_t stats_sums(Ctx &c, float4 *rec, bool raw, bool bins, double reach, const float *eps_o, double nu,
+                              double *res) {
+    cudaError_t e;
+    const int ibb = c.armed_bc == LBM_BC_IBB;
+    count_launch(c, G_STATS, 3);
+    // what the masked solid cells held counts in mass and momentum unless the wall is IBB
+    const bool solid_held = !raw && !ibb;
+    double *bpart = c.partials + (size_t)SNB * NP;
+    if (!raw && !(c.zlay && c.q == 19 && ibb))
+        if ((e = mask_cells(c, solid_held ? c.partials : nullptr, rec)) != cudaSuccess) return e;
+    const int mblk = solid_held && (c.np > 0 || c.has_pipe) ? mask_blocks(c) : 0;
+    StatsArgs a{c.u_f, c.rho_f, rec, rec ? rec + c.N : nullptr, c.flags, c.near_key, c.X, c.R,
+                c.same_radius ? 20.0f / (float)c.max_radius : 0.f, 2e-7f * (float)(reach + 4.0), eps_o, c.nx, c.ny, c.nz, c.N,
+                nu, c.has_pipe, ibb, raw, c.partials, bpart};
+    const long long tiles = (long long)((c.nx + 31) / 32) * ((c.ny + 3) / 4) * ((c.nz + ST_RUN - 1) / ST_RUN);
+    const int nblk = (int)std::min<long long>(tiles, SNB);
+    const size_t smem = bins ? sizeof(double) * 2 * NBIN * ST_TB + sizeof(int) * NBIN : 0;
+    void (*kernel)(StatsArgs) = bins ? (rec ? stats_kernel<true, float2> : stats_kernel<true, double>)
+                                     : (rec ? stats_kernel<false, float2> : stats_kernel<false, double>);
+    if (bins && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
+    kernel<<<nblk, ST_TB, smem, c.stream>>>(a);
+    stats_reduce_kernel<<<NP + (bins ? 3 * NBIN : 0), SB, 0, c.stream>>>(c.partials, bpart, nblk, mblk, res);
+    return cudaGetLastError();
+}
+
+// Whether sums of float pairs hold what FP64 would: products below 2^-102
+// lose their low parts to underflow and those below 2^-149 vanish, which
+// shows where the mean square of a sum's terms is below 2^-97 (velocities or
+// differences below 2.5e-15: 48 bits of it are left above 2^-149); squares
+// beyond FP32's range (an unstable state) show as infinities or NaN. Zero
+// sums (a fluid at rest) count as unresolved too: nothing tells them from
+// vanished ones.
+static bool pairs_resolve(const Ctx &c, const double *s, bool bins, double nu) {
+    auto mean = [](double sum, double n) { return n == 0.0 || (sum >= 0x1p-97 * n && std::isfinite(sum)); };
+    const double N = (double)c.N, nf = s[ST_NF], four_ss = 1.0 / (0.5 * nu);  // sums hold (nu / 2) 4 s_ij s_ij
+    bool ok = std::isfinite(s[ST_MASS] + s[ST_MX] + s[ST_MY] + s[ST_MZ]) && mean(s[ST_KF], nf) && mean(s[ST_EF] * four_ss, nf) &&
+              mean(s[ST_KF] + s[ST_KS], N) && mean((s[ST_EF] + s[ST_ES]) * four_ss, N);
+    for (int k = 0; bins && k < NBIN; k++) {
+        const double *b = s + NP + k;
+        ok = ok && mean(b[0], b[2 * NBIN]) && mean(b[NBIN] * four_ss, b[2 * NBIN]);
+    }
+    return ok;
+}
+
 cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
     cudaError_t e;
     memset(o, 0, sizeof(*o));
-    const int ibb = c.armed_bc == LBM_BC_IBB;
     const int ibm = c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B;
     const bool closure = (flags & LBM_STATS_CLOSURE) && c.np > 0 && c.cl_ready && c.max_cl > 0 && c.q == 19;
     // FP32 records of the fields, 16 B per cell: all that 32- and 16-bit
@@ -914,8 +962,7 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
     const bool rec = c.storage != LBM_F64;
     float *u32 = rec ? (float *)c.rho_f : (closure ? (float *)c.fB : nullptr);
     if ((e = launch_macro(c, 0, u32, rec)) != cudaSuccess) return e;
-    count_launch(c, G_STATS, 3);
-    const bool mask = !(ibm && (flags & LBM_STATS_UNMASK));
+    const bool raw = ibm && (flags & LBM_STATS_UNMASK);
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     const double nu = (c.tau - 0.5) / 3.0;
     const bool bins = (flags & LBM_STATS_BINS) && c.np > 0;
@@ -944,26 +991,9 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
         prof_span(c, G_CLOSURE, t0, prof_event(c));
         eps_o = c.cl_eps;
     }
-    // what the masked solid cells held counts in mass and momentum unless the wall is IBB
-    const bool solid_held = mask && !ibb;
-    double *bpart = c.partials + (size_t)SNB * NP, *res = bpart + (size_t)SNB * 3 * NBIN;
-    if (mask && !(c.zlay && c.q == 19 && ibb))
-        if ((e = mask_cells(c, solid_held ? c.partials : nullptr, rec ? (float4 *)u32 : nullptr)) != cudaSuccess) return e;
-    const int mblk = solid_held && (c.np > 0 || c.has_pipe) ? mask_blocks(c) : 0;
-    StatsArgs a{c.u_f, c.rho_f, rec ? (const float4 *)u32 : nullptr, rec ? (const float4 *)u32 + c.N : nullptr, c.flags, c.near_key, c.X, c.R,
-                c.same_radius ? 20.0f / (float)c.max_radius : 0.f, 2e-7f * (float)(reach + 4.0), eps_o, c.nx, c.ny, c.nz, c.N, nu, c.has_pipe, ibb, !mask,
-                c.partials, bpart};
-    const long long tiles = (long long)((c.nx + 31) / 32) * ((c.ny + 3) / 4) * ((c.nz + ST_RUN - 1) / ST_RUN);
-    const int nblk = (int)std::min<long long>(tiles, SNB);
-    const size_t smem = bins ? sizeof(double) * 2 * NBIN * ST_TB + sizeof(int) * NBIN : 0;
-    void (*kernel)(StatsArgs) = bins ? (rec ? stats_kernel<true, float2> : stats_kernel<true, double>)
-                                     : (rec ? stats_kernel<false, float2> : stats_kernel<false, double>);
-    if (bins && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
-    kernel<<<nblk, ST_TB, smem, c.stream>>>(a);
+    double *res = c.partials + (size_t)SNB * (NP + 3 * NBIN);
+    if ((e = stats_sums(c, rec ? (float4 *)u32 : nullptr, raw, bins, reach, eps_o, nu, res)) != cudaSuccess) return e;
     const int ncol = NP + (bins ? 3 * NBIN : 0);
-    stats_reduce_kernel<<<ncol, SB, 0, c.stream>>>(c.partials, bpart, nblk, mblk, res);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     double s[NP + 3 * NBIN] = {0};
     if ((e = cudaMemcpyAsync(s, res, sizeof(double) * ncol, cudaMemcpyDeviceToHost, c.stream)) != cudaSuccess) return e;
     std::vector<double> P(3 * c.np), Uh(3 * c.np), Wh(3 * c.np), Fh(3 * c.np), Th(3 * c.np), mass(c.np), inertia(c.np);
@@ -981,6 +1011,13 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
         return e;
     if ((e = cudaStreamSynchronize(c.stream)) != cudaSuccess) return e;
     if (tc_err) return cudaErrorLaunchTimeout;  // a tensor-core wait of the closure ran out
+    if (rec && !pairs_resolve(c, s, bins, nu)) {  // the same from FP64 fields and in FP64 sums
+        if ((e = launch_macro(c, 0)) != cudaSuccess ||
+            (e = stats_sums(c, nullptr, raw, bins, reach, eps_o, nu, res)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(s, res, sizeof(double) * ncol, cudaMemcpyDeviceToHost, c.stream)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(c.stream)) != cudaSuccess)
+            return e;
+    }
     o->mass = s[ST_MASS] + s[ST_SMASS];
     for (int d = 0; d < 3; d++) o->momentum[d] = s[ST_MX + d] + s[ST_SX + d];
     o->kinetic_energy = 0.5 * (s[ST_KF] + s[ST_KS]) / (double)c.N;

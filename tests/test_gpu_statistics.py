@@ -144,3 +144,33 @@ def test_bins_of_a_small_sphere_beside_a_large_one(lbm):
     ok = (near > 0) & (b < 40)
     assert np.array_equal(got["bin_count"], np.bincount(b[ok], minlength=40))
     g.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16s"])
+@pytest.mark.parametrize("u_scale,p_scale", [(1e-18, 1e-18), (1e-30, 1e-30), (1e-18, 1.0), (1.0, 0.0)])
+def test_stats_of_tiny_velocities(lbm, storage, u_scale, p_scale):
+    """Squares far below FP32's range, of the whole field or of the fluid
+    beside particles that move at an ordinary speed: the sums are those of
+    FP64. (FP16 storage rounds the small fields to rest: zeros.)"""
+    shape = (17, 19, 21)
+    nz, ny, nx = shape
+    R = np.array([3.0, 2.5])
+    X = np.array([[1.3, 2.1, 0.7], [12.2, 11.0, 9.4]])
+    rng = np.random.default_rng(3)
+    U, W = p_scale * rng.normal(0, 0.01, (2, 3)), p_scale * rng.normal(0, 0.002, (2, 3))
+    g = lbm.Lattice(nx, ny, nz, 0.56, storage=storage, max_particles=2)
+    g.init_velocity(u_scale * (workloads.noise_velocity(shape, 0.02, seed=4) + 0.01))
+    g.add_spheres(X, R, U=U, W=W)
+    got = g.stats(lbm.STATS_BINS)
+    rho, u = g.macro()
+    with np.errstate(invalid="ignore", divide="ignore"):
+        ref = expected(u, rho, g.flags(), g.particles(), R, shape, 0.06 / 3)
+    assert np.array_equal(got["bin_count"], ref["bin_count"])
+    # sums of N terms in FP64, or as pairs of 48 bits
+    for k in ("kinetic_energy", "dissipation", "kinetic_energy_fluid", "dissipation_fluid"):
+        assert got[k] == pytest.approx(ref[k], rel=1e-12, abs=0), k
+    if np.any(u):
+        assert got["kinetic_energy_fluid"] > 0
+        for k in ("bin_tke", "bin_eps"):
+            assert np.allclose(got[k], ref[k], rtol=1e-11, atol=0), k
+    g.close()
