@@ -32,6 +32,7 @@
 #include "lbm_internal.cuh"
 #include "spectra_scratch.h"
 
+#include <cmath>
 #include <vector>
 
 namespace lbmgb {
@@ -142,10 +143,11 @@ __device__ __forceinline__ void twiddle_table(float2 *tw, int n) {
     }
 }
 
-// lines along x of field blockIdx.y (0: u_x + i u_y, 1: u_z); L consecutive
-// lines per block, through shared memory with one column of padding
+// lines along x of field blockIdx.y (0: u_x + i u_y, 1: u_z), the velocity
+// times pre (a power of two); L consecutive lines per block, through shared
+// memory with one column of padding
 template <int LOGN>
-__global__ void __launch_bounds__(fft_threads(LOGN)) fft_x_kernel(const double *u, float2 *d, long long N) {
+__global__ void __launch_bounds__(fft_threads(LOGN)) fft_x_kernel(const double *u, float2 *d, long long N, float pre) {
     constexpr int n = 1 << LOGN, L = fft_lines(LOGN), LS = L + 1, TB = fft_threads(LOGN);
     extern __shared__ float2 sm[];
     float2 *S = sm, *tw = sm + n * LS;
@@ -154,7 +156,7 @@ __global__ void __launch_bounds__(fft_threads(LOGN)) fft_x_kernel(const double *
     twiddle_table(tw, n);
     const double *p = u + (f ? 2 * N : 0) + first;
     for (int e = threadIdx.x; e < L * n; e += TB)
-        S[(e & (n - 1)) * LS + (e >> LOGN)] = make_float2((float)p[e], f ? 0.0f : (float)p[N + e]);
+        S[(e & (n - 1)) * LS + (e >> LOGN)] = make_float2(pre * (float)p[e], f ? 0.0f : pre * (float)p[N + e]);
     __syncthreads();
     const int l = threadIdx.x % L, j = threadIdx.x / L;
     float2 v[8];
@@ -268,7 +270,8 @@ __global__ void __launch_bounds__(fft_threads(LOGN)) fft_z_bins_kernel(const flo
 }
 
 template <int LOGN>
-static cudaError_t spectrum_t(Ctx &c, int nbins, float2 *field, double *part, double scale, double dfac, int &blocks) {
+static cudaError_t spectrum_t(Ctx &c, int nbins, float2 *field, double *part, double scale, double dfac, float pre,
+                              int &blocks) {
     constexpr int n = 1 << LOGN, Lx = fft_lines(LOGN), L = Lx < n ? Lx : n, TB = fft_threads(LOGN), TZ = L * n / 8;
     const size_t smx = sizeof(float2) * (size_t)(n * (Lx + 1) + n), smy = sizeof(float2) * (size_t)(n * L + n),
                  smz = smy + sizeof(double) * 2 * (size_t)nbins,
@@ -288,7 +291,7 @@ static cudaError_t spectrum_t(Ctx &c, int nbins, float2 *field, double *part, do
                              (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1));
     if (blocks < 1) return cudaErrorInvalidValue;  // refused by the caller already
     count_launch(c, G_STATS, 3);
-    fft_x_kernel<LOGN><<<dim3((unsigned)(n * n / Lx), 2), TB, smx, c.stream>>>(c.u_f, field, c.N);
+    fft_x_kernel<LOGN><<<dim3((unsigned)(n * n / Lx), 2), TB, smx, c.stream>>>(c.u_f, field, c.N, pre);
     fft_y_kernel<LOGN><<<dim3((unsigned)(n * n / L), 2), TZ, smy, c.stream>>>(field, c.N);
     fft_z_bins_kernel<LOGN><<<(unsigned)blocks, TZ, smz, c.stream>>>(field, c.N, scale, dfac, nbins, part);
     return cudaGetLastError();
@@ -310,28 +313,42 @@ cudaError_t run_spectrum(Ctx &c, int flags, int nbins, double *E, double *D) {
     const double scale = 0.5 / ((double)N * (double)N);
     const double two_pi_n = 2.0 * 3.141592653589793 / n;
     const double dfac = 2.0 * nu * two_pi_n * two_pi_n;
-    int blocks = 0;
-    switch (logn) {
-#define SP(K) case K: e = spectrum_t<K>(c, nbins, field, part, scale, dfac, blocks); break
-        SP(3); SP(4); SP(5); SP(6); SP(7); SP(8); SP(9); SP(10);
+    std::vector<double> hp;
+    auto sums = [&](float pre) -> cudaError_t {  // E and D of the velocity times pre; their sum of |Z|^2 in total
+        int blocks = 0;
+        const double sc = scale / ((double)pre * (double)pre);
+        switch (logn) {
+#define SP(K) case K: e = spectrum_t<K>(c, nbins, field, part, sc, dfac, pre, blocks); break
+            SP(3); SP(4); SP(5); SP(6); SP(7); SP(8); SP(9); SP(10);
 #undef SP
-    default: return cudaErrorInvalidValue;  // refused by the caller already
-    }
-    if (e != cudaSuccess) return e;
-    std::vector<double> hp((size_t)2 * nbins * blocks);
-    if ((e = cudaMemcpyAsync(hp.data(), part, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, c.stream)) !=
-        cudaSuccess)
-        return e;
-    if ((e = cudaStreamSynchronize(c.stream)) != cudaSuccess) return e;
-    for (int k = 0; k < nbins; k++) {
-        double se = 0.0, sd = 0.0;
-        for (int b = 0; b < blocks; b++) {  // fixed block order
-            se += hp[(size_t)b * 2 * nbins + k];
-            sd += hp[(size_t)b * 2 * nbins + nbins + k];
+        default: return cudaErrorInvalidValue;  // refused by the caller already
         }
-        E[k] = se;
-        D[k] = sd;
-    }
+        if (e != cudaSuccess) return e;
+        hp.resize((size_t)2 * nbins * blocks);
+        if ((e = cudaMemcpyAsync(hp.data(), part, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, c.stream)) !=
+            cudaSuccess)
+            return e;
+        if ((e = cudaStreamSynchronize(c.stream)) != cudaSuccess) return e;
+        for (int k = 0; k < nbins; k++) {
+            double se = 0.0, sd = 0.0;
+            for (int b = 0; b < blocks; b++) {  // fixed block order
+                se += hp[(size_t)b * 2 * nbins + k];
+                sd += hp[(size_t)b * 2 * nbins + nbins + k];
+            }
+            E[k] = se;
+            D[k] = sd;
+        }
+        return cudaSuccess;
+    };
+    if ((e = sums(1.0f)) != cudaSuccess) return e;
+    // |Z|^2 is formed in FP32. Where its mean over the wave vectors is below
+    // 2^-72, the transform's own rounding (2^-24 of Z) has squares that
+    // underflow; the velocity goes in again times 2^80 (|Z| < 2^59 then).
+    // Beyond FP32's range (an unstable state), times 2^-64.
+    double total = 0.0;
+    for (int k = 0; k < nbins; k++) total += E[k];
+    if (!std::isfinite(total)) return sums(0x1p-64f);
+    if (total < 0x1p-72 * scale * (double)N) return sums(0x1p80f);
     return cudaSuccess;
 }
 

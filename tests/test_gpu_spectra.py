@@ -131,3 +131,19 @@ def test_most_bins_of_a_small_cube_stay_in_the_scratch(lbm, storage):
         pair[0].spectrum(nb + 1)
     for g in pair:
         g.close()
+
+
+@pytest.mark.parametrize("scale", [1e-18, 1e-24, 1e-33])
+def test_tiny_velocities_keep_their_spectrum(lbm, scale):
+    """Squares below FP32's range: the shells are those of the same field at
+    an ordinary size, on the bars of the other tests (a fluid coming to rest)."""
+    n = 32
+    u = workloads.noise_velocity((n, n, n), 0.02, seed=n) * scale
+    g = lbm.Lattice(n, n, n, 0.6, storage=lbm.F64)
+    g.init_velocity(u)
+    Eg, Dg = g.spectrum(n)
+    Eo, Do = spectra.spectra(g.macro()[1] / scale, n, 0.1 / 3, n)
+    okE, eE = close(Eg / scale ** 2, Eo)
+    okD, eD = close(Dg / scale ** 2, Do)
+    assert okE and okD, (eE, eD)
+    g.close()
