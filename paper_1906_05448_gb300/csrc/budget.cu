@@ -232,7 +232,7 @@ size_t tke_budget_scratch_bytes(int nbins) { return sizeof(double) * ((size_t)30
 // sums, copies of the bins, bin means, bin products)
 cudaError_t run_tke_budget(Ctx &c, int flags, int nbins, double *out) {
     cudaError_t e;
-    if ((e = launch_macro(c, 0)) != cudaSuccess) return e;
+    if ((e = launch_macro(c)) != cudaSuccess) return e;
     const int ibm = c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B;
     if (!(ibm && (flags & LBM_STATS_UNMASK)))
         if ((e = launch_mask(c)) != cudaSuccess) return e;

@@ -76,7 +76,7 @@ __global__ void macro_kernel(const void *A, const uint8_t *flags, const int *aux
     u_o[2 * N + c] = double(uz);
 }
 
-cudaError_t launch_macro(Ctx &c, int /*mask_mode*/, float *u32, bool rec_only) {
+cudaError_t launch_macro(Ctx &c, float *u32, bool rec_only) {
     if (c.q == 27) return launch_q27_macro(c, rec_only ? (float4 *)u32 : nullptr);
     if (c.zlay) return launch_column_macro(c, rec_only ? (float4 *)u32 : nullptr);
     count_launch(c, G_STATS);
@@ -753,7 +753,7 @@ static void near_surface(Ctx &c, const unsigned nb, double reach) {
 
 cudaError_t closure_samples(Ctx &c, double u_scale, float *X, int *cells, long long cap, long long *n_out) {
     cudaError_t e;
-    if ((e = launch_macro(c, 0)) != cudaSuccess) return e;
+    if ((e = launch_macro(c)) != cudaSuccess) return e;
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     near_surface(c, nb, 2.0);
     count_launch(c, G_STATS);
@@ -771,7 +771,7 @@ cudaError_t closure_samples(Ctx &c, double u_scale, float *X, int *cells, long l
 
 cudaError_t closure_targets(Ctx &c, const int *cells, long long n, double g_scale, float *T) {
     cudaError_t e;
-    if ((e = launch_macro(c, 0)) != cudaSuccess) return e;
+    if ((e = launch_macro(c)) != cudaSuccess) return e;
     count_launch(c, G_STATS, 2);
     if ((e = mask_cells(c, nullptr)) != cudaSuccess) return e;
     if (n > 0)
@@ -872,7 +872,7 @@ size_t pipe_profile_scratch_bytes(int nbins) { return sizeof(double) * (size_t)3
 // scratch: the population buffer that the next step overwrites
 cudaError_t run_pipe_profiles(Ctx &c, int flags, int nbins, double *out) {
     cudaError_t e;
-    if ((e = launch_macro(c, 0)) != cudaSuccess) return e;
+    if ((e = launch_macro(c)) != cudaSuccess) return e;
     const int ibm = c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B;
     if (!(ibm && (flags & LBM_STATS_UNMASK)))
         if ((e = launch_mask(c)) != cudaSuccess) return e;
@@ -961,7 +961,7 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
     // population buffer that the next step overwrites.
     const bool rec = c.storage != LBM_F64;
     float *u32 = rec ? (float *)c.rho_f : (closure ? (float *)c.fB : nullptr);
-    if ((e = launch_macro(c, 0, u32, rec)) != cudaSuccess) return e;
+    if ((e = launch_macro(c, u32, rec)) != cudaSuccess) return e;
     const bool raw = ibm && (flags & LBM_STATS_UNMASK);
     const unsigned nb = (unsigned)((c.N + 255) / 256);
     const double nu = (c.tau - 0.5) / 3.0;
@@ -1012,7 +1012,7 @@ cudaError_t run_stats(Ctx &c, int flags, lbm_stats_t *o) {
     if ((e = cudaStreamSynchronize(c.stream)) != cudaSuccess) return e;
     if (tc_err) return cudaErrorLaunchTimeout;  // a tensor-core wait of the closure ran out
     if (rec && !pairs_resolve(c, s, bins, nu)) {  // the same from FP64 fields and in FP64 sums
-        if ((e = launch_macro(c, 0)) != cudaSuccess ||
+        if ((e = launch_macro(c)) != cudaSuccess ||
             (e = stats_sums(c, nullptr, raw, bins, reach, eps_o, nu, res)) != cudaSuccess ||
             (e = cudaMemcpyAsync(s, res, sizeof(double) * ncol, cudaMemcpyDeviceToHost, c.stream)) != cudaSuccess ||
             (e = cudaStreamSynchronize(c.stream)) != cudaSuccess)

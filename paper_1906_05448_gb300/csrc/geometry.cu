@@ -390,9 +390,6 @@ struct SiteArgs {
     int *site_own;
 };
 
-// minimum image with the box size and its half given as doubles (no
-// int-to-double conversion per call; the same values as gmimg)
-
 // solid-neighbour mask of a fluid cell (bit l: x + c_l solid)
 __device__ __forceinline__ unsigned solid_mask(const SiteArgs &a, int x, int y, int z) {
     unsigned m = 0;

@@ -1143,7 +1143,7 @@ lbm_status lbm_get_field(lbm_ctx *h, int which, void *dst, size_t bytes) {
     case LBM_FIELD_RHO:
     case LBM_FIELD_U: {
         if (bytes < need) return fail(c, LBM_EINVAL, "destination too small");
-        CK(launch_macro(c, 0));
+        CK(launch_macro(c));
         CK(cudaMemcpyAsync(dst, which == LBM_FIELD_RHO ? (void *)c.rho_f : (void *)c.u_f, need,
                            cudaMemcpyDeviceToHost, c.stream));
         break;

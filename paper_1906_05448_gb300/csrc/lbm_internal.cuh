@@ -145,8 +145,6 @@ struct lbm_ctx {
 // ------------------------------------------------ cross-file launchers ----
 namespace lbmgb {
 cudaError_t launch_init_equilibrium(Ctx &c, const double *u_dev, double rho0);
-cudaError_t launch_set_populations(Ctx &c, const double *f_dev);
-cudaError_t launch_get_populations(Ctx &c, double *f_dev);
 cudaError_t launch_stream_collide(Ctx &c, int bc);
 cudaError_t launch_column_sweep(Ctx &c);  // sweep_columns.cu: the pipe's IBB step
 // columns.cu: the state between the two layouts, one plane to or from
@@ -180,7 +178,7 @@ cudaError_t launch_ibm_particle_sums(Ctx &c, bool init_only);
 cudaError_t launch_ibm_rigid_overwrite(Ctx &c);
 // rho and u into c.rho_f and c.u_f (FP64); u32, if not null, receives FP32
 // records (ux, uy, uz, rho) per cell, alone with rec_only (32- and 16-bit storage)
-cudaError_t launch_macro(Ctx &c, int mask_mode, float *u32 = nullptr, bool rec_only = false);
+cudaError_t launch_macro(Ctx &c, float *u32 = nullptr, bool rec_only = false);
 cudaError_t launch_mask(Ctx &c);  // statistics velocity: solid cells take the rigid-body velocity
 cudaError_t run_spectrum(Ctx &c, int flags, int nbins, double *E, double *D);
 cudaError_t run_pipe_profiles(Ctx &c, int flags, int nbins, double *out);

@@ -1,5 +1,6 @@
-// Work list and wall tables of the pipe sweep with two cells per lane
-// (sweep_pair16.cu; host code, no CUDA).
+// Work list and wall tables of a pipe sweep with two cells per lane (host
+// code, no CUDA). The pipe's sweeps walk columns now (columns.cuh); nothing
+// but this file's own test builds it.
 //
 // Each run of fluid cells of an x-row is taken from an even cell to an odd
 // one: an odd first cell adds its (solid) left neighbour, an even last cell

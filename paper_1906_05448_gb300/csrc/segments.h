@@ -1,4 +1,6 @@
-// Work list of the IBB sweep for a static wall (host code, no CUDA).
+// Work list of an IBB sweep over x-fast rows for a static wall (host code, no
+// CUDA). The pipe's sweeps walk columns now (columns.cuh); nothing but the
+// tests of this file and of pairs.h builds it.
 //
 // Each run of fluid cells of an x-row is cut into segments of at most 32
 // lanes; one warp sweeps one segment, so solid cells are never pulled and

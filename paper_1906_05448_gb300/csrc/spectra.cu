@@ -305,7 +305,7 @@ cudaError_t run_spectrum(Ctx &c, int flags, int nbins, double *E, double *D) {
     const long long N = c.N;
     float2 *field = (float2 *)c.fB;
     double *part = (double *)((char *)c.fB + spectrum_bins_offset(N));
-    if ((e = launch_macro(c, 0)) != cudaSuccess) return e;
+    if ((e = launch_macro(c)) != cudaSuccess) return e;
     const int ibm = c.armed_bc == LBM_BC_IBM_U || c.armed_bc == LBM_BC_IBM_B;
     if (!(ibm && (flags & LBM_STATS_UNMASK)))
         if ((e = launch_mask(c)) != cudaSuccess) return e;

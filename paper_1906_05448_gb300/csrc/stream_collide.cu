@@ -377,31 +377,7 @@ cudaError_t launch_ibm_collide(Ctx &c) {
     }
 }
 
-// ------------------------------------------------- population transfer ----
-template <int S>
-__global__ void set_pops_kernel(void *dst, const double *f, long long N) {
-    typedef typename Store<S>::T T;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 19 * N) return;
-    const int i = (int)(idx / N);
-    Store<S>::st((T *)dst + idx, typename Store<S>::R(f[idx] - wgt(i)));
-}
-
-template <int S>
-__global__ void get_pops_kernel(const void *src, double *f, long long N) {
-    typedef typename Store<S>::T T;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 19 * N) return;
-    const int i = (int)(idx / N);
-    const T *p = (const T *)src + idx;
-    double v;
-    if (S == LBM_F64) v = (double)*(const double *)p;
-    else if (S == LBM_F32) v = (double)*(const float *)p;
-    else if (S == LBM_F16S) v = (double)__half2float(*(const __half *)p) / F16_SCALE;
-    else v = (double)__bfloat162float(*(const __nv_bfloat16 *)p);
-    f[idx] = v + wgt(i);
-}
-
+// ------------------------------------------------------- initial state ----
 template <int S>
 __global__ void init_eq_kernel(void *dst, const double *u, double rho0, long long N) {
     typedef typename Store<S>::T T;
@@ -419,30 +395,6 @@ __global__ void init_eq_kernel(void *dst, const double *u, double rho0, long lon
         const R geq = R(wgt(i)) * ((r0 - R(1)) + r0 * (R(3) * cu + R(4.5) * cu * cu - R(1.5) * u2));
         Store<S>::st((T *)dst + (size_t)i * N + c, geq);
     }
-}
-
-cudaError_t launch_set_populations(Ctx &c, const double *f_dev) {
-    const long long n = 19 * c.N;
-    const unsigned nb = (unsigned)((n + 255) / 256);
-    switch (c.storage) {
-    case LBM_F64: set_pops_kernel<LBM_F64><<<nb, 256, 0, c.stream>>>(c.fA, f_dev, c.N); break;
-    case LBM_F32: set_pops_kernel<LBM_F32><<<nb, 256, 0, c.stream>>>(c.fA, f_dev, c.N); break;
-    case LBM_F16S: set_pops_kernel<LBM_F16S><<<nb, 256, 0, c.stream>>>(c.fA, f_dev, c.N); break;
-    default: set_pops_kernel<LBM_BF16S><<<nb, 256, 0, c.stream>>>(c.fA, f_dev, c.N); break;
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_get_populations(Ctx &c, double *f_dev) {
-    const long long n = 19 * c.N;
-    const unsigned nb = (unsigned)((n + 255) / 256);
-    switch (c.storage) {
-    case LBM_F64: get_pops_kernel<LBM_F64><<<nb, 256, 0, c.stream>>>(c.fA, f_dev, c.N); break;
-    case LBM_F32: get_pops_kernel<LBM_F32><<<nb, 256, 0, c.stream>>>(c.fA, f_dev, c.N); break;
-    case LBM_F16S: get_pops_kernel<LBM_F16S><<<nb, 256, 0, c.stream>>>(c.fA, f_dev, c.N); break;
-    default: get_pops_kernel<LBM_BF16S><<<nb, 256, 0, c.stream>>>(c.fA, f_dev, c.N); break;
-    }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_init_equilibrium(Ctx &c, const double *u_dev, double rho0) {
