@@ -12,12 +12,10 @@
 // without it those across the low faces overflow on planes of nearly 2^31.
 #pragma once
 
-#ifndef LBM_HD
 #ifdef __CUDACC__
 #define LBM_HD __host__ __device__ __forceinline__
 #else
 #define LBM_HD inline
-#endif
 #endif
 
 namespace lbmgb {

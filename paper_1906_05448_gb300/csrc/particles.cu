@@ -11,7 +11,6 @@
 // All reductions are block trees in a fixed order (bitwise reproducible for
 // a given launch configuration); only the IBM spreading uses FP64 atomics.
 #include "lbm_internal.cuh"
-#include "spread_sum.h"
 
 #include <algorithm>
 
@@ -890,9 +889,14 @@ __global__ void __launch_bounds__(256) ibm_spread_particle_kernel(ParticleSpread
 // took 147 + 170 us at 256^3 with 2000 spheres of radius 4; a warp per marker
 // on the box 215; this takes 118.
 //
-// FP32: the box of forces is in integers, each component on a scale of its
-// own (spread_sum.h). Shared-memory integer atomics are native (FP32 ones are
-// a compare-and-swap loop), and the sum does not depend on their order.
+// FP32: the box of forces is in integers, scaled by the power of two that
+// puts the largest |F_l dV_l| of the particle at 2^28 .. 2^29. Shared-memory
+// integer atomics are native (FP32 ones are a compare-and-swap loop), the
+// sum does not depend on their order, and its quantum, 2^-28 or less of that
+// force, is finer than the rounding of FP32 sums of that size. Four times
+// the largest term fits: the weights of a cell over the markers of a sphere
+// (about one per unit of surface) add up to 0.92 at most, at a radius of 1.1,
+// and to 0.5 .. 0.6 beyond 2.
 template <typename R>
 struct __align__(4 * sizeof(R)) PassBox {
     R rho, u0, u1, u2;
@@ -900,9 +904,12 @@ struct __align__(4 * sizeof(R)) PassBox {
 template <typename R> struct SpreadSum;
 template <> struct SpreadSum<float> {
     typedef int T;
-    static __device__ __forceinline__ float scale(float m) { return spread_scale(m); }
-    static __device__ __forceinline__ int of(float v, float s) { return spread_term(v, s); }
-    static __device__ __forceinline__ float value(int v, float s) { return spread_value(v, s); }
+    static __device__ __forceinline__ float scale(float m) {  // 2^(28 - exponent of m)
+        const int e = (int)(__float_as_uint(m) >> 23) - 127;
+        return m > 0.f ? exp2f((float)min(28 - e, 120)) : 1.f;
+    }
+    static __device__ __forceinline__ int of(float v, float s) { return __float2int_rn(v * s); }
+    static __device__ __forceinline__ float value(int v, float s) { return (float)v / s; }
 };
 template <> struct SpreadSum<double> {
     typedef double T;
@@ -933,7 +940,7 @@ __global__ void __launch_bounds__(256) ibm_pass_particle_kernel(IbmArgs a, const
     T *F = (T *)(box + nb);  // three components
     R *phi = (R *)(F + 3 * nb), *Fl = phi + 12 * max_markers;
     int *first = (int *)(Fl + 3 * max_markers), *site = first + max_markers;
-    __shared__ R wmax[3][8];
+    __shared__ R wmax[8];
     const int p = blockIdx.x, tid = threadIdx.x;
     __shared__ int head[3];
     if (tid < 3) head[tid] = (int)floor(a.X[3 * p + tid]) - (int)ceil(Rp[p] - rd) - 1;  // the box, once per block
@@ -1027,18 +1034,13 @@ __global__ void __launch_bounds__(256) ibm_pass_particle_kernel(IbmArgs a, const
             bad = bad || !(fabs(g) < R(1e30));
         }
     }
-    // the largest force of each component (lane & 3) sets the scale of its integer sums
+    // the particle's largest force sets the scale of the integer sums
 #pragma unroll
-    for (int o = 16; o > 3; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
-    if ((tid & 31) < 3) wmax[tid & 31][tid >> 5] = big;
+    for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    if ((tid & 31) == 0) wmax[tid >> 5] = big;
     bad = __syncthreads_or(bad);
-    R sc[3];
-    for (int d = 0; d < 3; d++) {
-        big = wmax[d][0];
-        for (int k = 1; k < 8; k++) big = fmax(big, wmax[d][k]);
-        sc[d] = Sum::scale(big);
-    }
-    const bool few = sizeof(T) == sizeof(R) && spread_few(n);  // the box of forces holds R then
+    for (int k = 0; k < 8; k++) big = fmax(big, wmax[k]);
+    const R sc = Sum::scale(big);
     for (int t = tid; t < 4 * n; t += 256) {
         const int m = t >> 2, kz = t & 3;
         if (first[m] < 0) continue;
@@ -1051,15 +1053,9 @@ __global__ void __launch_bounds__(256) ibm_pass_particle_kernel(IbmArgs a, const
             for (int kx = 0; kx < 4; kx++) {
                 const R w = ph[kx] * ph[4 + ky] * pz;
                 T *c = q + kx + W * ky;
-                if (few) {
-                    atomicAdd((R *)c, f0 * w);
-                    atomicAdd((R *)(c + nb), f1 * w);
-                    atomicAdd((R *)(c + 2 * nb), f2 * w);
-                    continue;
-                }
-                atomicAdd(c, Sum::of(f0 * w, sc[0]));
-                atomicAdd(c + nb, Sum::of(f1 * w, sc[1]));
-                atomicAdd(c + 2 * nb, Sum::of(f2 * w, sc[2]));
+                atomicAdd(c, Sum::of(f0 * w, sc));
+                atomicAdd(c + nb, Sum::of(f1 * w, sc));
+                atomicAdd(c + 2 * nb, Sum::of(f2 * w, sc));
             }
     }
     __syncthreads();
@@ -1072,10 +1068,9 @@ __global__ void __launch_bounds__(256) ibm_pass_particle_kernel(IbmArgs a, const
         if (f0 == T(0) && f1 == T(0) && f2 == T(0) && !bad) continue;
         // a force that is no number reaches the fluid (and the watchdog) as one
         const R nan = bad ? R(0) / R(0) : R(0);
-        const R *Fr = (const R *)F;
-        atomicAdd(Fp + 3 * s, (few ? Fr[b] : Sum::value(f0, sc[0])) + nan);
-        atomicAdd(Fp + 3 * s + 1, (few ? Fr[nb + b] : Sum::value(f1, sc[1])) + nan);
-        atomicAdd(Fp + 3 * s + 2, (few ? Fr[2 * nb + b] : Sum::value(f2, sc[2])) + nan);
+        atomicAdd(Fp + 3 * s, Sum::value(f0, sc) + nan);
+        atomicAdd(Fp + 3 * s + 1, Sum::value(f1, sc) + nan);
+        atomicAdd(Fp + 3 * s + 2, Sum::value(f2, sc) + nan);
     }
 }
 
