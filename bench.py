@@ -444,13 +444,13 @@ def cpu_baseline(target_seconds=12.0):
             "sample": f"FP64 oracle, IBB pipe slab 148x148x16 ({fluid} fluid cells), {steps} steps, {sec:.1f} s"}
 
 
-SWEEP_SOURCES = {"sweep_columns_pipe148_f32": ("sweep_columns.cu", "lbm_device.cuh", "columns.cuh"),
-                 "stream_collide_bulk_pipe148_ibm_f32": ("sweep.cu", "lbm_device.cuh")}
+SWEEP_SOURCES = {"sweep_columns_pipe148_f32": ("sweep_columns.cu", "lbm_device.cuh", "columns.cuh", "column_index.h"),
+                 "ibm_columns_sweep_pipe148_f32": ("ibm_columns.cu", "lbm_device.cuh", "columns.cuh", "column_index.h")}
 
 
 def source_hash(kernel_key):
-    """Hash of a sweep kernel's sources (kernel, device header, segment
-    list): a recorded DRAM traffic figure is used only while it matches."""
+    """Hash of a sweep kernel's sources (kernel and headers): a recorded DRAM
+    traffic figure is used only while it matches."""
     h = hashlib.sha256()
     for f in SWEEP_SOURCES[kernel_key]:
         with open(os.path.join(ROOT, "paper_1906_05448_gb300", "csrc", f), "rb") as fh:
@@ -670,12 +670,13 @@ def main():
                        "fluid_cells": main_res["fluid_cells"], "parallelism": f"replicas x{world}",
                        "l2": "no flush: populations 2x1.46 GB >> 129 MB L2"},
             "roofline": {"bound": "hbm",
-                         "kernel": ("sweep_columns<" if args.wall == "ibb" else "stream_collide_bulk<") +
+                         "kernel": ("sweep_columns<" if args.wall == "ibb" else "ibm_columns_sweep<") +
                                    args.storage + ",srt," + args.wall[:3] + ">",
                          "achieved": round(achieved, 1), "peak": hbm_peak, "unit": "GB/s",
                          "frac": round(achieved / hbm_peak, 4), "peak_source": peak_kind,
-                         "traffic": traffic_for("sweep_columns_pipe148_f32")
-                         if (args.wall == "ibb" and args.storage == "f32" and NZ == PIPE["nz"]) else None,
+                         "traffic": traffic_for("sweep_columns_pipe148_f32" if args.wall == "ibb"
+                                                else "ibm_columns_sweep_pipe148_f32")
+                         if (args.storage == "f32" and NZ == PIPE["nz"]) else None,
                          "algorithmic_bytes_per_launch": bulk_bytes,
                          "avg_launch_ms": round(bulk_ms, 5),
                          "step_achieved": round(bulk_bytes / (ms_total / args.steps * 1e-3) / 1e9, 1),

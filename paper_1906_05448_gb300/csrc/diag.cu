@@ -1,8 +1,10 @@
 // Diagnostics (Sec. 3.2, Sec. 2.2): macroscopic fields of the current state,
 // rigid-body masking of particle regions, kinetic energy, dissipation
 // 2 nu s_ij s_ij from second-order central differences, radial profiles
-// around particles and the pipe bulk velocity. Sums are FP64 block partials
-// reduced on the host in block order (deterministic).
+// around particles and the pipe bulk velocity. The sums of lbm_stats are
+// block partials added on the device in a fixed order (deterministic): FP64,
+// or pairs of floats of 48 bits for 32- and 16-bit storage. The pipe profiles
+// add their columns with global FP64 atomics, in no fixed order.
 #include "columns.cuh"
 
 #include <algorithm>

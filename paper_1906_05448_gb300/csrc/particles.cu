@@ -1,4 +1,6 @@
-// Particle-side kernels, FP64 throughout:
+// Particle-side kernels. Particle state and equations are FP64; sums over
+// links, markers and box cells form their terms in the storage's arithmetic
+// type and add them up in FP64:
 //  - gimem_reduce: per-particle sum of the per-link momentum exchange
 //    (Galilean-invariant form of Wen et al. 2014, Sec. 3.1);
 //  - release_kernel: initial particle velocity = fluid velocity averaged
@@ -9,7 +11,8 @@
 //    passes (interpolate with the Peskin 4-point delta, force, spread;
 //    Sec. 2.1 / 3.1) and the particle force with Kempe's inner-fluid term.
 // All reductions are block trees in a fixed order (bitwise reproducible for
-// a given launch configuration); only the IBM spreading uses FP64 atomics.
+// a given launch configuration); only the IBM spreading adds to the support
+// cells with atomics (of the storage's arithmetic type).
 #include "lbm_internal.cuh"
 
 #include <algorithm>

@@ -23,8 +23,9 @@
 // (hi + lo), are added before one FP64 addition per quadruple goes to the
 // block's bins; FP64 is the scarce unit here. The blocks' bins are added on
 // the host in a fixed order.
-// 256^3, 222 shells: 5.4 ms with a radix-2 transform per component and two
-// shared-memory FP64 atomics per cell and component, 1.28 ms now.
+// 256^3, 222 shells, the whole call: 6.3 ms with a radix-2 transform per
+// component and two shared-memory FP64 atomics per cell and component, 1.22
+// ms now.
 //
 // Scratch: the population buffer that the next step overwrites holds the
 // two complex fields (16 bytes per cell of its 38 or more) and the

@@ -10,7 +10,7 @@
 //   exchange of the link (Wen et al. 2014, Sec. 3.1).
 // ibm_collide: collides support cells with the body force plus the IBM force
 //   accumulated over the forcing passes.
-// Population transfer and equilibrium initialisation kernels.
+// Equilibrium initialisation.
 
 #include "lbm_internal.cuh"
 
