@@ -899,7 +899,10 @@ __global__ void __launch_bounds__(256) ibm_spread_particle_kernel(ParticleSpread
 // force, is finer than the rounding of FP32 sums of that size. Four times
 // the largest term fits: the weights of a cell over the markers of a sphere
 // (about one per unit of surface) add up to 0.92 at most, at a radius of 1.1,
-// and to 0.5 .. 0.6 beyond 2.
+// and to 0.5 .. 0.6 beyond 2. The quantum is the same for all components: one
+// that is a hundredth of the strongest keeps 8e-6 of itself in its sums (CPU
+// emulation, radius 3.6), less than what rounding the velocities to FP32
+// leaves of it.
 template <typename R>
 struct __align__(4 * sizeof(R)) PassBox {
     R rho, u0, u1, u2;
