@@ -137,13 +137,34 @@ def test_d3q27_refuses_what_it_does_not_build(lbm):
         lbm.Lattice(16, 16, 16, 0.6, storage=lbm.F16S, lattice=27)
 
 
+def halfway_links(nx, ny, R):
+    """Links of a plane that take the halfway fallback (q < 1/2, x_f - c_i solid)."""
+    links = q27.pipe_links(q27.pipe_solid(nx, ny, 1, R), R)
+    return sum(int(np.count_nonzero(m & (q < 0.5) & ~up)) for m, q, up in links)
+
+
+@pytest.mark.parametrize("nx,nz,R", [(17, 5, 7.1), (16, 32, 6.4)])  # cells in turn, warps per column
+@pytest.mark.parametrize("storage,tol", [("f64", 1e-12), ("f32", 1e-5)])
+def test_halfway_fallback_matches_the_oracle(lbm, nx, nz, R, storage, tol):
+    assert halfway_links(nx, nx, R) > 0
+    g, o, solid, links = _pipe_pair(lbm, nx, nx, nz, R, 0.62, (0.0, 0.0, 3e-6), lbm.STORAGE[storage], seed=3)
+    fl = ~solid.reshape(-1)
+    for _ in range(4):
+        g.step(1, lbm.BC_IBB)
+        o = q27.step_pipe(o, solid, links, 0.62, (0.0, 0.0, 3e-6))
+        assert rel(g.populations()[:, fl], o.reshape(27, -1)[:, fl]) < tol
+    g.close()
+
+
 @pytest.mark.parametrize("lattice,storage", [(27, "f64"), (27, "f32"), (19, "f64"), (19, "f32"), (19, "f16s"),
                                              (19, "bf16s")])
 def test_what_solid_cells_hold_never_reaches_the_fluid(lbm, lattice, storage):
-    """A wall with the schemes for walls one cell apart (the 6.4 radius in a
-    16 x 15 section): a context whose solid cells hold NaN steps the fluid bit
-    for bit as one whose solid cells hold the state at rest."""
-    nx, ny, nz, R = 16, 15, 5, 6.4
+    """A wall with the schemes for walls one cell apart (halfway links on
+    D3Q27, single-node ones on D3Q19): a context whose solid cells hold NaN
+    steps the fluid bit for bit as one whose solid cells hold the state at
+    rest."""
+    nx, ny, nz, R = (17, 17, 5, 7.1) if lattice == 27 else (16, 16, 5, 6.4)
+    assert lattice == 19 or halfway_links(nx, ny, R) > 0
     u = workloads.pipe_velocity(nx, ny, nz, R, 0.02, perturbation=0.1, seed=3)
     runs = []
     for fill in (None, np.nan):
