@@ -38,9 +38,9 @@ struct ColumnPtrs {
 // need shifted offsets (column_shifted). us per step of the IBB pipe with warps
 // per column, and so:
 //   148 x 148 x 4    FP32 12.3 and 6.2   FP16 13.1 and 6.2   FP64 254 and 41
-//   148 x 148 x 16   FP32 12.3 and 10.3  FP16 13.5 and 10.3  FP64 254 and 131
-//   300 x 300 x 8    FP32 33.4 and 16.5  FP16 35.5 and 14.4  FP64 1033 and 274
-//   300 x 300 x 33   FP32 75.8 and 63.7  FP16 70.8 and 49.4  FP64 2044 and 1071
+//   148 x 148 x 16   FP32 12.3 and 10.3  FP16 13.5 and 9.7   FP64 254 and 131
+//   300 x 300 x 8    FP32 33.4 and 16.4  FP16 35.6 and 14.4  FP64 1033 and 274
+//   300 x 300 x 33   FP32 75.8 and 65.4  FP16 70.5 and 49.5  FP64 2044 and 1071
 //   148 x 148 x 58   FP32 37.1 and 31.3  FP16 22.1 and 20.8  FP64 505 and 456
 //   148 x 148 x 438  FP32 176.4 and 179.7, FP16 124.7 and 125.1 (14 warps of
 //                    32 for 438 cells: the wall and the sectors decide)
